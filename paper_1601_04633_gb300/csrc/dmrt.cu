@@ -22,6 +22,7 @@
 #include "step_direct.cuh"
 #include "step_tma.cuh"
 #include "step_tma_batch.cuh"
+#include "step_march.cuh"
 #include "tma_variants.h"
 
 using dmrt::plane_f;
@@ -74,7 +75,7 @@ Layout make_layout(const dmrt_params& p, int halo_rows = 0) {
     L.off_b = o; o += L.buf_bytes;
     L.off_hot = o; o += align256((size_t)p.ny * sizeof(float));
     L.off_cold = o; o += align256((size_t)p.ny * sizeof(float));
-    L.off_rows = o; o += align256((size_t)2 * p.ny * sizeof(double));  // by source buffer
+    L.off_rows = o; o += align256((size_t)2 * dmrt::kMarchMax * p.ny * sizeof(double));  // by source buffer; march launches: each of their steps
     L.off_ring = o; o += align256((size_t)p.nu_capacity * sizeof(double));
     L.off_misc = o; o += 256;
     L.total = o;
@@ -127,6 +128,13 @@ struct dmrt_ctx {
     // Adjoint: a second stream and events for the overlapped recompute (created at first use).
     cudaStream_t aux;
     cudaEvent_t ev[5];
+    // March kernel (several steps per launch, for runs of steps of a whole cavity
+    // under AUTO): its compiled forms, items and arguments.
+    const void* march[dmrt::kMarchMax + 1];  // by steps per launch (2, 3); nullptr: not used
+    int mstrips, mchunks[dmrt::kMarchMax + 1], mchunk[dmrt::kMarchMax + 1];
+    unsigned msmem;
+    dmrt::MarchMaps mmaps[2];  // per source buffer
+    dmrt::PairConsts pc;
     cudaGraphExec_t graph[2];
     int graph_len;
     long long nu_floor;  // ring values of steps before this one are unavailable (after a load)
@@ -855,6 +863,124 @@ int setup_kernel(dmrt_ctx* c) {
     return DMRT_OK;
 }
 
+// Runs of steps on the march kernel (step_march.cuh): three steps per launch,
+// two where three would leave a single step.
+//
+// AUTO takes it for whole cavities of at least 40000 nodes and 160 columns that
+// do not fit a cluster. Microseconds per step, march / one launch per step, on one GB300:
+// float32 192^2 3.4 / 3.1, 256^2 3.4 / 4.2, 512^2 6.1 / 9.5, 1024^2 12.7 / 22.7,
+// 2048^2 34.6 / 78.0, 4096^2 118 / 288; mixed, stochastic 128^2 3.7 / 3.0, 256^2
+// 3.7 / 4.4, 1024^2 14.6 / 20.0, 4096^2 145 / 212; THETA32, stochastic 1024^2
+// 15.9 / 18.1, 1999 x 1531 35.7 / 43.6; float16, stochastic 2048^2 45.9 / 51.6.
+// (Two steps per launch: 163 us at 4096^2 in float32, bound by HBM; three are
+// bound by the float32 pipe, 65 % busy, and by the tail of a launch.)
+//
+// Narrow cavities leave a strip's lanes idle (100 x 500: 4.3 against 3.9).
+constexpr long long kMarchNodes = 40000;
+constexpr int kMarchWidth = 160;
+
+// Rows per chunk of a march launch of T steps: a warp marches through chunk + 2 (T - 1)
+// rows, so long chunks recompute less, and short ones use more warps. The
+// cheapest under what a row's iteration took on one GB300: 1.15 us with one
+// block on an SM (one warp per scheduler), 2.0 with two, 2.14 with more; a
+// single wave of long chunks ends unevenly (4096^2: one wave of 158 rows 129 us per step, two of 80 rows 120).
+int march_chunk(int ny, int strips, int T, int sms, int per_sm) {
+    const int per = dmrt::kMarchThreads / 32;
+    int best = ny;
+    double cost = 1e300;
+    for (int chunk = 1; chunk <= ny; ++chunk) {
+        const long long blocks = ((long long)strips * ((ny + chunk - 1) / chunk) + per - 1) / per;
+        const long long k = (blocks + sms - 1) / sms;
+        const long long waves = (blocks + (long long)sms * per_sm - 1) / ((long long)sms * per_sm);
+        double c = chunk + 2 * (T - 1);
+        c *= k == 1 ? 1.15 : k == 2 ? 2.0 : 2.14 * (double)waves;
+        if (waves == 1 && chunk > 120) c *= 1.12;
+        if (c < cost) cost = c, best = chunk;
+    }
+    return best;
+}
+
+int setup_march(dmrt_ctx* c) {
+    const dmrt_params& p = c->p;
+    std::memset(c->march, 0, sizeof c->march);
+    if (c->cluster || c->slab || p.kernel != DMRT_KERNEL_AUTO || p.tma_npt > 0 || p.tma_rows > 0 || p.tma_stages > 0)
+        return DMRT_OK;
+    if (p.nx < kMarchWidth || (long long)p.nx * p.ny < kMarchNodes) return DMRT_OK;
+    const dmrt::MarchForm F2 = dmrt::march_form(p.storage, p.rounding, 2), F = dmrt::march_form(p.storage, p.rounding, 3);
+    int dev = 0, sms = 0, per_sm = 0;
+    CK(cudaGetDevice(&dev), "cudaGetDevice");
+    CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev), "SM count");
+    CK(cudaFuncSetAttribute(F2.func, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)F.smem), "set march shared memory");
+    CK(cudaFuncSetAttribute(F.func, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)F.smem), "set march shared memory");
+    c->mstrips = (p.nx + F.cols - 1) / F.cols;
+    for (int t = 2; t <= dmrt::kMarchMax; ++t) {
+        CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, t == 2 ? F2.func : F.func, dmrt::kMarchThreads, F.smem),
+           "occupancy");
+        if (per_sm < 1) return DMRT_OK;
+        c->mchunk[t] = march_chunk(p.ny, c->mstrips, t, sms, per_sm);
+        c->mchunks[t] = (p.ny + c->mchunk[t] - 1) / c->mchunk[t];
+    }
+    c->msmem = F.smem;
+    for (int b = 0; b < 2; ++b) {
+        // Loads of whole rows from buffer b, stores (nx columns wide) to the other one.
+        dmrt::MarchMaps& m = c->mmaps[b];
+        std::memset(&m, 0, sizeof m);
+        char* src = reinterpret_cast<char*>(buf(c, b));
+        char* dst = reinterpret_cast<char*>(buf(c, 1 - b));
+        const size_t goff = (size_t)9 * c->L.plane * 2, doff = goff + (size_t)c->L.plane * 4;
+        int rc;
+        if (p.storage == DMRT_THETA32) {
+            rc = encode_map(c, &m.ld[0], src, DMRT_FP16, 9, 9, 1, F.box);
+            if (!rc) rc = encode_map(c, &m.ld[1], src + goff, DMRT_FP32, 1, 1, 1, F.box);
+            if (!rc) rc = encode_map(c, &m.ld[2], src + doff, DMRT_FP16, 4, 4, 1, F.box);
+            if (!rc) rc = encode_map(c, &m.st[0], dst, DMRT_FP16, 9, 9, 1, F.cols, p.nx);
+            if (!rc) rc = encode_map(c, &m.st[1], dst + goff, DMRT_FP32, 1, 1, 1, F.cols, p.nx);
+            if (!rc) rc = encode_map(c, &m.st[2], dst + doff, DMRT_FP16, 4, 4, 1, F.cols, p.nx);
+        } else if (p.storage == DMRT_MIXED) {
+            rc = encode_map(c, &m.ld[0], src, DMRT_FP16, 9, 9, 1, F.box);
+            if (!rc) rc = encode_map(c, &m.ld[1], src + goff, DMRT_FP32, 5, 5, 1, F.box);
+            if (!rc) rc = encode_map(c, &m.st[0], dst, DMRT_FP16, 9, 9, 1, F.cols, p.nx);
+            if (!rc) rc = encode_map(c, &m.st[1], dst + goff, DMRT_FP32, 5, 5, 1, F.cols, p.nx);
+        } else {
+            rc = encode_map(c, &m.ld[0], src, p.storage, kPlanes, kPlanes, 1, F.box);
+            if (!rc) rc = encode_map(c, &m.st[0], dst, p.storage, kPlanes, kPlanes, 1, F.cols, p.nx);
+        }
+        if (rc) return rc;
+    }
+    c->pc = dmrt::make_pair_consts(c->sc);
+    c->march[2] = F2.func;
+    c->march[3] = F.func;
+    return DMRT_OK;
+}
+int march_grid(const dmrt_ctx* c, int steps) {
+    const int per = dmrt::kMarchThreads / 32;
+    return (c->mstrips * c->mchunks[steps] + per - 1) / per + 1;  // the last block sums Nusselt rows
+}
+
+// Arguments of a march launch of `steps` steps from buffer `from` (the finalize launch takes any).
+dmrt::MarchArgs march_args(dmrt_ctx* c, int from, int steps) {
+    dmrt::MarchArgs M;
+    M.A = step_args(c, from);
+    double* rows = reinterpret_cast<double*>(c->ws + c->L.off_rows);
+    for (int k = 0; k < dmrt::kMarchMax; ++k) {
+        M.nu_rows[k] = rows + (size_t)(2 * k + from) * c->p.ny;
+        M.prev_rows[k] = rows + (size_t)(2 * k + 1 - from) * c->p.ny;
+    }
+    M.n_strips = c->mstrips;
+    M.n_chunks = c->mchunks[steps];
+    M.chunk = c->mchunk[steps];
+    M.sign_l = c->sc.left_fixed ? -1.f : 1.f;
+    M.sign_r = c->sc.right_fixed ? -1.f : 1.f;
+    M.gsh0 = c->sc.gsh0;
+    M.gsh1 = c->sc.gsh1;
+    M.w0 = c->sc.w0;
+    M.w1 = c->sc.w1;
+    M.abb_l = c->sc.left_fixed ? c->sc.abb : 0.f;
+    M.abb_r = c->sc.right_fixed ? c->sc.abb : 0.f;
+    M.nu_scale = c->sc.nu_scale;
+    return M;
+}
+
 int validate(const dmrt_params* p, dmrt_ctx* c) {
     if (!p) {
         set_err(c, "params is NULL");
@@ -1058,6 +1184,7 @@ static int create_ctx(const dmrt_params* pg, int y0, int rows, bool slab, const 
         return code;
     };
     int rc2 = setup_kernel(c);
+    if (!rc2) rc2 = setup_march(c);
     if (rc2) return fail(rc2);
     // Zero the scalars and the ring, set the wall profiles, write the initial state.
     if (cudaMemsetAsync(c->ws + L.off_hot, 0, L.total - L.off_hot, c->stream) != cudaSuccess)
@@ -1209,19 +1336,37 @@ static cudaError_t add_step_node(cudaGraph_t g, cudaGraphNode_t prev, const cuda
     return e;
 }
 
-// A graph of graph_len (even) steps starting from buffer `from`, built node by
+// Steps of one launch in a run of n steps (march contexts: three, and two where
+// three would leave a single step; else one).
+static int launch_steps(const dmrt_ctx* c, int64_t n) {
+    if (!c->march[2] || n < 2) return 1;
+    return n != 2 && n != 4 ? 3 : 2;
+}
+// Steps of a whole graph: graph_len launches.
+static int graph_steps(const dmrt_ctx* c) { return c->graph_len * (c->march[2] ? 3 : 1); }
+
+// A graph of graph_len (an even number of) launches starting from buffer `from`, built node by
 // node (no stream capture, so it works on any stream, the legacy default included).
 static int build_graph(dmrt_ctx* c, int from) {
     cudaGraph_t g;
     CK(cudaGraphCreate(&g, 0), "cudaGraphCreate");
     cudaGraphNode_t prev = nullptr;
     dmrt::StepArgs args[2] = {step_args(c, from), step_args(c, 1 - from)};
+    dmrt::MarchArgs margs[2] = {march_args(c, from, 3), march_args(c, 1 - from, 3)};
     for (int i = 0; i < c->graph_len; ++i) {
-        const int src = (i & 1) ? 1 - from : from;
+        const int odd = i & 1;
+        const int src = odd ? 1 - from : from;
         cudaKernelNodeParams kp = {};
-        void* dparams[2] = {&args[i & 1], &c->sc};
-        void* tparams[4] = {&c->tmaps[src], &args[i & 1], &c->sc, &c->geo};
-        if (c->kernel == DMRT_KERNEL_TMA) {
+        void* dparams[2] = {&args[odd], &c->sc};
+        void* tparams[4] = {&c->tmaps[src], &args[odd], &c->sc, &c->geo};
+        void* mparams[3] = {&c->mmaps[src], &margs[odd], &c->pc};
+        if (c->march[2]) {
+            kp.func = const_cast<void*>(c->march[3]);
+            kp.gridDim = dim3(march_grid(c, 3));
+            kp.blockDim = dim3(dmrt::kMarchThreads);
+            kp.sharedMemBytes = c->msmem;
+            kp.kernelParams = mparams;
+        } else if (c->kernel == DMRT_KERNEL_TMA) {
             kp.func = const_cast<void*>(c->tma_func);
             kp.gridDim = dim3(c->tma_grid);
             kp.blockDim = dim3(c->tma_block);
@@ -1251,6 +1396,11 @@ static int build_graph(dmrt_ctx* c, int from) {
 // After a run of steps: sum the last step's local Nusselt numbers into the ring
 // (every step sums its predecessor's; the last one has no successor yet).
 static int finalize_nu(dmrt_ctx* c) {
+    if (c->march[2]) {
+        dmrt::march_finalize_kernel<<<1, dmrt::kMarchThreads, 0, c->stream>>>(march_args(c, c->cur, 2));
+        CK(cudaGetLastError(), "step launch");
+        return DMRT_OK;
+    }
     dmrt::nu_finalize_kernel<<<1, 256, 0, c->stream>>>(step_args(c, c->cur));
     CK(cudaGetLastError(), "step launch");
     return DMRT_OK;
@@ -1378,6 +1528,7 @@ static int step_run(dmrt_ctx* c, int64_t nsteps, bool finalize, float* record = 
                    "exchanged in between");
         return DMRT_E_STATE;
     }
+    bool marched = false;  // the last launch was the march kernel's
     while (nsteps > 0) {
         if (c->t >= c->next_poll) {
             // Every kPollSteps steps: stop a run that has diverged (the steps
@@ -1387,21 +1538,34 @@ static int step_run(dmrt_ctx* c, int64_t nsteps, bool finalize, float* record = 
             if (!rc) rc = poll_error(c);
             if (rc) return rc;
         }
-        if (nsteps >= c->graph_len) {
+        if (nsteps >= graph_steps(c)) {
             if (!c->graph[c->cur]) {
                 int rc = build_graph(c, c->cur);
                 if (rc) return rc;
             }
             CK(cudaGraphLaunch(c->graph[c->cur], c->stream), "cudaGraphLaunch");
-            c->t += c->graph_len;  // even length: the state stays in the same buffer
-            nsteps -= c->graph_len;
+            c->t += graph_steps(c);  // an even number of launches: the state stays in the same buffer
+            nsteps -= graph_steps(c);
+            marched = c->march[2] != nullptr;
+        } else if (const int n = launch_steps(c, nsteps); n > 1) {
+            dmrt::MarchArgs M = march_args(c, c->cur, n);
+            void* params[3] = {&c->mmaps[c->cur], &M, &c->pc};
+            CK(launch_overlapped(c->march[n], dim3(march_grid(c, n)), dim3(dmrt::kMarchThreads), c->msmem, c->stream, params),
+               "march launch");
+            c->cur ^= 1;
+            c->t += n;
+            nsteps -= n;
+            marched = true;
         } else {
-            int rc = launch_one(c);
+            // (a single step sums one earlier step's Nusselt rows, not a march launch's two)
+            int rc = marched ? finalize_nu(c) : DMRT_OK;
+            if (!rc) rc = launch_one(c);
             if (rc) return rc;
+            marched = false;
             nsteps -= 1;
         }
     }
-    return finalize ? finalize_nu(c) : DMRT_OK;
+    return finalize || marched ? finalize_nu(c) : DMRT_OK;
 }
 
 int dmrt_step(dmrt_ctx* c, int64_t nsteps) { return step_run(c, nsteps, true); }

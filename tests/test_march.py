@@ -1,0 +1,67 @@
+"""The march kernel (several steps per launch, AUTO's choice for runs of steps of
+larger cavities) against the one-step TMA kernel: a launch gives the bits of
+its single steps, in every storage mode and rounding, at the edges of its strips
+(60 columns in float32, 56 in 16-bit storage), of its row chunks, and for every
+remainder of a run after launches of three and two steps."""
+import os
+import subprocess
+import sys
+
+import numpy as np
+import pytest
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+sys.path.insert(0, ROOT)
+
+pytestmark = pytest.mark.gpu
+
+RUNS = (1, 2, 3, 4, 5, 7, 200, 1)  # 200: past a graph of 64 launches
+MODES = [(0, 0), (1, 0), (1, 1), (2, 0), (2, 1), (3, 0), (3, 1), (4, 0), (4, 1)]
+SIZES = [(60 * 4, 170), (60 * 4 + 1, 171), (56 * 4, 181), (56 * 4 - 1, 180), (160, 251), (181, 667), (5000, 9), (383, 389)]
+
+
+def advance(nx, ny, storage, rounding, kernel, walls=(0, 0), cap=4096):
+    from paper_1601_04633_gb300 import dmrt as D
+
+    p = D.make_params(nx, ny, 1e4, 0.01, storage=storage, rounding=rounding, kernel=kernel, nu_capacity=cap,
+                      left_wall=walls[0], right_wall=walls[1], theta_ref=0.1)
+    rng = np.random.default_rng(nx * 10007 + ny)
+    sim = D.Cavity2D(p, theta0=0.3 * rng.standard_normal((ny, nx)),
+                     theta_hot_profile=0.5 + 0.01 * rng.standard_normal(ny))
+    for n in RUNS:
+        sim.step(n)
+    sim.check()
+    mean, rows, series = sim.nusselt(cap)
+    out = [sim.get_state(), rows, series, np.array(mean)] + [t.cpu().numpy() for t in sim.fields()]
+    sim.close()
+    return out
+
+
+def assert_same(a, b):
+    for x, y in zip(a, b):
+        np.testing.assert_array_equal(x, y)
+
+
+@pytest.mark.parametrize("storage,rounding", MODES)
+@pytest.mark.parametrize("nx,ny", SIZES)
+def test_march_equals_single_steps(nx, ny, storage, rounding):
+    assert nx * ny >= 40000 and nx >= 160  # the sizes that AUTO marches
+    assert_same(advance(nx, ny, storage, rounding, 0), advance(nx, ny, storage, rounding, 2))
+
+
+@pytest.mark.parametrize("walls", [(1, 0), (0, 1), (1, 1)])
+@pytest.mark.parametrize("storage", [0, 3, 4])
+def test_march_wall_kinds(walls, storage):
+    assert_same(advance(243, 170, storage, 2, 0, walls), advance(243, 170, storage, 2, 2, walls))
+
+
+@pytest.mark.parametrize("cap", [1, 2, 5])
+def test_march_short_nusselt_ring(cap):
+    assert_same(advance(243, 170, 0, 0, 0, cap=cap), advance(243, 170, 0, 0, 2, cap=cap))
+
+
+def test_march_bounds_checked_build():
+    code = ("import sys; sys.path.insert(0, %r); from tests.test_march import advance;"
+            "[advance(nx, ny, s, 2, 0) for nx, ny in ((241, 171), (160, 251), (223, 180)) for s in range(5)]" % ROOT)
+    subprocess.run([sys.executable, "-c", code], check=True, cwd=ROOT,
+                   env=dict(os.environ, DMRT_LIBRARY="bounds_check"))
