@@ -1336,11 +1336,14 @@ static cudaError_t add_step_node(cudaGraph_t g, cudaGraphNode_t prev, const cuda
     return e;
 }
 
-// Steps of one launch in a run of n steps (march contexts: three, and two where
-// three would leave a single step; else one).
+// Steps of the next launch in a run of n steps. A march launch of three steps
+// changes buffers once, as three single launches would; two steps go in a
+// launch only in pairs, so that a run of n steps always ends in the buffer that
+// n single steps would end in (a batch's members, and replays of captured
+// runs, rely on it).
 static int launch_steps(const dmrt_ctx* c, int64_t n) {
-    if (!c->march[2] || n < 2) return 1;
-    return n != 2 && n != 4 ? 3 : 2;
+    if (!c->march[2] || n < 3) return 1;
+    return n == 4 || n == 5 ? 2 : 3;
 }
 // Steps of a whole graph: graph_len launches.
 static int graph_steps(const dmrt_ctx* c) { return c->graph_len * (c->march[2] ? 3 : 1); }
@@ -1529,6 +1532,7 @@ static int step_run(dmrt_ctx* c, int64_t nsteps, bool finalize, float* record = 
         return DMRT_E_STATE;
     }
     bool marched = false;  // the last launch was the march kernel's
+    bool pair = false;     // half of a pair of two-step launches is done
     while (nsteps > 0) {
         if (c->t >= c->next_poll) {
             // Every kPollSteps steps: stop a run that has diverged (the steps
@@ -1547,7 +1551,8 @@ static int step_run(dmrt_ctx* c, int64_t nsteps, bool finalize, float* record = 
             c->t += graph_steps(c);  // an even number of launches: the state stays in the same buffer
             nsteps -= graph_steps(c);
             marched = c->march[2] != nullptr;
-        } else if (const int n = launch_steps(c, nsteps); n > 1) {
+        } else if (const int n = pair ? 2 : launch_steps(c, nsteps); n > 1) {
+            pair = n == 2 && !pair;  // the second launch of a pair
             dmrt::MarchArgs M = march_args(c, c->cur, n);
             void* params[3] = {&c->mmaps[c->cur], &M, &c->pc};
             CK(launch_overlapped(c->march[n], dim3(march_grid(c, n)), dim3(dmrt::kMarchThreads), c->msmem, c->stream, params),

@@ -37,6 +37,27 @@ def advance(nx, ny, storage, rounding, kernel, walls=(0, 0), cap=4096):
     return out
 
 
+def test_march_members_stay_in_phase():
+    """A batch takes members that were stepped alone by an even number of steps."""
+    from paper_1601_04633_gb300 import dmrt as D
+    from paper_1601_04633_gb300 import inputs
+
+    cavs = [inputs.Cavity(230, 200, 1e4, 0.01, seed=s) for s in (1, 2)]
+    for n in (2, 4, 6, 8, 10, 14):
+        b = D.Batch.from_inputs(cavs, nu_capacity=64)
+        b.members[0].step(n)
+        b.step(3)
+        b.members[1].step(n)
+        b.check()
+        states = [m.get_state() for m in b.members]
+        b.close()
+        for c, got in zip(cavs, states):
+            sim = D.Cavity2D.from_inputs(c, kernel=D.DMRT_KERNEL_TMA, nu_capacity=64)
+            sim.step(n + 3)
+            np.testing.assert_array_equal(sim.get_state(), got)
+            sim.close()
+
+
 def assert_same(a, b):
     for x, y in zip(a, b):
         np.testing.assert_array_equal(x, y)
