@@ -27,10 +27,16 @@ __device__ __forceinline__ F2 f2_pack(float lo, float hi) {
     return d;
 }
 __device__ __forceinline__ float f2_lo(F2 a) {
-    return __uint_as_float((unsigned)a);
+    float lo, hi;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(a));
+    (void)hi;
+    return lo;
 }
 __device__ __forceinline__ float f2_hi(F2 a) {
-    return __uint_as_float((unsigned)(a >> 32));
+    float lo, hi;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(a));
+    (void)lo;
+    return hi;
 }
 __device__ __forceinline__ F2 f2_set(F2 a, bool hi, float v) {
     return hi ? f2_pack(f2_lo(a), v) : f2_pack(v, f2_hi(a));

@@ -22,6 +22,7 @@
 #include "step_direct.cuh"
 #include "step_tma.cuh"
 #include "step_tma_batch.cuh"
+#include "step_band.cuh"
 #include "step_march.cuh"
 #include "tma_variants.h"
 
@@ -41,6 +42,7 @@ struct Layout {
                           // float16 flow planes, a float32 theta plane, 4 float16
                           // deviation planes)
     size_t off_a, off_b, off_hot, off_cold, off_rows, off_ring, off_misc;
+    size_t off_mail, off_record;  // band kernel: messages, theta at x = 0, 1 by step (0: none)
     size_t total;
 };
 
@@ -64,8 +66,27 @@ dmrt_params resolved(const dmrt_params& p) {
     return q;
 }
 
-// halo_rows: extra population rows held by a y-slab (one below, one above its ny rows).
-Layout make_layout(const dmrt_params& p, int halo_rows = 0) {
+// Band kernel (step_band.cuh): rows per block over at most kBandBlocks blocks.
+// At least two, since a row next to both neighbours waits for one message after
+// the other (64^2 to 128^2: 1.8 us per step with one row, 1.3 with two), but one
+// where a row alone fills half a block (900 x 100: 2.9 and 3.7 us).
+constexpr int kBandBlocks = 152;
+int band_rows(const dmrt_params& p) {
+    return std::min(p.ny, std::max(p.nx > 512 ? 1 : 2, (p.ny + kBandBlocks - 1) / kBandBlocks));
+}
+// Whether a cavity's rows split like this fit the blocks' shared memory (up to
+// about 512^2), under AUTO. Batch members (stepped by the batch's launches) go without.
+bool band_fits(const dmrt_params& p) {
+    if (p.kernel != DMRT_KERNEL_AUTO || p.tma_npt > 0 || p.tma_rows > 0 || p.tma_stages > 0) return false;
+    return p.nx >= 8 && p.nx <= 1024 && dmrt::band_smem(band_rows(p), p.nx) <= (size_t)dmrt::kMaxSmem;
+}
+size_t band_mail_bytes(const dmrt_params& p) {
+    return (size_t)2 * std::min(p.ny, kBandBlocks) * 2 * 4 * dmrt::band_stride(p.nx) * sizeof(unsigned long long);
+}
+
+// halo_rows: extra population rows held by a y-slab (one below, one above its ny
+// rows); band: with the band kernel's messages and record.
+Layout make_layout(const dmrt_params& p, int halo_rows = 0, bool band = false) {
     Layout L;
     L.pitch = ((p.nx + 127) / 128) * 128;
     L.plane = (long long)(p.ny + halo_rows) * L.pitch;
@@ -78,6 +99,11 @@ Layout make_layout(const dmrt_params& p, int halo_rows = 0) {
     L.off_rows = o; o += align256((size_t)2 * dmrt::kMarchMax * p.ny * sizeof(double));  // by source buffer; march launches: each of their steps
     L.off_ring = o; o += align256((size_t)p.nu_capacity * sizeof(double));
     L.off_misc = o; o += 256;
+    L.off_mail = L.off_record = 0;
+    if (band && band_fits(p)) {
+        L.off_mail = o; o += align256(band_mail_bytes(p));
+        L.off_record = o; o += align256((size_t)dmrt::kBandSteps * p.ny * sizeof(dmrt::F2));
+    }
     L.total = o;
     return L;
 }
@@ -92,6 +118,11 @@ struct Misc {
     double nu_last;      // mean Nu of the latest step
     unsigned pending;    // the last step's local Nu rows are not yet summed into the ring
     unsigned err;        // error bits
+};
+// The band kernel's scalars (second half of the block; kept when a checkpoint is loaded).
+struct BandScalars {
+    unsigned epoch;      // tags used so far
+    long long t_base;    // steps before the launch in flight
 };
 
 }  // namespace
@@ -135,6 +166,11 @@ struct dmrt_ctx {
     unsigned msmem;
     dmrt::MarchMaps mmaps[2];  // per source buffer
     dmrt::PairConsts pc;
+    // Band kernel (many steps per launch, the cavity on chip across the GPU).
+    const void* band;    // nullptr: not used
+    int brows, bblocks, bthreads;
+    size_t bsmem;
+    bool nu_open;        // a step's Nusselt rows may not be in the ring yet
     cudaGraphExec_t graph[2];
     int graph_len;
     long long nu_floor;  // ring values of steps before this one are unavailable (after a load)
@@ -171,6 +207,7 @@ int cuda_fail(dmrt_ctx* c, cudaError_t e, const char* what) {
 float* buf(dmrt_ctx* c, int which) {
     return reinterpret_cast<float*>(c->ws + (which == 0 ? c->L.off_a : c->L.off_b));
 }
+BandScalars* band_scalars(dmrt_ctx* c) { return reinterpret_cast<BandScalars*>(c->ws + c->L.off_misc + 128); }
 Misc* misc(dmrt_ctx* c) { return reinterpret_cast<Misc*>(c->ws + c->L.off_misc); }
 // Local Nu rows of the last step taken (it ran from buffer 1 - cur).
 double* last_rows(dmrt_ctx* c) {
@@ -747,8 +784,9 @@ int setup_cluster(dmrt_ctx* c) {
 // AUTO takes the cluster kernel for runs of steps of a small float32 cavity:
 // rows split over 16 blocks with at most 1024 nodes per block (e.g. up to
 // 128^2), whose state fits the cluster's shared memory, and no tile asked for.
-// Measured per step, cluster / one-row TMA items: 16^2 1.23 / 3.11, 32^2 1.23 /
-// 2.98, 64^2 1.43 / 2.66, 96^2 1.65 / 2.95, 128^2 2.60 / 2.78 us.
+// Measured per step, cluster / one-row TMA items: 16^2 0.98 / 3.11, 32^2 0.98 /
+// 2.98, 64^2 1.13 / 2.66, 96^2 1.39 / 2.95, 128^2 2.52 / 2.78 us. (Runs of the
+// larger of these step with the band kernel, see setup_band.)
 bool auto_cluster(const dmrt_params& p) {
     if (p.kernel != DMRT_KERNEL_AUTO || p.storage != DMRT_FP32) return false;
     if (p.tma_npt > 0 || p.tma_rows > 0 || p.tma_stages > 0) return false;
@@ -866,8 +904,8 @@ int setup_kernel(dmrt_ctx* c) {
 // Runs of steps on the march kernel (step_march.cuh): three steps per launch,
 // two where three would leave a single step.
 //
-// AUTO takes it for whole cavities of at least 40000 nodes and 160 columns that
-// do not fit a cluster. Microseconds per step, march / one launch per step, on one GB300:
+// AUTO takes it for whole cavities of at least 40000 nodes and 160 columns (runs
+// too short for, or cavities too large for, the band kernel). Microseconds per step, march / one launch per step, on one GB300:
 // float32 192^2 3.4 / 3.1, 256^2 3.4 / 4.2, 512^2 6.1 / 9.5, 1024^2 12.7 / 22.7,
 // 2048^2 34.6 / 78.0, 4096^2 118 / 288; mixed, stochastic 128^2 3.7 / 3.0, 256^2
 // 3.7 / 4.4, 1024^2 14.6 / 20.0, 4096^2 145 / 212; THETA32, stochastic 1024^2
@@ -952,6 +990,41 @@ int setup_march(dmrt_ctx* c) {
     c->march[3] = F.func;
     return DMRT_OK;
 }
+// Runs of at least kBandMinSteps steps on the band kernel: AUTO's choice for
+// whole cavities that fit it, in every storage mode, but for small float32
+// cavities, where a cluster's barrier costs less than messages through L2 (at
+// most kClusterNodes nodes per block of the cluster). Microseconds per step,
+// band / cluster / the kernels above: float32 64^2 1.28 / 1.13 / 2.7, 80^2 1.29 /
+// 1.27, 96^2 1.30 / 1.39, 128^2 1.30 / 2.52 / 2.7, 192^2 1.41 / - / 2.97, 256^2
+// 1.54 / - / 3.39, 383 x 389 2.68 / - / 4.26, 512^2 3.49 / - / 5.51; mixed,
+// stochastic 64^2 1.33 / - / 3.26, 256^2 1.64 / - / 3.75, 512^2 3.87 / - / 6.63;
+// 100 x 500 1.44 / - / 3.90. A call of 8 steps: 128^2 20.8 us against 32.0,
+// 512^2 47.8 against 69.6.
+constexpr int kClusterNodes = 480;
+int setup_band(dmrt_ctx* c) {
+    const dmrt_params& p = c->p;
+    c->band = nullptr;
+    if (c->slab || c->L.off_mail == 0) return DMRT_OK;
+    if (c->cluster && (long long)c->crows * p.nx <= kClusterNodes) return DMRT_OK;
+    const void* fn = dmrt::band_kernel(p.storage, p.rounding);
+    int dev = 0, sms = 0, per_sm = 0, coop = 0;
+    CK(cudaGetDevice(&dev), "cudaGetDevice");
+    CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev), "SM count");
+    CK(cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev), "cooperative launch");
+    c->brows = band_rows(p);
+    c->bblocks = (p.ny + c->brows - 1) / c->brows;
+    const int pairs = c->brows * (((p.nx + 1) / 2 + 31) / 32 * 32), passes = (pairs + dmrt::kBandThreads - 1) / dmrt::kBandThreads;
+    c->bthreads = ((pairs + passes - 1) / passes + 31) / 32 * 32;
+    c->bsmem = dmrt::band_smem(c->brows, p.nx);
+    CK(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)c->bsmem), "set band shared memory");
+    CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, c->bthreads, c->bsmem), "occupancy");
+    // Every block has to be resident at once.
+    if (!coop || (long long)per_sm * sms < c->bblocks) return DMRT_OK;
+    c->pc = dmrt::make_pair_consts(c->sc);
+    c->band = fn;
+    return DMRT_OK;
+}
+
 int march_grid(const dmrt_ctx* c, int steps) {
     const int per = dmrt::kMarchThreads / 32;
     return (c->mstrips * c->mchunks[steps] + per - 1) / per + 1;  // the last block sums Nusselt rows
@@ -1099,7 +1172,7 @@ int dmrt_workspace_size(const dmrt_params* p, size_t* bytes) {
     int rc = validate(p, nullptr);
     if (rc) return rc;
     if (!bytes) return DMRT_E_ARG;
-    *bytes = make_layout(*p).total;
+    *bytes = make_layout(*p, 0, true).total;
     return DMRT_OK;
 }
 
@@ -1109,8 +1182,8 @@ int dmrt_workspace_size(const dmrt_params* p, size_t* bytes) {
 // y0 = 0, rows = pg->ny, slab = false). The model constants come from the
 // whole cavity (H = pg->ny in Eqs. 9 and 18); the context's own parameters are
 // those of its rows.
-static int create_ctx(const dmrt_params* pg, int y0, int rows, bool slab, const double* theta0, void* workspace,
-                      size_t workspace_bytes, void* stream, dmrt_ctx** out) {
+static int create_ctx(const dmrt_params* pg, int y0, int rows, bool slab, bool band, const double* theta0,
+                      void* workspace, size_t workspace_bytes, void* stream, dmrt_ctx** out) {
     if (!out) {
         set_err(nullptr, "out is NULL");
         return DMRT_E_ARG;
@@ -1132,7 +1205,7 @@ static int create_ctx(const dmrt_params* pg, int y0, int rows, bool slab, const 
     dmrt_params pl = resolved(*pg);
     pl.ny = rows;
     const int row0 = slab ? 1 : 0;
-    Layout L = make_layout(pl, 2 * row0);
+    Layout L = make_layout(pl, 2 * row0, band);
     if (!workspace || (reinterpret_cast<uintptr_t>(workspace) & 255)) {
         set_err(nullptr, "workspace must be a 256-byte aligned device pointer");
         return DMRT_E_ARG;
@@ -1185,6 +1258,7 @@ static int create_ctx(const dmrt_params* pg, int y0, int rows, bool slab, const 
     };
     int rc2 = setup_kernel(c);
     if (!rc2) rc2 = setup_march(c);
+    if (!rc2) rc2 = setup_band(c);
     if (rc2) return fail(rc2);
     // Zero the scalars and the ring, set the wall profiles, write the initial state.
     if (cudaMemsetAsync(c->ws + L.off_hot, 0, L.total - L.off_hot, c->stream) != cudaSuccess)
@@ -1229,7 +1303,7 @@ int dmrt_create(const dmrt_params* p, const double* theta0, void* workspace,
         set_err(nullptr, "params is NULL");
         return DMRT_E_ARG;
     }
-    return create_ctx(p, 0, p->ny, false, theta0, workspace, workspace_bytes, stream, out);
+    return create_ctx(p, 0, p->ny, false, true, theta0, workspace, workspace_bytes, stream, out);
 }
 
 int dmrt_slab_workspace_size(const dmrt_params* p, int32_t rows, size_t* bytes) {
@@ -1255,7 +1329,7 @@ int dmrt_create_slab(const dmrt_params* p, int32_t y0, int32_t rows, const doubl
         set_err(nullptr, "params is NULL");
         return DMRT_E_ARG;
     }
-    return create_ctx(p, y0, rows, true, theta0, workspace, workspace_bytes, stream, out);
+    return create_ctx(p, y0, rows, true, false, theta0, workspace, workspace_bytes, stream, out);
 }
 
 extern "C++" {
@@ -1313,6 +1387,7 @@ static int launch_one(dmrt_ctx* c) {
     if (rc) return rc;
     c->cur ^= 1;
     c->t += 1;
+    c->nu_open = true;
     return DMRT_OK;
 }
 
@@ -1399,6 +1474,7 @@ static int build_graph(dmrt_ctx* c, int from) {
 // After a run of steps: sum the last step's local Nusselt numbers into the ring
 // (every step sums its predecessor's; the last one has no successor yet).
 static int finalize_nu(dmrt_ctx* c) {
+    c->nu_open = false;
     if (c->march[2]) {
         dmrt::march_finalize_kernel<<<1, dmrt::kMarchThreads, 0, c->stream>>>(march_args(c, c->cur, 2));
         CK(cudaGetLastError(), "step launch");
@@ -1499,6 +1575,42 @@ static int launch_cluster(dmrt_ctx* c, int n, float* record = nullptr, long long
     return DMRT_OK;
 }
 
+// n steps (at most kBandSteps) in one band launch, their Nusselt numbers included.
+static int launch_band(dmrt_ctx* c, int n, float* record = nullptr, long long stride = 0) {
+    if (c->nu_open) {
+        int rc = finalize_nu(c);
+        if (rc) return rc;
+    }
+    const int end = c->cur ^ (n & 1);
+    dmrt::BandArgs B;
+    B.M = march_args(c, c->cur, 2);
+    B.out = reinterpret_cast<unsigned char*>(buf(c, end));
+    B.record = reinterpret_cast<dmrt::F2*>(c->ws + c->L.off_record);
+    B.mail = reinterpret_cast<ulonglong2*>(c->ws + c->L.off_mail);
+    Misc* m = misc(c);
+    B.epoch = &band_scalars(c)->epoch;
+    B.t_base = &band_scalars(c)->t_base;
+    // (where a last single step, which runs from the other buffer, leaves its rows)
+    B.last_rows = reinterpret_cast<double*>(c->ws + c->L.off_rows) + (size_t)(1 - end) * c->p.ny;
+    B.step_end = &m->step[end];
+    B.steps = n;
+    B.rows = c->brows;
+    B.pairs = (c->p.nx + 1) / 2;
+    B.words = dmrt::band_stride(c->p.nx);
+    B.row_threads = (B.pairs + 31) / 32 * 32;
+    B.magic = (unsigned)((0x100000000ull + (unsigned)B.row_threads - 1) / (unsigned)B.row_threads);
+    B.states = record;
+    B.stride = stride;
+    void* params[2] = {&B, &c->pc};
+    CK(cudaLaunchCooperativeKernel(c->band, dim3(c->bblocks), dim3(c->bthreads), params, c->bsmem, c->stream),
+       "band launch");
+    dmrt::band_nu_kernel<<<(n + dmrt::kBandNuWarps - 1) / dmrt::kBandNuWarps, 32 * dmrt::kBandNuWarps, 0, c->stream>>>(B);
+    CK(cudaGetLastError(), "band Nusselt launch");
+    c->cur = end;
+    c->t += n;
+    return DMRT_OK;
+}
+
 // nsteps steps; with `finalize`, the last step's Nusselt rows are summed into
 // the ring at the end (without, the next launch sums them). With `record`
 // (cluster kernel only), the state after the run's step s is also written to
@@ -1506,7 +1618,7 @@ static int launch_cluster(dmrt_ctx* c, int n, float* record = nullptr, long long
 static int step_run(dmrt_ctx* c, int64_t nsteps, bool finalize, float* record = nullptr, long long stride = 0) {
     if (!c || nsteps < 0) return DMRT_E_ARG;
     if (record && !c->cluster) return DMRT_E_ARG;
-    if (c->cluster) {
+    if (c->cluster && (!c->band || nsteps < dmrt::kBandMinSteps)) {
         while (nsteps > 0) {
             if (c->t >= c->next_poll) {
                 c->next_poll = c->t + kPollSteps;
@@ -1542,6 +1654,19 @@ static int step_run(dmrt_ctx* c, int64_t nsteps, bool finalize, float* record = 
             if (!rc) rc = poll_error(c);
             if (rc) return rc;
         }
+        if (c->band && (nsteps >= dmrt::kBandMinSteps || record)) {
+            // Up to the next divergence poll, with no remainder too short for a launch of its own.
+            long long n = std::min<long long>(nsteps, std::max<long long>(dmrt::kBandMinSteps, c->next_poll - c->t));
+            n = std::min<long long>(n, dmrt::kBandSteps);
+            const long long rest = nsteps - n;
+            if (rest > 0 && rest < dmrt::kBandMinSteps) n = nsteps <= dmrt::kBandSteps ? nsteps : n - dmrt::kBandMinSteps;
+            int rc = launch_band(c, (int)n, record, stride);
+            if (rc) return rc;
+            if (record) record += n * stride;
+            nsteps -= n;
+            finalize = finalize && nsteps > 0;
+            continue;
+        }
         if (nsteps >= graph_steps(c)) {
             if (!c->graph[c->cur]) {
                 int rc = build_graph(c, c->cur);
@@ -1551,6 +1676,7 @@ static int step_run(dmrt_ctx* c, int64_t nsteps, bool finalize, float* record = 
             c->t += graph_steps(c);  // an even number of launches: the state stays in the same buffer
             nsteps -= graph_steps(c);
             marched = c->march[2] != nullptr;
+            c->nu_open = true;
         } else if (const int n = pair ? 2 : launch_steps(c, nsteps); n > 1) {
             pair = n == 2 && !pair;  // the second launch of a pair
             dmrt::MarchArgs M = march_args(c, c->cur, n);
@@ -1561,6 +1687,7 @@ static int step_run(dmrt_ctx* c, int64_t nsteps, bool finalize, float* record = 
             c->t += n;
             nsteps -= n;
             marched = true;
+            c->nu_open = true;
         } else {
             // (a single step sums one earlier step's Nusselt rows, not a march launch's two)
             int rc = marched ? finalize_nu(c) : DMRT_OK;
@@ -2114,6 +2241,7 @@ int dmrt_load(dmrt_ctx* c, const void* host_buf, size_t size) {
     CK(cudaMemcpy(misc(c), &m, sizeof m, cudaMemcpyHostToDevice), "write scalars");
     c->t = h.t;
     c->next_poll = h.t + kPollSteps;
+    c->nu_open = false;
     c->nu_floor = h.recorded - keep;
     return DMRT_OK;
 }
@@ -2487,7 +2615,8 @@ int dmrt_batch_create(const dmrt_params* arr, int32_t n, const double* const* th
     // Members: ordinary contexts on slices of the workspace.
     for (int i = 0; i < n; ++i) {
         dmrt_ctx* c = nullptr;
-        rc = dmrt_create(&arr[i], theta0 ? theta0[i] : nullptr, b->ws + L.off[i], L.bytes[i], stream, &c);
+        rc = create_ctx(&arr[i], 0, arr[i].ny, false, false, theta0 ? theta0[i] : nullptr, b->ws + L.off[i], L.bytes[i],
+                        stream, &c);
         if (rc) {
             char msg[256];
             std::snprintf(msg, sizeof msg, "cavity %d: %.200s", i, g_create_error);

@@ -254,6 +254,11 @@ __device__ __forceinline__ F2 row_g(const unsigned char* s, int k, int c, const 
 __device__ __forceinline__ F2 pull_px(F2 v) { return f2_pack(__shfl_up_sync(kFull, f2_hi(v), 1), f2_lo(v)); }
 __device__ __forceinline__ F2 pull_mx(F2 v) { return f2_pack(f2_hi(v), __shfl_down_sync(kFull, f2_lo(v), 1)); }
 
+// A temperature wall's value: the node's own opposite, negated across a fixed-
+// temperature wall (sign), plus the wall term, which is a product rounded on
+// its own (as in the other step kernels).
+__device__ __forceinline__ float wall_value(float sign, float og, float add) { return __fmaf_rn(sign, og, add); }
+
 // Side walls at a pulled pair: links from outside x = 0 (directions 1, 5, 8 and
 // g 1) and x = nx - 1 (3, 6, 7 and g 3) from the node's own opposites: own f 3,
 // f 7, f 6, g 3 (left) or f 1, f 8, f 5, g 1 (right), and the wall's temperature term.
@@ -263,13 +268,13 @@ __device__ __forceinline__ void side_walls(F2 (&f)[9], F2 (&g)[5], const MarchLa
         f[1] = f2_set(f[1], false, of);
         f[5] = f2_set(f[5], false, oa);
         f[8] = f2_set(f[8], false, ob);
-        g[1] = f2_set(g[1], false, M.sign_l * og + add);
+        g[1] = f2_set(g[1], false, wall_value(M.sign_l, og, add));
     }
     if (n.right) {
         f[3] = f2_set(f[3], n.rhi, of);
         f[6] = f2_set(f[6], n.rhi, oa);
         f[7] = f2_set(f[7], n.rhi, ob);
-        g[3] = f2_set(g[3], n.rhi, M.sign_r * og + add);
+        g[3] = f2_set(g[3], n.rhi, wall_value(M.sign_r, og, add));
     }
 }
 
@@ -465,7 +470,7 @@ __global__ void __launch_bounds__(kMarchThreads, MINB)
         X.wa = X.wadd = 0.f;
     }
     auto wall_term = [&](int r) {
-        return n.left ? M.abb_l * __ldg(A.hot + r) : n.right ? M.abb_r * __ldg(A.cold + r) : 0.f;
+        return n.left ? __fmul_rn(M.abb_l, __ldg(A.hot + r)) : n.right ? __fmul_rn(M.abb_r, __ldg(A.cold + r)) : 0.f;
     };
     float nadd = n.wall ? wall_term(rs) : 0.f;  // the next row's wall term
     auto own = [&](F2 v) { return n.right && n.rhi ? f2_hi(v) : f2_lo(v); };
