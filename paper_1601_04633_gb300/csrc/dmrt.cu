@@ -736,7 +736,8 @@ bool cluster_fit(dmrt_ctx* c, int* csize_out, int* crows_out, int* threads_out, 
             (void)cudaGetLastError();
             continue;
         }
-        if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) {
+        // (the limit is the kernel's, for every context: the most a block may have)
+        if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, dmrt::kMaxSmem) != cudaSuccess) {
             (void)cudaGetLastError();
             continue;
         }
@@ -1016,7 +1017,8 @@ int setup_band(dmrt_ctx* c) {
     const int pairs = c->brows * (((p.nx + 1) / 2 + 31) / 32 * 32), passes = (pairs + dmrt::kBandThreads - 1) / dmrt::kBandThreads;
     c->bthreads = ((pairs + passes - 1) / passes + 31) / 32 * 32;
     c->bsmem = dmrt::band_smem(c->brows, p.nx);
-    CK(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)c->bsmem), "set band shared memory");
+    // (the limit is the kernel's, for every context: the most a block may have)
+    CK(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, dmrt::kMaxSmem), "set band shared memory");
     CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, c->bthreads, c->bsmem), "occupancy");
     // Every block has to be resident at once.
     if (!coop || (long long)per_sm * sms < c->bblocks) return DMRT_OK;

@@ -94,6 +94,19 @@ def test_band_on_two_streams():
         np.testing.assert_array_equal(sim.get_state(), ref.get_state())
 
 
+@pytest.mark.parametrize("sizes", [((300, 290), (130, 127)), ((80, 90), (60, 60))], ids=["band", "cluster"])
+def test_a_smaller_context_leaves_a_larger_one_its_shared_memory(sizes):
+    from paper_1601_04633_gb300 import dmrt as D
+
+    sims = [D.Cavity2D(D.make_params(nx, ny, 1e3, 0.01, nu_capacity=64)) for nx, ny in sizes]
+    for sim in sims:
+        sim.step(20)
+    for sim, (nx, ny) in zip(sims, sizes):
+        ref = D.Cavity2D(D.make_params(nx, ny, 1e3, 0.01, nu_capacity=64, kernel=2))
+        ref.step(20)
+        np.testing.assert_array_equal(sim.get_state(), ref.get_state())
+
+
 def test_band_captured_and_replayed():
     """A captured run of an even number of steps goes on from where the last replay ended."""
     import torch
