@@ -27,15 +27,13 @@ __device__ __forceinline__ F2 f2_pack(float lo, float hi) {
     return d;
 }
 __device__ __forceinline__ float f2_lo(F2 a) {
-    float lo, hi;
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(a));
-    (void)hi;
+    float lo;
+    asm("mov.b64 {%0, _}, %1;" : "=f"(lo) : "l"(a));
     return lo;
 }
 __device__ __forceinline__ float f2_hi(F2 a) {
-    float lo, hi;
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(a));
-    (void)lo;
+    float hi;
+    asm("mov.b64 {_, %0}, %1;" : "=f"(hi) : "l"(a));
     return hi;
 }
 __device__ __forceinline__ F2 f2_set(F2 a, bool hi, float v) {
@@ -65,53 +63,65 @@ __device__ __forceinline__ F2 f2_all(float v) { return f2_pack(v, v); }
 
 // The constants of collide_pair as pairs (both halves equal), with the signs
 // they are used in, so that a kernel takes them from its parameters as 64-bit
-// operands.
-struct PairConsts {
+// operands: a cavity's relaxation rates, buoyancy and reference temperature,
+// and the numbers of the transforms.
+struct PairRates {
     F2 n_se36, snu4, sq12, n_seps36;
     F2 sk2, n_sk2, se20, snu4t, n_snu4t, n_a;
     F2 gbeta, theta_ref;
+};
+struct PairNumbers {
     F2 c2, m2, c3, m3, c4, m4, m1, c6, m6, m12, mh, q;  // 2, -2, 3, -3, 4, -4, -1, 1/6, -1/6, -1/12, -1/2, 1/4
 };
+struct PairConsts {
+    PairRates r;
+    PairNumbers n;
+};
 
-inline PairConsts make_pair_consts(const StepConsts& s) {
-    auto two = [](float v) {
-        unsigned u;
-        memcpy(&u, &v, sizeof u);
-        return (F2)u | ((F2)u << 32);
-    };
-    PairConsts p;
-    p.n_se36 = two(-s.se36);
-    p.snu4 = two(s.snu4);
-    p.sq12 = two(s.sq12);
-    p.n_seps36 = two(-s.seps36);
-    p.sk2 = two(s.sk2);
-    p.n_sk2 = two(-s.sk2);
-    p.se20 = two(s.se20);
-    p.snu4t = two(s.snu4t);
-    p.n_snu4t = two(-s.snu4t);
-    p.n_a = two(-s.a);
-    p.gbeta = two(s.gbeta);
-    p.theta_ref = two(s.theta_ref);
-    p.c2 = two(2.f);
-    p.m2 = two(-2.f);
-    p.c3 = two(3.f);
-    p.m3 = two(-3.f);
-    p.c4 = two(4.f);
-    p.m4 = two(-4.f);
-    p.m1 = two(-1.f);
-    p.c6 = two(1.f / 6.f);
-    p.m6 = two(-(1.f / 6.f));
-    p.m12 = two(-(1.f / 12.f));
-    p.mh = two(-0.5f);
-    p.q = two(0.25f);
+inline F2 pair_const(float v) {
+    unsigned u;
+    memcpy(&u, &v, sizeof u);
+    return (F2)u | ((F2)u << 32);
+}
+inline PairRates make_pair_rates(const StepConsts& s) {
+    PairRates p;
+    p.n_se36 = pair_const(-s.se36);
+    p.snu4 = pair_const(s.snu4);
+    p.sq12 = pair_const(s.sq12);
+    p.n_seps36 = pair_const(-s.seps36);
+    p.sk2 = pair_const(s.sk2);
+    p.n_sk2 = pair_const(-s.sk2);
+    p.se20 = pair_const(s.se20);
+    p.snu4t = pair_const(s.snu4t);
+    p.n_snu4t = pair_const(-s.snu4t);
+    p.n_a = pair_const(-s.a);
+    p.gbeta = pair_const(s.gbeta);
+    p.theta_ref = pair_const(s.theta_ref);
     return p;
 }
+inline PairNumbers make_pair_numbers() {
+    PairNumbers p;
+    p.c2 = pair_const(2.f);
+    p.m2 = pair_const(-2.f);
+    p.c3 = pair_const(3.f);
+    p.m3 = pair_const(-3.f);
+    p.c4 = pair_const(4.f);
+    p.m4 = pair_const(-4.f);
+    p.m1 = pair_const(-1.f);
+    p.c6 = pair_const(1.f / 6.f);
+    p.m6 = pair_const(-(1.f / 6.f));
+    p.m12 = pair_const(-(1.f / 12.f));
+    p.mh = pair_const(-0.5f);
+    p.q = pair_const(0.25f);
+    return p;
+}
+inline PairConsts make_pair_consts(const StepConsts& s) { return PairConsts{make_pair_rates(s), make_pair_numbers()}; }
 
 // collide_node for a pair of nodes, in place (see there for the model; n_x is
 // -x, used where it saves a negation).
-__device__ __forceinline__ void collide_pair(F2 (&f)[9], F2 (&g)[5], const PairConsts& K, F2& rho_out,
-                                             F2& theta_out) {
-    const F2 c2 = K.c2, m2 = K.m2, c3 = K.c3, m3 = K.m3, c4 = K.c4, m4 = K.m4;
+__device__ __forceinline__ void collide_pair(F2 (&f)[9], F2 (&g)[5], const PairRates& K,
+                                             const PairNumbers& C, F2& rho_out, F2& theta_out) {
+    const F2 c2 = C.c2, m2 = C.m2, c3 = C.c3, m3 = C.m3, c4 = C.c4, m4 = C.m4;
     const F2 a13 = f2_sub(f[1], f[3]), a24 = f2_sub(f[2], f[4]);
     const F2 s13 = f2_add(f[1], f[3]), s24 = f2_add(f[2], f[4]);
     const F2 a56 = f2_sub(f[5], f[6]), a78 = f2_sub(f[7], f[8]);
@@ -133,13 +143,13 @@ __device__ __forceinline__ void collide_pair(F2 (&f)[9], F2 (&g)[5], const PairC
 
     // Force terms of the moments, negated.
     const F2 Gy = f2_mul(K.gbeta, f2_sub(theta, K.theta_ref));
-    const F2 n_g12 = f2_mul(Gy, K.m12);
+    const F2 n_g12 = f2_mul(Gy, C.m12);
     const F2 n_fe = f2_mul(f2_mul(n_g12, v), f2_fma(m3, uu, c2));
-    const F2 n_fqx = f2_mul(f2_mul(f2_mul(K.mh, Gy), u), v);
-    const F2 n_fqy = f2_mul(n_g12, f2_fma(f2_mul(c3, u), u, K.m1));
-    const F2 g4 = f2_mul(K.q, Gy);
+    const F2 n_fqx = f2_mul(f2_mul(f2_mul(C.mh, Gy), u), v);
+    const F2 n_fqy = f2_mul(n_g12, f2_fma(f2_mul(c3, u), u, C.m1));
+    const F2 g4 = f2_mul(C.q, Gy);
     const F2 n_fpxx = f2_mul(f2_mul(g4, v), f2_fma(m3, n_uud, c2));
-    const F2 n_fpxy = f2_mul(f2_mul(g4, u), f2_fma(f2_mul(c3, v), v, K.m1));
+    const F2 n_fpxy = f2_mul(f2_mul(g4, u), f2_fma(f2_mul(c3, v), v, C.m1));
 
     const F2 d3 = f2_fma(K.n_se36, f2_fma(c3, uu, f2_fma(m2, rho, n_e)), n_fe);
     const F2 d4 = f2_fma(K.snu4, f2_add(pxx, n_uud), n_fpxx);
@@ -148,7 +158,7 @@ __device__ __forceinline__ void collide_pair(F2 (&f)[9], F2 (&g)[5], const PairC
     const F2 d7 = f2_fma(K.sq12, f2_add(qy, v), n_fqy);
     const F2 n_d8 = f2_fma(K.n_seps36, f2_fma(c3, uu, f2_sub(eps, rho)), n_fe);
 
-    const F2 c6 = K.c6, m6 = K.m6;
+    const F2 c6 = C.c6, m6 = C.m6;
     f[0] = f2_fma(c4, n_d8, f2_fma(c4, d3, f[0]));
     f[1] = f2_fma(m2, n_d8, f2_fma(c2, d6, f2_sub(f2_add(f[1], d3), d4)));
     f[2] = f2_fma(Gy, c6, f2_fma(m2, n_d8, f2_fma(c2, d7, f2_add(f2_add(f[2], d3), d4))));

@@ -918,17 +918,53 @@ int setup_kernel(dmrt_ctx* c) {
 constexpr long long kMarchNodes = 40000;
 constexpr int kMarchWidth = 160;
 
-// Rows per chunk of a march launch of T steps: a warp marches through chunk + 2 (T - 1)
+// The march launches' tensor maps of c, by source buffer.
+int march_maps(dmrt_ctx* c, const dmrt::MarchForm& F, dmrt::MarchMaps* maps) {
+    const dmrt_params& p = c->p;
+    for (int b = 0; b < 2; ++b) {
+        // Loads of whole rows from buffer b, stores (nx columns wide) to the other one.
+        dmrt::MarchMaps& m = maps[b];
+        std::memset(&m, 0, sizeof m);
+        char* src = reinterpret_cast<char*>(buf(c, b));
+        char* dst = reinterpret_cast<char*>(buf(c, 1 - b));
+        const size_t goff = (size_t)9 * c->L.plane * 2, doff = goff + (size_t)c->L.plane * 4;
+        int rc;
+        if (p.storage == DMRT_THETA32) {
+            rc = encode_map(c, &m.ld[0], src, DMRT_FP16, 9, 9, 1, F.box);
+            if (!rc) rc = encode_map(c, &m.ld[1], src + goff, DMRT_FP32, 1, 1, 1, F.box);
+            if (!rc) rc = encode_map(c, &m.ld[2], src + doff, DMRT_FP16, 4, 4, 1, F.box);
+            if (!rc) rc = encode_map(c, &m.st[0], dst, DMRT_FP16, 9, 9, 1, F.cols, p.nx);
+            if (!rc) rc = encode_map(c, &m.st[1], dst + goff, DMRT_FP32, 1, 1, 1, F.cols, p.nx);
+            if (!rc) rc = encode_map(c, &m.st[2], dst + doff, DMRT_FP16, 4, 4, 1, F.cols, p.nx);
+        } else if (p.storage == DMRT_MIXED) {
+            rc = encode_map(c, &m.ld[0], src, DMRT_FP16, 9, 9, 1, F.box);
+            if (!rc) rc = encode_map(c, &m.ld[1], src + goff, DMRT_FP32, 5, 5, 1, F.box);
+            if (!rc) rc = encode_map(c, &m.st[0], dst, DMRT_FP16, 9, 9, 1, F.cols, p.nx);
+            if (!rc) rc = encode_map(c, &m.st[1], dst + goff, DMRT_FP32, 5, 5, 1, F.cols, p.nx);
+        } else {
+            rc = encode_map(c, &m.ld[0], src, p.storage, kPlanes, kPlanes, 1, F.box);
+            if (!rc) rc = encode_map(c, &m.st[0], dst, p.storage, kPlanes, kPlanes, 1, F.cols, p.nx);
+        }
+        if (rc) return rc;
+    }
+    return DMRT_OK;
+}
+
+// Rows per chunk of a march launch of T steps over some cavities: a warp marches through chunk + 2 (T - 1)
 // rows, so long chunks recompute less, and short ones use more warps. The
 // cheapest under what a row's iteration took on one GB300: 1.15 us with one
 // block on an SM (one warp per scheduler), 2.0 with two, 2.14 with more; a
 // single wave of long chunks ends unevenly (4096^2: one wave of 158 rows 129 us per step, two of 80 rows 120).
-int march_chunk(int ny, int strips, int T, int sms, int per_sm) {
+int march_chunk(const std::vector<std::pair<int, int>>& cavities, int T, int sms, int per_sm) {  // (rows, strips)
     const int per = dmrt::kMarchThreads / 32;
+    int ny = 0;
+    for (const auto& c : cavities) ny = std::max(ny, c.first);
     int best = ny;
     double cost = 1e300;
     for (int chunk = 1; chunk <= ny; ++chunk) {
-        const long long blocks = ((long long)strips * ((ny + chunk - 1) / chunk) + per - 1) / per;
+        long long items = 0;
+        for (const auto& c : cavities) items += (long long)c.second * ((c.first + chunk - 1) / chunk);
+        const long long blocks = (items + per - 1) / per;
         const long long k = (blocks + sms - 1) / sms;
         const long long waves = (blocks + (long long)sms * per_sm - 1) / ((long long)sms * per_sm);
         double c = chunk + 2 * (T - 1);
@@ -956,36 +992,12 @@ int setup_march(dmrt_ctx* c) {
         CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, t == 2 ? F2.func : F.func, dmrt::kMarchThreads, F.smem),
            "occupancy");
         if (per_sm < 1) return DMRT_OK;
-        c->mchunk[t] = march_chunk(p.ny, c->mstrips, t, sms, per_sm);
+        c->mchunk[t] = march_chunk({{p.ny, c->mstrips}}, t, sms, per_sm);
         c->mchunks[t] = (p.ny + c->mchunk[t] - 1) / c->mchunk[t];
     }
     c->msmem = F.smem;
-    for (int b = 0; b < 2; ++b) {
-        // Loads of whole rows from buffer b, stores (nx columns wide) to the other one.
-        dmrt::MarchMaps& m = c->mmaps[b];
-        std::memset(&m, 0, sizeof m);
-        char* src = reinterpret_cast<char*>(buf(c, b));
-        char* dst = reinterpret_cast<char*>(buf(c, 1 - b));
-        const size_t goff = (size_t)9 * c->L.plane * 2, doff = goff + (size_t)c->L.plane * 4;
-        int rc;
-        if (p.storage == DMRT_THETA32) {
-            rc = encode_map(c, &m.ld[0], src, DMRT_FP16, 9, 9, 1, F.box);
-            if (!rc) rc = encode_map(c, &m.ld[1], src + goff, DMRT_FP32, 1, 1, 1, F.box);
-            if (!rc) rc = encode_map(c, &m.ld[2], src + doff, DMRT_FP16, 4, 4, 1, F.box);
-            if (!rc) rc = encode_map(c, &m.st[0], dst, DMRT_FP16, 9, 9, 1, F.cols, p.nx);
-            if (!rc) rc = encode_map(c, &m.st[1], dst + goff, DMRT_FP32, 1, 1, 1, F.cols, p.nx);
-            if (!rc) rc = encode_map(c, &m.st[2], dst + doff, DMRT_FP16, 4, 4, 1, F.cols, p.nx);
-        } else if (p.storage == DMRT_MIXED) {
-            rc = encode_map(c, &m.ld[0], src, DMRT_FP16, 9, 9, 1, F.box);
-            if (!rc) rc = encode_map(c, &m.ld[1], src + goff, DMRT_FP32, 5, 5, 1, F.box);
-            if (!rc) rc = encode_map(c, &m.st[0], dst, DMRT_FP16, 9, 9, 1, F.cols, p.nx);
-            if (!rc) rc = encode_map(c, &m.st[1], dst + goff, DMRT_FP32, 5, 5, 1, F.cols, p.nx);
-        } else {
-            rc = encode_map(c, &m.ld[0], src, p.storage, kPlanes, kPlanes, 1, F.box);
-            if (!rc) rc = encode_map(c, &m.st[0], dst, p.storage, kPlanes, kPlanes, 1, F.cols, p.nx);
-        }
-        if (rc) return rc;
-    }
+    const int rc = march_maps(c, F, c->mmaps);
+    if (rc) return rc;
     c->pc = dmrt::make_pair_consts(c->sc);
     c->march[2] = F2.func;
     c->march[3] = F.func;
@@ -2334,6 +2346,12 @@ struct dmrt_batch {
     const void* func;
     int K;                 // steps per launch (1: one launch per step; else the multi-step kernel)
     const void* mfunc;     // the multi-step kernel (K > 1)
+    // March launches (three steps each, two in pairs), when no tile or schedule was
+    // asked for: kernels by steps per launch, and per group of up to kMarchBatch
+    // cavities the arguments by steps and source buffer.
+    const void* march[dmrt::kMarchMax + 1];
+    unsigned msmem;
+    std::vector<dmrt::MarchBatchArgs> margs[dmrt::kMarchMax + 1][2];
     int parity;
     long long t;
     int graph_len;
@@ -2344,7 +2362,7 @@ namespace {
 
 struct BatchLayout {
     std::vector<size_t> off, bytes;
-    size_t off_cav, off_maps, off_ib, off_err, off_sync, total;
+    size_t off_cav, off_maps, off_mmaps, off_ib, off_err, off_sync, total;
 };
 
 int batch_layout(const dmrt_params* arr, int32_t n, BatchLayout* L) {
@@ -2378,6 +2396,8 @@ int batch_layout(const dmrt_params* arr, int32_t n, BatchLayout* L) {
     o += align256((size_t)n * sizeof(dmrt::BatchCavity));
     L->off_maps = o;
     o += align256((size_t)n * 2 * dmrt::kBatchMaps * sizeof(CUtensorMap));
+    L->off_mmaps = o;  // march launches: six maps per cavity and source buffer, buffer by buffer
+    o += align256((size_t)n * 2 * 6 * sizeof(CUtensorMap));
     L->off_ib = o;  // item tables of at most n groups: n + groups entries
     o += align256((size_t)(2 * n) * sizeof(int));
     L->off_err = o;  // the error word, then two pool counters per group
@@ -2508,6 +2528,68 @@ int batch_build_graph(dmrt_batch* b, BatchGroup& G, int from) {
     cudaError_t e = cudaGraphInstantiate(&G.graph[from], g, 0);
     cudaGraphDestroy(g);
     if (e != cudaSuccess) return batch_cuda_fail(b, e, "cudaGraphInstantiate");
+    return DMRT_OK;
+}
+
+// The march launches of a batch: its cavities in groups of kMarchBatch, one
+// chunk height for all of a group. Taken whenever no tile or schedule was asked
+// for. Microseconds per step of all cavities, march / one launch per step
+// (default tile): the 64-cavity sweep (sides 128 to 384) float32 46.4 / 98.6,
+// mixed stochastic 55.0 / 73.0; 512 of 32^2 49.0 / 56.4; 64 of 32^2 5.7 / 11.7; 128 of
+// 64^2 17.5 / 24.1; 64 of 128^2 16.1 / 26.8; 9 of 300 x 280 10.1 / 22.1; 3 of 1024^2
+// 29.1 / 65.7; 3 of 100 x 80 3.5 / 6.4.
+int batch_setup_march(dmrt_batch* b, CUtensorMap* d_maps, int sms) {
+    const dmrt_params& p0 = b->sub[0]->p;
+    const dmrt::MarchForm F[4] = {{}, {}, dmrt::batch_march_form(p0.storage, p0.rounding, 2),
+                                  dmrt::batch_march_form(p0.storage, p0.rounding, 3)};
+    if (!F[3].func) return DMRT_OK;
+    for (const dmrt_ctx* c : b->sub)
+        if (c->p.nx < 8) return DMRT_OK;
+    std::vector<CUtensorMap> maps((size_t)b->n * 2 * 6);
+    for (int i = 0; i < b->n; ++i) {
+        dmrt::MarchMaps m[2];
+        int rc = march_maps(b->sub[i], F[3], m);
+        if (rc) return rc;
+        for (int bf = 0; bf < 2; ++bf) std::memcpy(&maps[((size_t)bf * b->n + i) * 6], &m[bf], 6 * sizeof(CUtensorMap));
+    }
+    BCK(cudaMemcpyAsync(d_maps, maps.data(), maps.size() * sizeof(maps[0]), cudaMemcpyHostToDevice, b->stream), "march maps");
+    BCK(cudaStreamSynchronize(b->stream), "synchronize");
+    for (int t = 2; t <= dmrt::kMarchMax; ++t) {
+        int per_sm = 0;
+        BCK(cudaFuncSetAttribute(F[t].func, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)F[t].smem), "march shared memory");
+        BCK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, F[t].func, dmrt::kMarchThreads, F[t].smem), "occupancy");
+        if (per_sm < 1) return DMRT_OK;
+        for (int first = 0; first < b->n; first += dmrt::kMarchBatch) {
+            const int count = std::min(dmrt::kMarchBatch, b->n - first);
+            std::vector<std::pair<int, int>> cav;
+            for (int i = first; i < first + count; ++i)
+                cav.emplace_back(b->sub[i]->p.ny, (b->sub[i]->p.nx + F[t].cols - 1) / F[t].cols);
+            const int chunk = march_chunk(cav, t, sms, per_sm);
+            for (int bf = 0; bf < 2; ++bf) {
+                dmrt::MarchBatchArgs B;
+                std::memset((void*)&B, 0, sizeof B);
+                B.maps = d_maps + ((size_t)bf * b->n + first) * 6;
+                B.err = b->d_err;
+                B.n = dmrt::make_pair_numbers();
+                B.n_cav = count;
+                for (int i = 0; i < count; ++i) {
+                    dmrt_ctx* c = b->sub[first + i];
+                    dmrt::MarchArgs& M = B.M[i];
+                    M = march_args(c, bf, t);
+                    M.n_strips = cav[i].second;
+                    M.chunk = std::min(chunk, c->p.ny);
+                    M.n_chunks = (c->p.ny + M.chunk - 1) / M.chunk;
+                    B.r[i] = dmrt::make_pair_rates(c->sc);
+                    B.first[i] = B.items;
+                    B.items += M.n_strips * M.n_chunks;
+                }
+                b->margs[t][bf].push_back(B);
+            }
+        }
+    }
+    b->msmem = F[3].smem;
+    b->march[2] = F[2].func;
+    b->march[3] = F[3].func;
     return DMRT_OK;
 }
 
@@ -2802,7 +2884,29 @@ int dmrt_batch_create(const dmrt_params* arr, int32_t n, const double* const* th
         // Three quarters of the items are split statically, the rest are drawn at run time.
         G.static_per_block = (int)((long long)G.total_items * 3 / 4 / G.grid);
     }
+    if (!opts || (opts->tma_npt <= 0 && opts->tma_rows <= 0 && opts->tma_stages <= 0 && opts->graph_steps <= 0 &&
+                  opts->group_bytes <= 0 && K == 1 && !ts && !fill)) {
+        rc = batch_setup_march(b, reinterpret_cast<CUtensorMap*>(b->ws + L.off_mmaps), sms);
+        if (rc) return fail(rc);
+    }
     *out = b;
+    return DMRT_OK;
+}
+
+// n (3, or 2) steps of every cavity by march launches; n = 0: their last Nusselt sums.
+static int batch_march(dmrt_batch* b, int n, int parity) {
+    for (dmrt::MarchBatchArgs& B : b->margs[n > 0 ? n : 3][parity]) {
+        if (n == 0) {
+            dmrt::batch_march_finalize_kernel<<<B.n_cav, dmrt::kMarchThreads, 0, b->stream>>>(B);
+            BCK(cudaGetLastError(), "batch Nusselt launch");
+            continue;
+        }
+        const int per = dmrt::kMarchThreads / 32;
+        void* params[1] = {&B};
+        BCK(launch_overlapped(b->march[n], dim3((B.items + per - 1) / per + B.n_cav), dim3(dmrt::kMarchThreads), b->msmem,
+                              b->stream, params),
+            "batch march launch");
+    }
     return DMRT_OK;
 }
 
@@ -2815,10 +2919,32 @@ int dmrt_batch_step(dmrt_batch* b, int64_t nsteps) {
             return DMRT_E_STATE;
         }
     }
+    // March launches for what they take of the steps (a remainder of one or two
+    // goes to the launches of single steps).
+    const int start0 = b->parity;
+    int start = start0;
+    const int64_t total = nsteps;
+    if (b->march[3] && nsteps >= 3) {
+        while (nsteps >= 3) {
+            const int n = nsteps == 4 || nsteps == 5 ? 2 : 3;
+            for (int k = 0; k < (n == 2 ? 2 : 1); ++k) {  // two steps in pairs only (see launch_steps)
+                int rc = batch_march(b, n, start);
+                if (rc) return rc;
+                start ^= 1;
+                nsteps -= n;
+            }
+        }
+        int rc = batch_march(b, 0, start);
+        if (rc) return rc;
+    }
+    // The single-step launches' work-pool counters alternate by source buffer, which
+    // march launches in between do not keep up.
+    if (b->march[3] && nsteps > 0)
+        BCK(cudaMemsetAsync(b->d_err + 1, 0, sizeof(unsigned) * 2 * b->groups.size(), b->stream), "work-pool counters");
     // Group after group, each for all nsteps steps (independent cavities: the
     // order of the groups does not change any result).
-    const int start = b->parity;
     for (BatchGroup& G : b->groups) {
+        if (nsteps == 0 && total > 0) break;
         int parity = start;
         long long done = 0;
         while (done < nsteps) {
@@ -2840,11 +2966,11 @@ int dmrt_batch_step(dmrt_batch* b, int64_t nsteps) {
             dmrt::nu_finalize_batch_kernel<<<G.count, 256, 0, b->stream>>>(b->d_cav + G.first, parity);
         BCK(cudaGetLastError(), "batch step launch");
     }
-    b->parity = start ^ (int)(nsteps & 1);
-    b->t += nsteps;
+    b->parity = start0 ^ (int)(total & 1);
+    b->t += total;
     for (dmrt_ctx* c : b->sub) {
         c->cur = b->parity;
-        c->t += nsteps;
+        c->t += total;
     }
     return DMRT_OK;
 }

@@ -305,7 +305,7 @@ __global__ void __launch_bounds__(kBandThreads) step_band_kernel(const __grid_co
             g[1] = f2_pack(w1[0], w1[1]);
             g[3] = f2_pack(w3[0], w3[1]);
             F2 rho, theta;
-            collide_pair(f, g, K, rho, theta);
+            collide_pair(f, g, K.r, K.n, rho, theta);
             peak0 = peak_of(peak0, f2_lo(rho), f2_lo(theta));
             if (n.two) peak1 = peak_of(peak1, f2_hi(rho), f2_hi(theta));
             if (n.left) B.record[(size_t)s * ny + j] = theta;

@@ -392,34 +392,16 @@ struct MarchCarry {
     float wa, wadd;
 };
 
-template <typename L, bool SR, int T, int MINB>
-__global__ void __launch_bounds__(kMarchThreads, MINB)
-    step_march_kernel(const __grid_constant__ MarchMaps maps, const __grid_constant__ MarchArgs M,
-                      const __grid_constant__ PairConsts K) {
+// One item (strip, chunk) of a cavity by one warp: ring and bars are the warp's,
+// the barriers freshly initialised.
+template <typename L, bool SR, int T>
+__device__ __forceinline__ void march_item(const CUtensorMap* ld, const CUtensorMap* st, const MarchArgs& M,
+                                           const PairRates& K, const PairNumbers& C9, int item, int lane,
+                                           unsigned char* ring, uint64_t* bars) {
     using G = MarchGeo<L>;
     static_assert(T >= 2 && T <= kMarchMax && T - 1 <= G::kLead, "a strip's side columns");
     const StepArgs& A = M.A;
-    extern __shared__ __align__(1024) unsigned char smem_m[];
-    const int lane = threadIdx.x & 31;
-    const int warp = __shfl_sync(kFull, (int)threadIdx.x >> 5, 0);  // (uniform, as the compiler sees it)
-    unsigned char* const ring = smem_m + warp * G::kWarp;
     unsigned char* const tile = ring + kMarchStages * G::kStage;
-    uint64_t* const bars =
-        reinterpret_cast<uint64_t*>(smem_m + (kMarchThreads / 32) * G::kWarp) + warp * kMarchStages;
-    if (lane == 0) {
-        for (int s = 0; s < kMarchStages; ++s) mbar_init(&bars[s], 1);
-        mbar_fence_init();
-    }
-    grid_dep_wait();
-    grid_dep_launch();
-    // After an expired wait in an earlier launch the state is invalid: return at once.
-    if (__syncthreads_or(threadIdx.x == 0 && (*reinterpret_cast<volatile unsigned*>(A.err) & kErrTimeout))) return;
-    if (blockIdx.x == gridDim.x - 1) {  // the extra block: the previous launch's Nusselt sums
-        march_nu_finish(M, T);
-        return;
-    }
-    const int item = blockIdx.x * (kMarchThreads / 32) + warp;
-    if (item >= M.n_strips * M.n_chunks) return;
     const int cidx = item / M.n_strips, strip = item - cidx * M.n_strips;
     const int j0 = cidx * M.chunk, j1 = min(j0 + M.chunk, A.ny);
     MarchLane n;
@@ -447,9 +429,9 @@ __global__ void __launch_bounds__(kMarchThreads, MINB)
         uint64_t* b = bar(row);
         const int x = strip * G::kCols - G::kHalo;
         mbar_expect_tx(b, G::kRowBytes);
-        tma_load_3d(s, &maps.ld[0], x, row, 0, b);
-        if constexpr (L::kSplit) tma_load_3d(s + G::g_at(G::kBox), &maps.ld[1], x, row, 0, b);
-        if constexpr (L::kTheta) tma_load_3d(s + G::d_at(G::kBox), &maps.ld[2], x, row, 0, b);
+        tma_load_3d(s, &ld[0], x, row, 0, b);
+        if constexpr (L::kSplit) tma_load_3d(s + G::g_at(G::kBox), &ld[1], x, row, 0, b);
+        if constexpr (L::kTheta) tma_load_3d(s + G::d_at(G::kBox), &ld[2], x, row, 0, b);
     };
     auto arrived = [&](int row) {
         return __all_sync(kFull, mbar_wait_bounded(bar(row), (unsigned)((row - lb) / kMarchStages) & 1u));
@@ -545,7 +527,7 @@ __global__ void __launch_bounds__(kMarchThreads, MINB)
             if (lane == 0) issue(issued);
             ++issued;
         }
-        collide_pair(f, g, K, rho, theta);
+        collide_pair(f, g, K, C9, rho, theta);
         if (r < A.ny) watch(rho, theta);
         if (strip == 0) nusselt(0, r, theta);
 #pragma unroll
@@ -594,7 +576,7 @@ __global__ void __launch_bounds__(kMarchThreads, MINB)
             for (int k = 0; k < 9; ++k) f[k] = F[k];
 #pragma unroll
             for (int k = 0; k < 5; ++k) g[k] = H[k];
-            collide_pair(f, g, K, rho, theta);
+            collide_pair(f, g, K, C9, rho, theta);
             if (q < A.ny && q >= max(j0 - (T - 1 - s), 0)) watch(rho, theta);
             if (strip == 0) nusselt(s, q, theta);
         }
@@ -610,9 +592,9 @@ __global__ void __launch_bounds__(kMarchThreads, MINB)
             __syncwarp();
             if (lane == 0) {
                 const int x = strip * G::kCols;
-                tma_store_3d(&maps.st[0], tile, x, q, 0);
-                if constexpr (L::kSplit) tma_store_3d(&maps.st[1], tile + G::g_at(G::kCols), x, q, 0);
-                if constexpr (L::kTheta) tma_store_3d(&maps.st[2], tile + G::d_at(G::kCols), x, q, 0);
+                tma_store_3d(&st[0], tile, x, q, 0);
+                if constexpr (L::kSplit) tma_store_3d(&st[1], tile + G::g_at(G::kCols), x, q, 0);
+                if constexpr (L::kTheta) tma_store_3d(&st[2], tile + G::d_at(G::kCols), x, q, 0);
                 bulk_commit();
             }
         }
@@ -626,6 +608,92 @@ __global__ void __launch_bounds__(kMarchThreads, MINB)
     if (n.out && (!(peak0 < 1e30f) || (n.two && !(peak1 < 1e30f)))) atomicOr(A.err, kErrNonFinite);
 }
 
+// A warp's ring and barriers.
+template <typename L>
+__device__ __forceinline__ void march_warp(unsigned char* smem, int warp, int lane, unsigned char*& ring, uint64_t*& bars) {
+    using G = MarchGeo<L>;
+    ring = smem + warp * G::kWarp;
+    bars = reinterpret_cast<uint64_t*>(smem + (kMarchThreads / 32) * G::kWarp) + warp * kMarchStages;
+    if (lane == 0) {
+        for (int s = 0; s < kMarchStages; ++s) mbar_init(&bars[s], 1);
+        mbar_fence_init();
+    }
+}
+
+template <typename L, bool SR, int T, int MINB>
+__global__ void __launch_bounds__(kMarchThreads, MINB)
+    step_march_kernel(const __grid_constant__ MarchMaps maps, const __grid_constant__ MarchArgs M,
+                      const __grid_constant__ PairConsts K) {
+    extern __shared__ __align__(1024) unsigned char smem_m[];
+    const int lane = threadIdx.x & 31;
+    const int warp = __shfl_sync(kFull, (int)threadIdx.x >> 5, 0);  // (uniform, as the compiler sees it)
+    unsigned char* ring;
+    uint64_t* bars;
+    march_warp<L>(smem_m, warp, lane, ring, bars);
+    grid_dep_wait();
+    grid_dep_launch();
+    // After an expired wait in an earlier launch the state is invalid: return at once.
+    if (__syncthreads_or(threadIdx.x == 0 && (*reinterpret_cast<volatile unsigned*>(M.A.err) & kErrTimeout))) return;
+    if (blockIdx.x == gridDim.x - 1) {  // the extra block: the previous launch's Nusselt sums
+        march_nu_finish(M, T);
+        return;
+    }
+    const int item = blockIdx.x * (kMarchThreads / 32) + warp;
+    if (item >= M.n_strips * M.n_chunks) return;
+    march_item<L, SR, T>(maps.ld, maps.st, M, K.r, K.n, item, lane, ring, bars);
+}
+
+// ---- batched sweep ----------------------------------------------------------------
+// The same launch over the items of up to kMarchBatch cavities, cavity after
+// cavity. The cavities' arguments and rates are kernel parameters, so that a
+// warp takes them from the constant bank at its cavity's (uniform) index, as
+// the single-cavity kernel does; the tensor maps lie in global memory. The last
+// n_cav blocks take the cavities' Nusselt sums.
+constexpr int kMarchBatch = 64;
+struct MarchBatchArgs {
+    const CUtensorMap* maps;  // [n_cav][6]: loads, stores of this launch's source buffer
+    unsigned* err;            // the batch's error word (an expired wait)
+    PairNumbers n;
+    int n_cav, items;
+    int first[kMarchBatch];   // first item of each cavity
+    MarchArgs M[kMarchBatch];
+    PairRates r[kMarchBatch];
+};
+
+template <typename L, bool SR, int T, int MINB>
+__global__ void __launch_bounds__(kMarchThreads, MINB) batch_march_kernel(const __grid_constant__ MarchBatchArgs B) {
+    extern __shared__ __align__(1024) unsigned char smem_m[];
+    const int lane = threadIdx.x & 31;
+    const int warp = __shfl_sync(kFull, (int)threadIdx.x >> 5, 0);
+    unsigned char* ring;
+    uint64_t* bars;
+    march_warp<L>(smem_m, warp, lane, ring, bars);
+    grid_dep_wait();
+    grid_dep_launch();
+    if (__syncthreads_or(threadIdx.x == 0 && (*reinterpret_cast<volatile unsigned*>(B.err) & kErrTimeout))) return;
+    const int extra = (int)blockIdx.x - ((int)gridDim.x - B.n_cav);
+    if (extra >= 0) {
+        march_nu_finish(B.M[extra], T);
+        return;
+    }
+    const int item = blockIdx.x * (kMarchThreads / 32) + warp;
+    if (item >= B.items) return;
+    int lo = 0, hi = B.n_cav - 1;  // the cavity whose items hold this one
+    while (lo < hi) {
+        const int mid = (lo + hi + 1) / 2;
+        if (B.first[mid] <= item) lo = mid;
+        else hi = mid - 1;
+    }
+    const CUtensorMap* maps = B.maps + (size_t)lo * 6;
+    march_item<L, SR, T>(maps, maps + 3, B.M[lo], B.r[lo], B.n, item - B.first[lo], lane, ring, bars);
+    if (lane == 0 && (*reinterpret_cast<volatile unsigned*>(B.M[lo].A.err) & kErrTimeout)) atomicOr(B.err, kErrTimeout);
+}
+
+// The last launch's Nusselt sums of every cavity, one block each.
+static __global__ void batch_march_finalize_kernel(const __grid_constant__ MarchBatchArgs B) {
+    march_nu_finish(B.M[blockIdx.x], 0);
+}
+
 // The compiled form for a storage, rounding and steps per launch, its shared memory, and the
 // columns of a strip, of a load box and left of the strip (nullptr: none).
 struct MarchForm {
@@ -634,5 +702,6 @@ struct MarchForm {
     int cols, box;
 };
 MarchForm march_form(int storage, int rounding, int steps);
+MarchForm batch_march_form(int storage, int rounding, int steps);  // float32 and mixed storage
 
 }  // namespace dmrt

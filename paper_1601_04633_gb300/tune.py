@@ -120,12 +120,15 @@ def tune_batch(cavities, steps=200, warmup=20, tiles=None, graph_steps=(64,), ca
         trials.append({"opts": opts, "mlups": nodes * steps / sec / 1e6, "groups": b.groups})
         b.close()
 
+    if tiles is None:
+        # No tile asked for: the library's own launches of three steps.
+        trial(0, 0, 0, 0, 0, 0)
     for npt, R, S in (tiles or BATCH_TILES):
         for g in graph_steps:
             for fill in strip_fill:
                 trial(npt, R, S, g, group_bytes[0], 1, fill=fill)
     if len(group_bytes) > 1 or len(steps_per_launch) > 1 or tensor_store:
-        top = sorted(trials, key=lambda r: -r["mlups"])[:finalists]
+        top = sorted((t for t in trials if t["opts"]["tma_npt"]), key=lambda r: -r["mlups"])[:finalists]
         for t in top:
             o = t["opts"]
             tile = (o["tma_npt"], o["tma_rows"], o["tma_stages"])

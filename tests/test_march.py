@@ -58,6 +58,37 @@ def test_march_members_stay_in_phase():
             sim.close()
 
 
+@pytest.mark.parametrize("storage,rounding", [(0, 0), (3, 0), (3, 1)])
+@pytest.mark.parametrize("count", [1, 3, 70])
+def test_march_batch_equals_members_alone(count, storage, rounding):
+    """Batches stepped by march launches (no tile asked for), one and two groups of
+    cavities, with single steps and members stepped alone in between."""
+    from paper_1601_04633_gb300 import dmrt as D
+    from paper_1601_04633_gb300 import inputs
+
+    rng = np.random.default_rng(count)
+    cavs = []
+    for k in range(count):
+        nx, ny = int(rng.integers(8, 150) if count > 3 else rng.integers(100, 400)), int(rng.integers(20, 150))
+        cavs.append(inputs.Cavity(nx, ny, min(1e4, 0.01 * (12 * ny) ** 2), 0.01, noise_amp=1e-2, seed=k))
+    b = D.Batch.from_inputs(cavs, nu_capacity=512, storage=storage, rounding=rounding)
+    for n in RUNS[:6] + (64, 8, 1):
+        b.step(n)
+    b.members[0].step(4)
+    b.step(3)
+    b.check()
+    total = sum(RUNS[:6]) + 64 + 8 + 1 + 3
+    for i in range(0, count, 9 if count > 3 else 1):
+        ref = D.Cavity2D.from_inputs(cavs[i], nu_capacity=512, storage=storage, rounding=rounding, kernel=2)
+        ref.step(total + (4 if i == 0 else 0))
+        got, want = b.members[i].nusselt(512), ref.nusselt(512)
+        np.testing.assert_array_equal(b.members[i].get_state(), ref.get_state())
+        np.testing.assert_array_equal(got[2], want[2])
+        np.testing.assert_array_equal(got[1], want[1])
+        ref.close()
+    b.close()
+
+
 def assert_same(a, b):
     for x, y in zip(a, b):
         np.testing.assert_array_equal(x, y)
