@@ -350,12 +350,15 @@ __global__ void fields_kernel(const unsigned char* __restrict__ S, float* __rest
                               float* __restrict__ v, float* __restrict__ th, int nx, int ny,
                               int pitch, long long plane, float gbeta, float theta_ref,
                               float sh0, float sh1, int row0) {
+    dmrt::grid_dep_wait();  // (launched while the last step finishes)
     const auto* Sf = f_base<L>(S);
     const auto* Sg = g_base<L>(S, plane);
-    const long long n = (long long)nx * ny;
-    for (long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x; q < n;
-         q += (long long)gridDim.x * blockDim.x) {
-        const int j = (int)(q / nx), i = (int)(q % nx);
+    // Tiles of blockDim.x nodes of a row: one 32-bit division per tile, none per node.
+    const int tx = (nx + (int)blockDim.x - 1) / (int)blockDim.x;
+    for (int tile = blockIdx.x; tile < tx * ny; tile += gridDim.x) {
+        const int j = tile / tx, i = (tile - j * tx) * (int)blockDim.x + (int)threadIdx.x;
+        if (i >= nx) continue;
+        const long long q = (long long)j * nx + i;
         const long long s = (long long)(j + row0) * pitch + i;
         float f[9];
         for (int k = 0; k < 9; ++k) f[k] = elem_to_f(Sf[L::pf(k) * plane + s]);
@@ -1490,12 +1493,12 @@ static int build_graph(dmrt_ctx* c, int from) {
 static int finalize_nu(dmrt_ctx* c) {
     c->nu_open = false;
     if (c->march[2]) {
-        dmrt::march_finalize_kernel<<<1, dmrt::kMarchThreads, 0, c->stream>>>(march_args(c, c->cur, 2));
-        CK(cudaGetLastError(), "step launch");
+        CK(launch_overlapped(dmrt::march_finalize_kernel, dim3(1), dim3(dmrt::kMarchThreads), c->stream,
+                             march_args(c, c->cur, 2)),
+           "step launch");
         return DMRT_OK;
     }
-    dmrt::nu_finalize_kernel<<<1, 256, 0, c->stream>>>(step_args(c, c->cur));
-    CK(cudaGetLastError(), "step launch");
+    CK(launch_overlapped(dmrt::nu_finalize_kernel, dim3(1), dim3(256), c->stream, step_args(c, c->cur)), "step launch");
     return DMRT_OK;
 }
 
@@ -1895,15 +1898,18 @@ int dmrt_fields(dmrt_ctx* c, float* u, float* v, float* theta, int on_device) {
         dv = v ? stage + n : nullptr;
         dt = theta ? stage + 2 * n : nullptr;
     }
-    const int blocks = (int)std::min<long long>((n + 255) / 256, 152 * 16);
+    // Tiles of up to 256 nodes of a row, a power of two near the row's length.
+    int width = 32;
+    while (width < 256 && width < p.nx) width *= 2;
+    const int blocks = (int)std::min<long long>((long long)((p.nx + width - 1) / width) * p.ny, 152 * 2048 / width);
+    cudaError_t fe = cudaSuccess;
     with_layout(p.storage, [&](auto tag) {
         using Lt = decltype(tag);
-        fields_kernel<Lt><<<blocks, 256, 0, c->stream>>>(reinterpret_cast<const unsigned char*>(buf(c, c->cur)),
-                                                         du, dv, dt, p.nx, p.ny, c->L.pitch, c->L.plane,
-                                                         c->sc.gbeta, c->sc.theta_ref, c->sc.gsh0, c->sc.gsh1,
-                                                         c->row0);
+        fe = launch_overlapped(fields_kernel<Lt>, dim3(blocks), dim3(width), c->stream,
+                               reinterpret_cast<const unsigned char*>(buf(c, c->cur)), du, dv, dt, p.nx, p.ny, c->L.pitch,
+                               c->L.plane, c->sc.gbeta, c->sc.theta_ref, c->sc.gsh0, c->sc.gsh1, c->row0);
     });
-    CK(cudaGetLastError(), "fields kernel");
+    CK(fe, "fields kernel");
     if (!on_device) {
         if (u) CK(cudaMemcpyAsync(u, du, n * sizeof(float), cudaMemcpyDeviceToHost, c->stream), "copy u");
         if (v) CK(cudaMemcpyAsync(v, dv, n * sizeof(float), cudaMemcpyDeviceToHost, c->stream), "copy v");

@@ -351,6 +351,9 @@ __device__ __forceinline__ void nu_finish_prev(const StepArgs& A, bool step) {
 }
 
 // Sums the last step of a run (one block of 256 threads).
-static __global__ void nu_finalize_kernel(StepArgs A) { nu_finish_prev(A, false); }
+static __global__ void nu_finalize_kernel(StepArgs A) {
+    grid_dep_wait();  // (launched while the last step finishes)
+    nu_finish_prev(A, false);
+}
 
 }  // namespace dmrt

@@ -379,7 +379,10 @@ __device__ __forceinline__ void march_nu_finish(const MarchArgs& M, int taken) {
     }
 }
 
-static __global__ void march_finalize_kernel(MarchArgs M) { march_nu_finish(M, 0); }
+static __global__ void march_finalize_kernel(MarchArgs M) {
+    grid_dep_wait();  // (launched while the last step finishes)
+    march_nu_finish(M, 0);
+}
 
 // What a step needs of the step before it (see the top), the next pull being
 // at row q: the P group of row q - 1, shifted for the pull, the P and Z groups
