@@ -1,25 +1,26 @@
-// The band kernel per storage mode and rounding.
+// The band kernel across the GPU per storage mode and rounding.
 #include "dmrt.h"
 #include "step_band.cuh"
 
 namespace dmrt {
 
-const void* band_kernel(int storage, int rounding) {
+const void* band_one_kernel(int storage, int rounding);  // band_one.cu
+
+template <typename L, bool SR>
+static const void* form() {
+    return (const void*)step_band_kernel<L, SR, false, false>;
+}
+
+const void* band_kernel(int storage, int rounding, bool one) {
     using Mixed = Split<__half, float>;
+    if (one) return band_one_kernel(storage, rounding);
     const bool sr = rounding == DMRT_ROUND_STOCHASTIC;
     switch (storage) {
-        case DMRT_FP32: return (const void*)step_band_kernel<OneType<float>, false>;
-        case DMRT_FP16:
-            return sr ? (const void*)step_band_kernel<OneType<__half>, true>
-                      : (const void*)step_band_kernel<OneType<__half>, false>;
-        case DMRT_BF16:
-            return sr ? (const void*)step_band_kernel<OneType<__nv_bfloat16>, true>
-                      : (const void*)step_band_kernel<OneType<__nv_bfloat16>, false>;
-        case DMRT_MIXED:
-            return sr ? (const void*)step_band_kernel<Mixed, true> : (const void*)step_band_kernel<Mixed, false>;
-        case DMRT_THETA32:
-            return sr ? (const void*)step_band_kernel<ThetaSplit, true>
-                      : (const void*)step_band_kernel<ThetaSplit, false>;
+        case DMRT_FP32: return form<OneType<float>, false>();
+        case DMRT_FP16: return sr ? form<OneType<__half>, true>() : form<OneType<__half>, false>();
+        case DMRT_BF16: return sr ? form<OneType<__nv_bfloat16>, true>() : form<OneType<__nv_bfloat16>, false>();
+        case DMRT_MIXED: return sr ? form<Mixed, true>() : form<Mixed, false>();
+        case DMRT_THETA32: return sr ? form<ThetaSplit, true>() : form<ThetaSplit, false>();
     }
     return nullptr;
 }

@@ -168,6 +168,7 @@ struct dmrt_ctx {
     dmrt::PairConsts pc;
     // Band kernel (many steps per launch, the cavity on chip across the GPU).
     const void* band;    // nullptr: not used
+    bool band_cluster;   // its blocks form one cluster
     int brows, bblocks, bthreads;
     size_t bsmem;
     bool nu_open;        // a step's Nusselt rows may not be in the ring yet
@@ -1007,31 +1008,74 @@ int setup_march(dmrt_ctx* c) {
     return DMRT_OK;
 }
 // Runs of at least kBandMinSteps steps on the band kernel: AUTO's choice for
-// whole cavities that fit it, in every storage mode, but for small float32
-// cavities, where a cluster's barrier costs less than messages through L2 (at
-// most kClusterNodes nodes per block of the cluster). Microseconds per step,
-// band / cluster / the kernels above: float32 64^2 1.28 / 1.13 / 2.7, 80^2 1.29 /
-// 1.27, 96^2 1.30 / 1.39, 128^2 1.30 / 2.52 / 2.7, 192^2 1.41 / - / 2.97, 256^2
-// 1.54 / - / 3.39, 383 x 389 2.68 / - / 4.26, 512^2 3.49 / - / 5.51; mixed,
-// stochastic 64^2 1.33 / - / 3.26, 256^2 1.64 / - / 3.75, 512^2 3.87 / - / 6.63;
-// 100 x 500 1.44 / - / 3.90. A call of 8 steps: 128^2 20.8 us against 32.0,
-// 512^2 47.8 against 69.6.
+// whole cavities that fit it, in every storage mode. In one cluster while its
+// blocks hold at most kBandClusterItems pairs (rows rounded up to whole warps),
+// else across the GPU; the smallest float32 cavities, and those of at most
+// kClusterNodes nodes per block in between, stay with step_cluster.cuh.
+// Microseconds per step, one cluster / across the GPU / step_cluster.cuh / one
+// or three steps per launch: float32 16^2 1.10 / 1.26 / 0.97 / 2.7, 32^2 0.98 / 1.25 /
+// 0.96, 64^2 0.92 / 1.24 / 1.12, 100 x 60 1.11 / 1.25 / 1.19, 80^2 1.27 / 1.25 / 1.25,
+// 96^2 1.35 / 1.25 / 1.39, 128^2 1.63 / 1.24 / 2.52 / 2.7, 192^2 - / 1.33 / - / 2.97,
+// 256^2 - / 1.44 / - / 3.39, 383 x 389 - / 2.67 / - / 4.26, 512^2 - / 3.49 / - / 5.51;
+// mixed, stochastic 64^2 0.95 / 1.28 / - / 3.26, 96^2 1.46 / 1.29, 256^2 - / 1.58 / - /
+// 3.75, 512^2 - / 3.87 / - / 6.63; 100 x 500 float32 - / 1.41 / - / 3.90. A call of 8
+// steps: 128^2 20.8 us against 32.0, 512^2 47.8 against 69.6.
 constexpr int kClusterNodes = 480;
+constexpr int kBandClusterItems = 256;
+void band_cluster_config(const dmrt_ctx* c, cudaLaunchConfig_t* cfg, cudaLaunchAttribute* attr) {
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = c->bblocks;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg->gridDim = dim3(c->bblocks);
+    cfg->blockDim = dim3(c->bthreads);
+    cfg->dynamicSmemBytes = c->bsmem;
+    cfg->stream = c->stream;
+    cfg->attrs = attr;
+    cfg->numAttrs = 1;
+}
 int setup_band(dmrt_ctx* c) {
     const dmrt_params& p = c->p;
     c->band = nullptr;
+    c->band_cluster = false;
     if (c->slab || c->L.off_mail == 0) return DMRT_OK;
+    auto threads = [&](int rows) {
+        const int items = rows * (((p.nx + 1) / 2 + 31) / 32 * 32), passes = (items + dmrt::kBandThreads - 1) / dmrt::kBandThreads;
+        return ((items + passes - 1) / passes + 31) / 32 * 32;
+    };
+    const int crows = (p.ny + dmrt::kBandCluster - 1) / dmrt::kBandCluster;
+    const int citems = crows * (((p.nx + 1) / 2 + 31) / 32 * 32);
+    if (c->cluster && citems <= 64) return DMRT_OK;
+    if (citems <= kBandClusterItems && dmrt::band_cluster_smem(crows, p.nx) <= (size_t)dmrt::kMaxSmem) {
+        const void* fn = dmrt::band_cluster_kernel(p.storage, p.rounding);
+        c->brows = crows;
+        c->bblocks = (p.ny + crows - 1) / crows;
+        c->bthreads = threads(crows);
+        c->bsmem = dmrt::band_cluster_smem(crows, p.nx);
+        cudaLaunchConfig_t cfg = {};
+        cudaLaunchAttribute attr[1];
+        band_cluster_config(c, &cfg, attr);
+        int nclusters = 0;
+        if (cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
+            cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, dmrt::kMaxSmem) == cudaSuccess &&
+            cudaOccupancyMaxActiveClusters(&nclusters, fn, &cfg) == cudaSuccess && nclusters >= 1) {
+            c->pc = dmrt::make_pair_consts(c->sc);
+            c->band = fn;
+            c->band_cluster = true;
+            return DMRT_OK;
+        }
+        (void)cudaGetLastError();
+    }
     if (c->cluster && (long long)c->crows * p.nx <= kClusterNodes) return DMRT_OK;
-    const void* fn = dmrt::band_kernel(p.storage, p.rounding);
     int dev = 0, sms = 0, per_sm = 0, coop = 0;
     CK(cudaGetDevice(&dev), "cudaGetDevice");
     CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev), "SM count");
     CK(cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev), "cooperative launch");
     c->brows = band_rows(p);
     c->bblocks = (p.ny + c->brows - 1) / c->brows;
-    const int pairs = c->brows * (((p.nx + 1) / 2 + 31) / 32 * 32), passes = (pairs + dmrt::kBandThreads - 1) / dmrt::kBandThreads;
-    c->bthreads = ((pairs + passes - 1) / passes + 31) / 32 * 32;
+    c->bthreads = threads(c->brows);
     c->bsmem = dmrt::band_smem(c->brows, p.nx);
+    const void* fn = dmrt::band_kernel(p.storage, p.rounding, c->brows * (((p.nx + 1) / 2 + 31) / 32 * 32) <= c->bthreads);
     // (the limit is the kernel's, for every context: the most a block may have)
     CK(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, dmrt::kMaxSmem), "set band shared memory");
     CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, c->bthreads, c->bsmem), "occupancy");
@@ -1619,8 +1663,15 @@ static int launch_band(dmrt_ctx* c, int n, float* record = nullptr, long long st
     B.states = record;
     B.stride = stride;
     void* params[2] = {&B, &c->pc};
-    CK(cudaLaunchCooperativeKernel(c->band, dim3(c->bblocks), dim3(c->bthreads), params, c->bsmem, c->stream),
-       "band launch");
+    if (c->band_cluster) {
+        cudaLaunchConfig_t cfg = {};
+        cudaLaunchAttribute attr[1];
+        band_cluster_config(c, &cfg, attr);
+        CK(cudaLaunchKernelExC(&cfg, c->band, params), "band launch");
+    } else {
+        CK(cudaLaunchCooperativeKernel(c->band, dim3(c->bblocks), dim3(c->bthreads), params, c->bsmem, c->stream),
+           "band launch");
+    }
     dmrt::band_nu_kernel<<<(n + dmrt::kBandNuWarps - 1) / dmrt::kBandNuWarps, 32 * dmrt::kBandNuWarps, 0, c->stream>>>(B);
     CK(cudaGetLastError(), "band Nusselt launch");
     c->cur = end;

@@ -29,13 +29,16 @@
 // to the global buffer. The temperatures at x = 0, 1 of every row and step go to
 // a record that the launch's last kernel turns into Nusselt numbers.
 //
-// What bounds it: up to 192^2 the exchange, above it the blocks' float32 pipes
-// as well (512^2: 1.2 us of its 3.5 us per step). Measured at the rule in
+// What bounds it: up to 192^2 the exchange and the serial chain of a pair's
+// collision, above it the blocks' float32 pipes as well (512^2: 1.2 us of its
+// 3.5 us per step). Measured at the rule in
 // dmrt.cu (setup_band).
 //
 // Every poll is bounded: on expiry the block records kErrTimeout and returns,
 // and its neighbours' polls expire in turn.
 #pragma once
+#include <cooperative_groups.h>
+
 #include "step_march.cuh"
 
 namespace dmrt {
@@ -74,6 +77,12 @@ __device__ __forceinline__ void band_item(const BandArgs& B, int i, int nr, int&
 // Shared-memory row stride in floats: the row's pairs with two columns on each side.
 __host__ __device__ constexpr int band_stride(int nx) { return (nx + 1) / 2 * 2 + 4; }
 __host__ __device__ constexpr size_t band_smem(int rows, int nx) { return (size_t)2 * 14 * rows * band_stride(nx) * 4; }
+
+// In one cluster: with the message slots and their barriers.
+constexpr int kBandCluster = 16;
+__host__ __device__ constexpr size_t band_cluster_smem(int rows, int nx) {
+    return band_smem(rows, nx) + (size_t)16 * band_stride(nx) * 4 + 4 * 8;
+}
 
 __device__ __forceinline__ void mail_put(ulonglong2* p, F2 v, unsigned tag) {
     const unsigned long long t = (unsigned long long)tag << 32;
@@ -126,7 +135,43 @@ __device__ __forceinline__ bool mail_read(const unsigned long long* box, int wor
     }
 }
 
-template <typename L, bool SR>
+// One cluster of up to 16 blocks (small cavities): the same steps, the messages
+// going straight into the neighbour's shared memory (st.async, which counts its
+// bytes on an mbarrier there) instead of through L2: a message then takes about a
+// quarter of a microsecond. A barrier per slot and side is armed with the
+// message's bytes one step ahead; a thread that needs the message waits for it.
+__device__ __forceinline__ unsigned cluster_addr(const void* p, unsigned rank) {
+    unsigned a;
+    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(smem_u32(p)), "r"(rank));
+    return a;
+}
+__device__ __forceinline__ void cluster_put(unsigned addr, F2 v, unsigned bar) {
+    asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.b64 [%0], %1, [%2];" ::"r"(addr), "l"(v), "r"(bar)
+                 : "memory");
+}
+__device__ __forceinline__ bool cluster_wait(uint64_t* bar, unsigned parity) {
+    unsigned long long t0 = 0;
+    for (;;) {
+        unsigned ok;
+        asm volatile(
+            "{\n\t.reg .pred p;\n\t"
+            "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
+            "selp.u32 %0, 1, 0, p;\n\t}"
+            : "=r"(ok)
+            : "r"(smem_u32(bar)), "r"(parity)
+            : "memory");
+        if (ok) return true;
+        const unsigned long long now = global_ns();
+        if (t0 == 0) t0 = now;
+        else if (now - t0 > kWaitLimitNs) return false;
+    }
+}
+
+// CL: one cluster, messages through shared memory; else a cooperative launch of
+// blocks, messages through L2.
+// ONE: a thread has at most one pair (its place, walls and addresses then are
+// fixed before the steps); else it loops over its pairs in every step.
+template <typename L, bool SR, bool CL, bool ONE>
 __global__ void __launch_bounds__(kBandThreads) step_band_kernel(const __grid_constant__ BandArgs B,
                                                                  const __grid_constant__ PairConsts K) {
     using Ef = typename L::Ef;
@@ -140,7 +185,21 @@ __global__ void __launch_bounds__(kBandThreads) step_band_kernel(const __grid_co
     const int plane = h * WS;  // floats per plane
     const int buffer = 14 * plane;
     const int items = nr * B.row_threads;
-    if (*reinterpret_cast<volatile unsigned*>(A.err) & kErrTimeout) return;  // (the same word for every block)
+    // Messages in shared memory (CL): [2 slots][2 sides][4 planes][WS], then a barrier per slot and side.
+    float* const inbox = smem_b + 2 * buffer;
+    uint64_t* const bars = reinterpret_cast<uint64_t*>(inbox + 16 * WS);
+    const unsigned message = 4u * 8u * (unsigned)B.pairs;
+    if constexpr (CL) {
+        if (threadIdx.x == 0) {
+            for (int b = 0; b < 4; ++b) mbar_init(&bars[b], 1);
+            mbar_fence_init();
+            if (blk > 0) mbar_expect_tx(&bars[2], message);  // the messages the first step reads (slot 1)
+            if (blk + 1 < nblk) mbar_expect_tx(&bars[3], message);
+        }
+        cooperative_groups::this_cluster().sync();
+    } else if (*reinterpret_cast<volatile unsigned*>(A.err) & kErrTimeout) {
+        return;  // an earlier launch's wait expired
+    }
     const unsigned tag0 = *B.epoch + 1u;
     const unsigned t_in = (unsigned)*A.step_in;
     if (blk == 0 && threadIdx.x == 0) *B.t_base = *A.step_in;
@@ -150,6 +209,26 @@ __global__ void __launch_bounds__(kBandThreads) step_band_kernel(const __grid_co
     auto box = [&](int slot, int b, int side) { return mail + slot * slot_words + ((size_t)(b * 2 + side) * 4) * B.words + 2; };
     // A pair's messages after a step (post-collision populations f, g of row r).
     auto send = [&](int s, int r, int x0, const F2 (&f)[9], const F2 (&g)[5], unsigned tag) {
+        if constexpr (CL) {
+            const int slot = s & 1;
+            if (r == 0 && blk > 0) {
+                const unsigned d = cluster_addr(inbox + (slot * 2 + 1) * 4 * WS + 2 + x0, blk - 1);
+                const unsigned b = cluster_addr(&bars[slot * 2 + 1], blk - 1);
+                cluster_put(d, f[4], b);
+                cluster_put(d + 4 * WS, f[7], b);
+                cluster_put(d + 8 * WS, f[8], b);
+                cluster_put(d + 12 * WS, g[4], b);
+            }
+            if (r == nr - 1 && blk + 1 < nblk) {
+                const unsigned d = cluster_addr(inbox + (slot * 2) * 4 * WS + 2 + x0, blk + 1);
+                const unsigned b = cluster_addr(&bars[slot * 2], blk + 1);
+                cluster_put(d, f[2], b);
+                cluster_put(d + 4 * WS, f[5], b);
+                cluster_put(d + 8 * WS, f[6], b);
+                cluster_put(d + 12 * WS, g[2], b);
+            }
+            return;
+        }
         if (r == 0 && blk > 0) {  // downward, into the previous block's box from above
             ulonglong2* p = reinterpret_cast<ulonglong2*>(box(s & 1, blk - 1, 1) + x0);
             const int w = B.words / 2;
@@ -203,167 +282,206 @@ __global__ void __launch_bounds__(kBandThreads) step_band_kernel(const __grid_co
     }
     float peak0 = 0.f, peak1 = 0.f;
     bool dead = false;
+    auto lane_of = [&](int x0) {
+        MarchLane n;
+        n.x0 = x0;
+        n.two = x0 + 1 < nx;
+        n.left = x0 == 0;
+        n.right = x0 + 2 >= nx;
+        n.rhi = x0 + 1 == nx - 1;
+        return n;
+    };
+    // The pair at row r, column x0 in step s, from buffer S to buffer D.
+    auto pair_step = [&](int s, const float* S, float* D, unsigned tag, unsigned salt, int r, int x0, const MarchLane& n) {
+        const int j = r0 + r;
+        if (!DMRT_IN(13 * plane + r * WS + 2 + x0 + 1, 0, buffer, A.err) || !DMRT_IN(j, 0, ny, A.err)) return;
+        const float* q = S + r * WS + 2 + x0;
+        auto at = [&](int k, int dr) { return *reinterpret_cast<const F2*>(q + k * plane + dr * WS); };
+        // The pulls shifted in x (directions 1, 5, 8, g 1 from the left, 3, 6, 7,
+        // g 3 from the right) stay single values until the side walls have
+        // replaced theirs: changing one half of a packed pair in a divergent
+        // branch here gave a wrong other half (nvcc 13.0).
+        auto px = [&](int k, int dr, float (&v)[2]) {
+            const float* p = q + k * plane + dr * WS;
+            v[0] = p[-1], v[1] = p[0];
+        };
+        auto mx = [&](int k, int dr, float (&v)[2]) {
+            const float* p = q + k * plane + dr * WS;
+            v[0] = p[1], v[1] = p[2];
+        };
+        auto un = [&](F2 a, float (&v)[2]) { v[0] = f2_lo(a), v[1] = f2_hi(a); };
+        F2 f[9], g[5];
+        float v1[2], v3[2], v5[2], v6[2], v7[2], v8[2], w1[2], w3[2];
+        f[0] = at(0, 0);
+        g[0] = at(9, 0);
+        px(1, 0, v1);
+        mx(3, 0, v3);
+        px(10, 0, w1);
+        mx(12, 0, w3);
+        if (r > 0) {
+            f[2] = at(2, -1);
+            px(5, -1, v5);
+            mx(6, -1, v6);
+            g[2] = at(11, -1);
+        } else if (j == 0) {  // bottom wall: the node's own opposites
+            f[2] = at(4, 0);
+            un(at(7, 0), v5);
+            un(at(8, 0), v6);
+            g[2] = at(13, 0);
+        } else if constexpr (CL) {
+            const int slot = (s & 1) ^ 1;
+            dead |= !cluster_wait(&bars[slot * 2], (unsigned)(s >> 1) & 1u);
+            const float* m = inbox + slot * 2 * 4 * WS + 2 + x0;
+            f[2] = *reinterpret_cast<const F2*>(m);
+            v5[0] = m[WS - 1], v5[1] = m[WS];
+            v6[0] = m[2 * WS + 1], v6[1] = m[2 * WS + 2];
+            g[2] = *reinterpret_cast<const F2*>(m + 3 * WS);
+        } else {
+            F2 v[4];
+            dead |= !mail_read<1>(box((s & 1) ^ 1, blk, 0), B.words, x0, n.left, n.right, tag, v);
+            f[2] = v[0], g[2] = v[3];
+            un(v[1], v5);
+            un(v[2], v6);
+        }
+        if (r + 1 < nr) {
+            f[4] = at(4, 1);
+            mx(7, 1, v7);
+            px(8, 1, v8);
+            g[4] = at(13, 1);
+        } else if (j == ny - 1) {
+            f[4] = at(2, 0);
+            un(at(5, 0), v7);
+            un(at(6, 0), v8);
+            g[4] = at(11, 0);
+        } else if constexpr (CL) {
+            const int slot = (s & 1) ^ 1;
+            dead |= !cluster_wait(&bars[slot * 2 + 1], (unsigned)(s >> 1) & 1u);
+            const float* m = inbox + (slot * 2 + 1) * 4 * WS + 2 + x0;
+            f[4] = *reinterpret_cast<const F2*>(m);
+            v7[0] = m[WS + 1], v7[1] = m[WS + 2];
+            v8[0] = m[2 * WS - 1], v8[1] = m[2 * WS];
+            g[4] = *reinterpret_cast<const F2*>(m + 3 * WS);
+        } else {
+            F2 v[4];
+            dead |= !mail_read<-1>(box((s & 1) ^ 1, blk, 1), B.words, x0, n.left, n.right, tag, v);
+            f[4] = v[0], g[4] = v[3];
+            un(v[1], v7);
+            un(v[2], v8);
+        }
+        // Side walls: links from outside x = 0 and x = nx - 1 from the node's own opposites.
+        auto own = [&](int k, int hi) { return q[k * plane + hi]; };
+        if (n.left) {
+            v1[0] = own(3, 0);
+            v5[0] = own(7, 0);
+            v8[0] = own(6, 0);
+            w1[0] = wall_value(M.sign_l, own(12, 0), __fmul_rn(M.abb_l, __ldg(A.hot + j)));
+        }
+        if (n.right) {
+            const int e = n.rhi ? 1 : 0;
+            const float wall = wall_value(M.sign_r, own(10, e), __fmul_rn(M.abb_r, __ldg(A.cold + j)));
+#pragma unroll
+            for (int i = 0; i < 2; ++i) {
+                if (i == e) v3[i] = own(1, e), v6[i] = own(8, e), v7[i] = own(5, e), w3[i] = wall;
+            }
+        }
+        f[1] = f2_pack(v1[0], v1[1]);
+        f[3] = f2_pack(v3[0], v3[1]);
+        f[5] = f2_pack(v5[0], v5[1]);
+        f[6] = f2_pack(v6[0], v6[1]);
+        f[7] = f2_pack(v7[0], v7[1]);
+        f[8] = f2_pack(v8[0], v8[1]);
+        g[1] = f2_pack(w1[0], w1[1]);
+        g[3] = f2_pack(w3[0], w3[1]);
+        F2 rho, theta;
+        collide_pair(f, g, K.r, K.n, rho, theta);
+        peak0 = peak_of(peak0, f2_lo(rho), f2_lo(theta));
+        if (n.two) peak1 = peak_of(peak1, f2_hi(rho), f2_hi(theta));
+        if (n.left) B.record[(size_t)s * ny + j] = theta;
+        if constexpr (!kShifted<Ef>) {
+            if (B.states) {
+                float* d = B.states + (size_t)s * B.stride + (size_t)j * A.pitch + x0;
+                if (n.two) {
+#pragma unroll
+                    for (int k = 0; k < 9; ++k) *reinterpret_cast<F2*>(d + plane_f(k) * A.plane) = f[k];
+#pragma unroll
+                    for (int k = 0; k < 5; ++k) *reinterpret_cast<F2*>(d + plane_g(k) * A.plane) = g[k];
+                } else {
+#pragma unroll
+                    for (int k = 0; k < 9; ++k) d[plane_f(k) * A.plane] = f2_lo(f[k]);
+#pragma unroll
+                    for (int k = 0; k < 5; ++k) d[plane_g(k) * A.plane] = f2_lo(g[k]);
+                }
+            }
+        }
+        const bool final_step = s == B.steps - 1;
+        if (kShifted<Ef> || final_step) {
+            unsigned h0 = 0, h1 = 0;
+            if constexpr (SR) pair_random(salt, j, n, A, h0, h1);
+            const PairStored<L> e = pair_encode<L, SR>(f, g, theta, M, h0, h1);
+            if (final_step) {
+                unsigned char* df = B.out;
+                unsigned char* dg = L::kSplit ? df + 9 * A.plane * (long long)sizeof(Ef) : df;
+                const long long o = (long long)j * A.pitch + x0;
+                if (!DMRT_IN(o + 1, 1, A.plane, A.err)) return;
+                auto put = [&](unsigned char* p, auto v) {
+                    using T = decltype(v);
+                    if (n.two) *reinterpret_cast<T*>(p) = v;
+                    else if constexpr (sizeof(T) == 8) *reinterpret_cast<unsigned*>(p) = (unsigned)v;
+                    else *reinterpret_cast<unsigned short*>(p) = (unsigned short)v;
+                };
+#pragma unroll
+                for (int k = 0; k < 9; ++k) put(df + (L::pf(k) * A.plane + o) * (long long)sizeof(Ef), e.f[k]);
+                if constexpr (L::kTheta) {
+                    put(dg + o * 4, e.theta);
+#pragma unroll
+                    for (int k = 1; k < 5; ++k) put(dg + A.plane * 4 + ((k - 1) * A.plane + o) * 2, e.g[k]);
+                } else {
+#pragma unroll
+                    for (int k = 0; k < 5; ++k) put(dg + (L::pg(k) * A.plane + o) * (long long)sizeof(Eg), e.g[k]);
+                }
+                return;
+            }
+            pair_decode<L>(e, M, f, g);
+        }
+        send(s, r, x0, f, g, tag + 1u);
+        float* d = D + r * WS + 2 + x0;
+#pragma unroll
+        for (int k = 0; k < 9; ++k) *reinterpret_cast<F2*>(d + k * plane) = f[k];
+#pragma unroll
+        for (int k = 0; k < 5; ++k) *reinterpret_cast<F2*>(d + (9 + k) * plane) = g[k];
+    };
+    int r1 = 0, x1 = 0;
+    band_item(B, min((int)threadIdx.x, items - 1), nr, r1, x1);
+    const bool has1 = (int)threadIdx.x < items && x1 < nx;
+    const MarchLane n1 = lane_of(x1);
     __syncthreads();
 #pragma unroll 1
     for (int s = 0; s < B.steps; ++s) {
         const float* S = smem_b + (s & 1) * buffer;
         float* D = smem_b + ((s & 1) ^ 1) * buffer;
         const unsigned tag = tag0 + (unsigned)s;  // of the messages this step reads
+        if constexpr (CL) {
+            // This step's messages come into slot s & 1, whose last ones were read in
+            // the step before.
+            if (threadIdx.x == 0 && s + 1 < B.steps) {
+                if (blk > 0) mbar_expect_tx(&bars[(s & 1) * 2], message);
+                if (blk + 1 < nblk) mbar_expect_tx(&bars[(s & 1) * 2 + 1], message);
+            }
+        }
         const unsigned salt = SR ? hash32((t_in + (unsigned)s) * 0x9e3779b9u + 0x632be5abu) : 0u;
+        if constexpr (ONE) {
+            if (has1) pair_step(s, S, D, tag, salt, r1, x1, n1);
+        } else {
 #pragma unroll 1
-        for (int i = threadIdx.x; i < items; i += blockDim.x) {
-            int r, x0;
-            band_item(B, i, nr, r, x0);
-            if (x0 >= nx) continue;
-            const int j = r0 + r;
-            if (!DMRT_IN(13 * plane + r * WS + 2 + x0 + 1, 0, buffer, A.err) || !DMRT_IN(j, 0, ny, A.err)) continue;
-            MarchLane n;
-            n.x0 = x0;
-            n.two = x0 + 1 < nx;
-            n.left = x0 == 0;
-            n.right = x0 + 2 >= nx;
-            n.rhi = x0 + 1 == nx - 1;
-            const float* q = S + r * WS + 2 + x0;
-            auto at = [&](int k, int dr) { return *reinterpret_cast<const F2*>(q + k * plane + dr * WS); };
-            // The pulls shifted in x (directions 1, 5, 8, g 1 from the left, 3, 6, 7,
-            // g 3 from the right) stay single values until the side walls have
-            // replaced theirs: changing one half of a packed pair in a divergent
-            // branch here gave a wrong other half (nvcc 13.0).
-            auto px = [&](int k, int dr, float (&v)[2]) {
-                const float* p = q + k * plane + dr * WS;
-                v[0] = p[-1], v[1] = p[0];
-            };
-            auto mx = [&](int k, int dr, float (&v)[2]) {
-                const float* p = q + k * plane + dr * WS;
-                v[0] = p[1], v[1] = p[2];
-            };
-            auto un = [&](F2 a, float (&v)[2]) { v[0] = f2_lo(a), v[1] = f2_hi(a); };
-            F2 f[9], g[5];
-            float v1[2], v3[2], v5[2], v6[2], v7[2], v8[2], w1[2], w3[2];
-            f[0] = at(0, 0);
-            g[0] = at(9, 0);
-            px(1, 0, v1);
-            mx(3, 0, v3);
-            px(10, 0, w1);
-            mx(12, 0, w3);
-            if (r > 0) {
-                f[2] = at(2, -1);
-                px(5, -1, v5);
-                mx(6, -1, v6);
-                g[2] = at(11, -1);
-            } else if (j == 0) {  // bottom wall: the node's own opposites
-                f[2] = at(4, 0);
-                un(at(7, 0), v5);
-                un(at(8, 0), v6);
-                g[2] = at(13, 0);
-            } else {
-                F2 v[4];
-                dead |= !mail_read<1>(box((s & 1) ^ 1, blk, 0), B.words, x0, n.left, n.right, tag, v);
-                f[2] = v[0], g[2] = v[3];
-                un(v[1], v5);
-                un(v[2], v6);
+            for (int i = threadIdx.x; i < items; i += blockDim.x) {
+                int r, x0;
+                band_item(B, i, nr, r, x0);
+                if (x0 < nx) pair_step(s, S, D, tag, salt, r, x0, lane_of(x0));
             }
-            if (r + 1 < nr) {
-                f[4] = at(4, 1);
-                mx(7, 1, v7);
-                px(8, 1, v8);
-                g[4] = at(13, 1);
-            } else if (j == ny - 1) {
-                f[4] = at(2, 0);
-                un(at(5, 0), v7);
-                un(at(6, 0), v8);
-                g[4] = at(11, 0);
-            } else {
-                F2 v[4];
-                dead |= !mail_read<-1>(box((s & 1) ^ 1, blk, 1), B.words, x0, n.left, n.right, tag, v);
-                f[4] = v[0], g[4] = v[3];
-                un(v[1], v7);
-                un(v[2], v8);
-            }
-            // Side walls: links from outside x = 0 and x = nx - 1 from the node's own opposites.
-            auto own = [&](int k, int hi) { return q[k * plane + hi]; };
-            if (n.left) {
-                v1[0] = own(3, 0);
-                v5[0] = own(7, 0);
-                v8[0] = own(6, 0);
-                w1[0] = wall_value(M.sign_l, own(12, 0), __fmul_rn(M.abb_l, __ldg(A.hot + j)));
-            }
-            if (n.right) {
-                const int e = n.rhi ? 1 : 0;
-                const float wall = wall_value(M.sign_r, own(10, e), __fmul_rn(M.abb_r, __ldg(A.cold + j)));
-#pragma unroll
-                for (int i = 0; i < 2; ++i) {
-                    if (i == e) v3[i] = own(1, e), v6[i] = own(8, e), v7[i] = own(5, e), w3[i] = wall;
-                }
-            }
-            f[1] = f2_pack(v1[0], v1[1]);
-            f[3] = f2_pack(v3[0], v3[1]);
-            f[5] = f2_pack(v5[0], v5[1]);
-            f[6] = f2_pack(v6[0], v6[1]);
-            f[7] = f2_pack(v7[0], v7[1]);
-            f[8] = f2_pack(v8[0], v8[1]);
-            g[1] = f2_pack(w1[0], w1[1]);
-            g[3] = f2_pack(w3[0], w3[1]);
-            F2 rho, theta;
-            collide_pair(f, g, K.r, K.n, rho, theta);
-            peak0 = peak_of(peak0, f2_lo(rho), f2_lo(theta));
-            if (n.two) peak1 = peak_of(peak1, f2_hi(rho), f2_hi(theta));
-            if (n.left) B.record[(size_t)s * ny + j] = theta;
-            if constexpr (!kShifted<Ef>) {
-                if (B.states) {
-                    float* d = B.states + (size_t)s * B.stride + (size_t)j * A.pitch + x0;
-                    if (n.two) {
-#pragma unroll
-                        for (int k = 0; k < 9; ++k) *reinterpret_cast<F2*>(d + plane_f(k) * A.plane) = f[k];
-#pragma unroll
-                        for (int k = 0; k < 5; ++k) *reinterpret_cast<F2*>(d + plane_g(k) * A.plane) = g[k];
-                    } else {
-#pragma unroll
-                        for (int k = 0; k < 9; ++k) d[plane_f(k) * A.plane] = f2_lo(f[k]);
-#pragma unroll
-                        for (int k = 0; k < 5; ++k) d[plane_g(k) * A.plane] = f2_lo(g[k]);
-                    }
-                }
-            }
-            const bool final_step = s == B.steps - 1;
-            if (kShifted<Ef> || final_step) {
-                unsigned h0 = 0, h1 = 0;
-                if constexpr (SR) pair_random(salt, j, n, A, h0, h1);
-                const PairStored<L> e = pair_encode<L, SR>(f, g, theta, M, h0, h1);
-                if (final_step) {
-                    unsigned char* df = B.out;
-                    unsigned char* dg = L::kSplit ? df + 9 * A.plane * (long long)sizeof(Ef) : df;
-                    const long long o = (long long)j * A.pitch + x0;
-                    if (!DMRT_IN(o + 1, 1, A.plane, A.err)) continue;
-                    auto put = [&](unsigned char* p, auto v) {
-                        using T = decltype(v);
-                        if (n.two) *reinterpret_cast<T*>(p) = v;
-                        else if constexpr (sizeof(T) == 8) *reinterpret_cast<unsigned*>(p) = (unsigned)v;
-                        else *reinterpret_cast<unsigned short*>(p) = (unsigned short)v;
-                    };
-#pragma unroll
-                    for (int k = 0; k < 9; ++k) put(df + (L::pf(k) * A.plane + o) * (long long)sizeof(Ef), e.f[k]);
-                    if constexpr (L::kTheta) {
-                        put(dg + o * 4, e.theta);
-#pragma unroll
-                        for (int k = 1; k < 5; ++k) put(dg + A.plane * 4 + ((k - 1) * A.plane + o) * 2, e.g[k]);
-                    } else {
-#pragma unroll
-                        for (int k = 0; k < 5; ++k) put(dg + (L::pg(k) * A.plane + o) * (long long)sizeof(Eg), e.g[k]);
-                    }
-                    continue;
-                }
-                pair_decode<L>(e, M, f, g);
-            }
-            send(s, r, x0, f, g, tag + 1u);
-            float* d = D + r * WS + 2 + x0;
-#pragma unroll
-            for (int k = 0; k < 9; ++k) *reinterpret_cast<F2*>(d + k * plane) = f[k];
-#pragma unroll
-            for (int k = 0; k < 5; ++k) *reinterpret_cast<F2*>(d + (9 + k) * plane) = g[k];
         }
         if (__syncthreads_or(dead)) break;
     }
+    if constexpr (CL) cooperative_groups::this_cluster().sync();  // no message still on its way to a block that is gone
     if (dead) atomicOr(A.err, kErrTimeout);
     if (!(peak0 < 1e30f) || !(peak1 < 1e30f)) atomicOr(A.err, kErrNonFinite);
 }
@@ -421,7 +539,9 @@ static __global__ void __launch_bounds__(32 * kBandNuWarps) band_nu_kernel(const
     }
 }
 
-// The compiled band kernel of a storage and rounding.
-const void* band_kernel(int storage, int rounding);
+// The compiled band kernel of a storage and rounding, across the GPU or in one cluster.
+// (one: blocks with at most one pair per thread; a cluster's are)
+const void* band_kernel(int storage, int rounding, bool one);
+const void* band_cluster_kernel(int storage, int rounding);
 
 }  // namespace dmrt

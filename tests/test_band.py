@@ -1,5 +1,5 @@
 """The band kernel (many steps per launch, the cavity on chip across the GPU, AUTO's
-choice for runs of steps of cavities up to about 512^2) against the one-step TMA
+choice for runs of steps of cavities up to about 512^2; small ones in one cluster) against the one-step TMA
 kernel: the same bits in every storage mode and rounding, for odd sizes, one and
 several rows and passes per block, and every way a run is split into launches."""
 import os
@@ -19,7 +19,8 @@ MODES = [(0, 0), (1, 0), (1, 1), (2, 0), (2, 1), (3, 0), (3, 1), (4, 0), (4, 1)]
 # The last columns: a whole warp of pairs per row, one pair more; rows that fill the
 # last block and that leave it one row; 16-bit storage of small cavities; rows wider
 # than half a block; several passes per thread.
-SIZES = [(128, 128), (130, 127), (193, 305), (64, 97), (33, 304), (640, 151), (512, 512), (8, 600)]
+SIZES = [(128, 128), (130, 127), (193, 305), (64, 97), (33, 304), (640, 151), (512, 512), (8, 600),
+         (64, 64), (100, 60), (127, 33), (66, 17), (8, 250)]
 
 
 def advance(nx, ny, storage, rounding, kernel, walls=(0, 0), cap=4096, runs=RUNS):
@@ -129,6 +130,6 @@ def test_band_captured_and_replayed():
 
 def test_band_bounds_checked_build():
     code = ("import sys; sys.path.insert(0, %r); from tests.test_band import advance;"
-            "[advance(nx, ny, s, 2, 0) for nx, ny in ((130, 127), (193, 305), (640, 151)) for s in range(5)]" % ROOT)
+            "[advance(nx, ny, s, 2, 0) for nx, ny in ((130, 127), (193, 305), (640, 151), (100, 60)) for s in range(5)]" % ROOT)
     subprocess.run([sys.executable, "-c", code], check=True, cwd=ROOT,
                    env=dict(os.environ, DMRT_LIBRARY="bounds_check"))
