@@ -4,16 +4,18 @@
 
 namespace dmrt {
 
-const void* band_one_kernel(int storage, int rounding);  // band_one.cu
+const void* band_one_kernel(int storage, int rounding);   // band_one.cu
+const void* band_wide_kernel(int storage, int rounding);  // band_wide.cu
 
 template <typename L, bool SR>
 static const void* form() {
-    return (const void*)step_band_kernel<L, SR, false, false>;
+    return (const void*)step_band_kernel<L, SR, false, false, kBandThreads>;
 }
 
-const void* band_kernel(int storage, int rounding, bool one) {
+const void* band_kernel(int storage, int rounding, int items) {
     using Mixed = Split<__half, float>;
-    if (one) return band_one_kernel(storage, rounding);
+    if (items <= kBandThreads) return band_one_kernel(storage, rounding);
+    if (items <= kBandWide) return band_wide_kernel(storage, rounding);
     const bool sr = rounding == DMRT_ROUND_STOCHASTIC;
     switch (storage) {
         case DMRT_FP32: return form<OneType<float>, false>();

@@ -6,7 +6,7 @@ namespace dmrt {
 
 template <typename L, bool SR>
 static const void* form() {
-    return (const void*)step_band_kernel<L, SR, true, true>;
+    return (const void*)step_band_kernel<L, SR, true, true, kBandThreads>;
 }
 
 const void* band_cluster_kernel(int storage, int rounding) {

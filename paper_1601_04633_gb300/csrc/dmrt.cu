@@ -1016,7 +1016,7 @@ int setup_march(dmrt_ctx* c) {
 // or three steps per launch: float32 16^2 1.10 / 1.26 / 0.97 / 2.7, 32^2 0.98 / 1.25 /
 // 0.96, 64^2 0.92 / 1.24 / 1.12, 100 x 60 1.11 / 1.25 / 1.19, 80^2 1.27 / 1.25 / 1.25,
 // 96^2 1.35 / 1.25 / 1.39, 128^2 1.63 / 1.24 / 2.52 / 2.7, 192^2 - / 1.33 / - / 2.97,
-// 256^2 - / 1.44 / - / 3.39, 383 x 389 - / 2.67 / - / 4.26, 512^2 - / 3.49 / - / 5.51;
+// 256^2 - / 1.44 / - / 3.39, 383 x 389 - / 2.09 / - / 4.26, 512^2 - / 3.49 / - / 5.51;
 // mixed, stochastic 64^2 0.95 / 1.28 / - / 3.26, 96^2 1.46 / 1.29, 256^2 - / 1.58 / - /
 // 3.75, 512^2 - / 3.87 / - / 6.63; 100 x 500 float32 - / 1.41 / - / 3.90. A call of 8
 // steps: 128^2 20.8 us against 32.0, 512^2 47.8 against 69.6.
@@ -1040,7 +1040,9 @@ int setup_band(dmrt_ctx* c) {
     c->band_cluster = false;
     if (c->slab || c->L.off_mail == 0) return DMRT_OK;
     auto threads = [&](int rows) {
-        const int items = rows * (((p.nx + 1) / 2 + 31) / 32 * 32), passes = (items + dmrt::kBandThreads - 1) / dmrt::kBandThreads;
+        const int items = rows * (((p.nx + 1) / 2 + 31) / 32 * 32);
+        if (items <= dmrt::kBandWide) return items;
+        const int passes = (items + dmrt::kBandThreads - 1) / dmrt::kBandThreads;
         return ((items + passes - 1) / passes + 31) / 32 * 32;
     };
     const int crows = (p.ny + dmrt::kBandCluster - 1) / dmrt::kBandCluster;
@@ -1075,7 +1077,7 @@ int setup_band(dmrt_ctx* c) {
     c->bblocks = (p.ny + c->brows - 1) / c->brows;
     c->bthreads = threads(c->brows);
     c->bsmem = dmrt::band_smem(c->brows, p.nx);
-    const void* fn = dmrt::band_kernel(p.storage, p.rounding, c->brows * (((p.nx + 1) / 2 + 31) / 32 * 32) <= c->bthreads);
+    const void* fn = dmrt::band_kernel(p.storage, p.rounding, c->brows * (((p.nx + 1) / 2 + 31) / 32 * 32));
     // (the limit is the kernel's, for every context: the most a block may have)
     CK(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, dmrt::kMaxSmem), "set band shared memory");
     CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, c->bthreads, c->bsmem), "occupancy");
@@ -1637,6 +1639,8 @@ static int launch_cluster(dmrt_ctx* c, int n, float* record = nullptr, long long
 }
 
 // n steps (at most kBandSteps) in one band launch, their Nusselt numbers included.
+// kNoBand: the GPU no longer holds every block at once, nothing was launched.
+constexpr int kNoBand = 1;
 static int launch_band(dmrt_ctx* c, int n, float* record = nullptr, long long stride = 0) {
     if (c->nu_open) {
         int rc = finalize_nu(c);
@@ -1669,8 +1673,9 @@ static int launch_band(dmrt_ctx* c, int n, float* record = nullptr, long long st
         band_cluster_config(c, &cfg, attr);
         CK(cudaLaunchKernelExC(&cfg, c->band, params), "band launch");
     } else {
-        CK(cudaLaunchCooperativeKernel(c->band, dim3(c->bblocks), dim3(c->bthreads), params, c->bsmem, c->stream),
-           "band launch");
+        const cudaError_t e = cudaLaunchCooperativeKernel(c->band, dim3(c->bblocks), dim3(c->bthreads), params, c->bsmem, c->stream);
+        if (e == cudaErrorCooperativeLaunchTooLarge) return kNoBand;  // (fewer SMs than at creation)
+        CK(e, "band launch");
     }
     dmrt::band_nu_kernel<<<(n + dmrt::kBandNuWarps - 1) / dmrt::kBandNuWarps, 32 * dmrt::kBandNuWarps, 0, c->stream>>>(B);
     CK(cudaGetLastError(), "band Nusselt launch");
@@ -1729,6 +1734,11 @@ static int step_run(dmrt_ctx* c, int64_t nsteps, bool finalize, float* record = 
             const long long rest = nsteps - n;
             if (rest > 0 && rest < dmrt::kBandMinSteps) n = nsteps <= dmrt::kBandSteps ? nsteps : n - dmrt::kBandMinSteps;
             int rc = launch_band(c, (int)n, record, stride);
+            if (rc == kNoBand) {
+                (void)cudaGetLastError();
+                c->band = nullptr;  // the other kernels take the rest, and later runs
+                return step_run(c, nsteps, finalize, record, stride);
+            }
             if (rc) return rc;
             if (record) record += n * stride;
             nsteps -= n;

@@ -43,7 +43,8 @@
 
 namespace dmrt {
 
-constexpr int kBandThreads = 512;  // most threads of a block
+constexpr int kBandThreads = 512;  // most threads of a block (128 registers each)
+constexpr int kBandWide = 576;     // ... of the form for 513 to 576 pairs (96 registers each)
 constexpr int kBandSteps = 512;    // most steps per launch (the Nusselt record's length)
 constexpr int kBandMinSteps = 6;   // shorter runs take the other kernels
 
@@ -171,8 +172,11 @@ __device__ __forceinline__ bool cluster_wait(uint64_t* bar, unsigned parity) {
 // blocks, messages through L2.
 // ONE: a thread has at most one pair (its place, walls and addresses then are
 // fixed before the steps); else it loops over its pairs in every step.
-template <typename L, bool SR, bool CL, bool ONE>
-__global__ void __launch_bounds__(kBandThreads) step_band_kernel(const __grid_constant__ BandArgs B,
+// MAXT: the most threads: a block of 513 to 576 pairs takes them in one pass with
+// fewer registers (383 x 389: 2.67 -> 2.09 us per step; blocks of two passes lose
+// 5 % with so few: 512^2 3.49 -> 3.68).
+template <typename L, bool SR, bool CL, bool ONE, int MAXT>
+__global__ void __launch_bounds__(MAXT) step_band_kernel(const __grid_constant__ BandArgs B,
                                                                  const __grid_constant__ PairConsts K) {
     using Ef = typename L::Ef;
     using Eg = typename L::Eg;
@@ -540,8 +544,8 @@ static __global__ void __launch_bounds__(32 * kBandNuWarps) band_nu_kernel(const
 }
 
 // The compiled band kernel of a storage and rounding, across the GPU or in one cluster.
-// (one: blocks with at most one pair per thread; a cluster's are)
-const void* band_kernel(int storage, int rounding, bool one);
+// (items: pairs of a block; a cluster's blocks have at most one per thread)
+const void* band_kernel(int storage, int rounding, int items);
 const void* band_cluster_kernel(int storage, int rounding);
 
 }  // namespace dmrt

@@ -19,7 +19,7 @@ MODES = [(0, 0), (1, 0), (1, 1), (2, 0), (2, 1), (3, 0), (3, 1), (4, 0), (4, 1)]
 # The last columns: a whole warp of pairs per row, one pair more; rows that fill the
 # last block and that leave it one row; 16-bit storage of small cavities; rows wider
 # than half a block; several passes per thread.
-SIZES = [(128, 128), (130, 127), (193, 305), (64, 97), (33, 304), (640, 151), (512, 512), (8, 600),
+SIZES = [(128, 128), (130, 127), (193, 305), (64, 97), (33, 304), (640, 151), (512, 512), (380, 307), (8, 600),
          (64, 64), (100, 60), (127, 33), (66, 17), (8, 250)]
 
 
