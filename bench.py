@@ -40,9 +40,8 @@ STORAGES = {"fp32": (0, 0), "fp16": (1, 0), "bf16": (2, 0), "fp16_sr": (1, 1), "
             "mixed": (3, 0), "mixed_sr": (3, 1), "theta32": (4, 0), "theta32_sr": (4, 1)}
 BYTES_PER_NODE = {"fp32": 112, "fp16": 56, "bf16": 56, "fp16_sr": 56, "bf16_sr": 56, "mixed": 76,
                   "mixed_sr": 76, "theta32": 60, "theta32_sr": 60}
-# Tiles (nodes per thread, rows, stages) of the secondary storage runs.
-SECONDARY_TILES = {"fp16": (2, 4, 2), "bf16": (2, 4, 2), "fp16_sr": (4, 4, 2), "bf16_sr": (4, 4, 2),
-                   "mixed": (2, 1, 2), "mixed_sr": (2, 1, 2), "theta32": (2, 1, 2), "theta32_sr": (4, 2, 2)}
+# Storage modes of the secondary runs, each with the kernel AUTO picks.
+SECONDARY_STORAGES = ("fp16", "bf16", "fp16_sr", "bf16_sr", "mixed", "mixed_sr", "theta32", "theta32_sr")
 FALLBACK_HBM_GBS = 6800.0
 GATE_STEPS = 20000  # the stated length of the 4096^2 workload; the Nu gate is taken over it
 NU_GATE = 1e-3
@@ -50,7 +49,26 @@ BATCH_MIN_STEPS = 2000  # batched sweeps are timed over at least this many steps
 SLAB_STEPS = 200  # timed steps of the single cavity split over the ranks (N > 1)
 PROFILE_SUMMARY = os.path.join(ROOT, "profiles", "step_kernel_4096x4096.json")
 KERNEL_SOURCES = [os.path.join(ROOT, "paper_1601_04633_gb300", "csrc", f)
-                  for f in ("lattice.cuh", "step_tma.cuh", "step_direct.cuh")]
+                  for f in ("lattice.cuh", "collide_pair.cuh", "step_tma.cuh", "step_march.cuh", "step_direct.cuh")]
+
+
+def steps_per_pass(args, cav):
+    """Steps that one pass over the state takes: three by the march kernel, which AUTO
+    runs for the large cavities (no kernel or tile asked for), else one."""
+    auto = args.kernel == 0 and args.tma_npt <= 0 and args.tma_rows <= 0 and args.tma_stages <= 0
+    return 3 if auto and cav.nx >= 1024 and cav.ny >= 1024 else 1
+
+
+def launches_of(steps, per_pass):
+    """Kernel launches of one run of `steps` steps, Nusselt sums included."""
+    if per_pass == 1 or steps < 3:
+        return steps + 1
+    rest = steps % 3
+    if rest == 0:
+        return steps // 3 + 1
+    if rest == 1:  # the last four steps in two launches
+        return (steps - 4) // 3 + 2 + 1
+    return (steps - 5) // 3 + 2 + 1 + 2  # the last five in two launches, their sums, and a single step
 
 
 def workload(name):
@@ -305,6 +323,7 @@ def run_dmrt(args):
               tma_npt=args.tma_npt, storage=STORAGES[args.storage][0], rounding=STORAGES[args.storage][1])
     sim = D.Cavity2D.from_inputs(cav, nu_capacity=max(args.steps + args.warmup, 1), **kw)
     launch = dict(sim.launch)
+    per_pass = steps_per_pass(args, cav)
     sim.step(args.warmup)
     sim.check()
     torch.cuda.synchronize()
@@ -357,14 +376,13 @@ def run_dmrt(args):
         ms_ref, nu_ref, _ = timed_run(**kw)
         secondary["fp32_gate_reference"] = {"value": nodes * gate_steps / (ms_ref / 1e3) / 1e6, "unit": UNIT,
                                             "steps": gate_steps, "nu_mean_last": float(nu_ref[-1])}
-        for st, (npt, rows, stages) in SECONDARY_TILES.items():
-            ms2, nu2, launch2 = timed_run(storage=STORAGES[st][0], rounding=STORAGES[st][1], kernel=2,
-                                          tma_npt=npt, tma_rows=rows, tma_stages=stages)
+        for st in SECONDARY_STORAGES:
+            ms2, nu2, launch2 = timed_run(storage=STORAGES[st][0], rounding=STORAGES[st][1])
             err = nu_rel_dev(nu2, nu_ref)
             v2 = nodes * gate_steps / (ms2 / 1e3) / 1e6
             secondary[st] = {"value": v2, "unit": UNIT, "steps": gate_steps,
-                             "bytes_per_node": BYTES_PER_NODE[st], "launch": launch2,
-                             "roofline_frac": BYTES_PER_NODE[st] * v2 * 1e6 / 1e9 / hbm_peak()[0],
+                             "bytes_per_node": BYTES_PER_NODE[st] / per_pass, "launch": launch2,
+                             "roofline_frac": BYTES_PER_NODE[st] / per_pass * v2 * 1e6 / 1e9 / hbm_peak()[0],
                              "nu_mean_last": float(nu2[-1]),
                              "nu_max_rel_dev_vs_fp32": err, "nu_gate_ok": bool(err <= NU_GATE),
                              "vs_fp32_single": v2 / secondary["fp32_gate_reference"]["value"]}
@@ -442,8 +460,8 @@ def run_dmrt(args):
                                        ("batched_mixed_sr", 3, 1, 76)):
             tuned = tune.tune_batch(sweep, steps=200, warmup=10, storage=storage, rounding=rnd,
                                     group_bytes=tune.GROUP_BYTES, steps_per_launch=tune.STEPS_PER_LAUNCH)
-            one = [t for t in tuned["trials"]
-                   if t["opts"].get("group_bytes", 0) == 0 and t["opts"].get("steps_per_launch", 1) <= 1]
+            one = [t for t in tuned["trials"] if t["opts"]["tma_npt"] > 0
+                   and t["opts"].get("group_bytes", 0) == 0 and t["opts"].get("steps_per_launch", 1) <= 1]
             best_one = max(one, key=lambda t: t["mlups"])["opts"]
             ms_st, nu_st, _ = run_batch(best_one, storage, rnd)
             v1 = bnodes * bsteps / (ms_st / 1e3) / 1e6
@@ -454,14 +472,18 @@ def run_dmrt(args):
             if tuned["opts"] != best_one:
                 ms_b2, nu_b2, ngroups = run_batch(tuned["opts"], storage, rnd)
                 v2 = bnodes * bsteps / (ms_b2 / 1e3) / 1e6
+                bpn2 = bpn / (1 if tuned["opts"]["tma_npt"] > 0 else 3)  # no tile: three steps per pass
                 entry["tuned_schedule"] = {"value": v2, "unit": UNIT, "tile": tuned["opts"], "groups": ngroups,
-                                           "roofline_frac": bpn * v2 * 1e6 / 1e9 / peak_hbm,
+                                           "bytes_per_node": bpn2,
+                                           "roofline_frac": bpn2 * v2 * 1e6 / 1e9 / peak_hbm,
                                            "nu_max_rel_diff_vs_one_launch_per_step": max_dev(nu_b2, nu_st)}
                 if v2 > best_value:
                     best_value, nu_best, entry["tile"] = v2, nu_b2, tuned["opts"]
             entry["value"] = best_value
             entry["unit"] = UNIT
-            entry["roofline_frac"] = bpn * best_value * 1e6 / 1e9 / peak_hbm
+            if entry["tile"]["tma_npt"] <= 0:
+                entry["bytes_per_node"] = bpn / 3
+            entry["roofline_frac"] = entry["bytes_per_node"] * best_value * 1e6 / 1e9 / peak_hbm
             entry["tuner_trials"] = [{"tile": t["opts"], "mlups": round(t["mlups"])} for t in tuned["trials"]]
             if storage == 0:
                 nu_fp32 = nu_best
@@ -557,7 +579,7 @@ def run_dmrt(args):
     steps = max(args.steps, 1)
     value = ws * nodes * args.steps / (ms / 1e3) / 1e6
     per_launch_s = ms / 1e3 / steps
-    bpn = BYTES_PER_NODE[args.storage]
+    bpn = BYTES_PER_NODE[args.storage] / per_pass  # one pass over the state takes per_pass steps
     achieved = bpn * nodes / per_launch_s / 1e9
     peak, peak_src = hbm_peak()
     traffic = ncu_traffic_per_launch(nodes) if args.storage == "fp32" else None
@@ -570,16 +592,19 @@ def run_dmrt(args):
                    "alpha": cav.alpha, "storage": args.storage, "parallelism": f"{ws} independent cavities",
                    "launch": launch,
                    "l2": "state (two 14-plane fp32 buffers) larger than L2: no flush"
-                   if bpn * nodes > 129e6 else "state fits in L2"},
+                   if BYTES_PER_NODE[args.storage] * nodes > 129e6 else "state fits in L2"},
         "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                      "frac": achieved / peak, "traffic": traffic,
                      "peak_source": f"{peak_src} HBM copy bandwidth",
                      "bytes_per_node": bpn,
-                     "kernel": "dmrt::step_tma_kernel" if launch["kernel"] == 2 else "dmrt::step_direct_kernel"},
+                     "steps_per_pass": per_pass,
+                     "one_step_per_pass_frac": BYTES_PER_NODE[args.storage] * nodes / per_launch_s / 1e9 / peak,
+                     "kernel": "dmrt::step_march_kernel" if per_pass > 1 else
+                     "dmrt::step_tma_kernel" if launch["kernel"] == 2 else "dmrt::step_direct_kernel"},
         "e2e": {"value": ws * nodes * args.steps / e2e_s / 1e6, "unit": UNIT,
                 "h2d_bytes_per_step": 8 * nodes / steps,
                 "d2h_bytes_per_step": (12 * nodes + 8 * args.steps) / steps},
-        "gpu_launches": args.steps + 1,  # one step kernel per step, one Nusselt finalize per run
+        "gpu_launches": launches_of(args.steps, per_pass),
         "clocks": sampler.summary(),
         "nu_mean_last": nu_mean,
     }

@@ -102,7 +102,12 @@ extern "C" {
  * 3) beyond (e.g. 112^2 to 256^2), DIRECT otherwise (e.g. 384^2); for runs of
  * steps of a float32 cavity whose rows split over 16 blocks give at most 1024
  * nodes per block (e.g. up to 128^2), and no tile asked for, the CLUSTER kernel
- * below where the GPU fits it (64^2: 1.43 against 2.66 us per step). TMA tiles
+ * below where the GPU fits it. Runs of steps of a whole cavity under AUTO, no tile
+ * asked for, take several steps per launch, with the same bits: six steps or
+ * more of a cavity up to about 512^2, in every storage mode, keep the state on
+ * chip across the GPU (64^2 0.92, 256^2 1.44, 512^2 3.5 us per step); larger
+ * cavities, from 40000 nodes and 160 columns, take three steps per pass over
+ * the state (4096^2 118 us per step, 288 with one). TMA tiles
  * compiled in, as (nodes per
  * thread, rows R, stages S): NPT 4 with (R,S) in (1,2) (1,3) (1,4) (1,5) (1,6)
  * (2,2) (2,3) (2,4) (4,2) (4,3); NPT 2 with (1,3) (1,4) (1,5) (2,2) (2,3)
@@ -475,16 +480,18 @@ int dmrt_adjoint(dmrt_ctx* c, int64_t nsteps, int64_t avg_last, void* workspace,
 /* ---- Batched sweep: many independent cavities per launch ----------------------
  *
  * Steps n independent side-heated cavities (any sizes and parameters; all
- * float32, or all mixed storage with one rounding mode) with one launch per time
- * step of a persistent TMA kernel over the
- * concatenated work items of all cavities, replayed from CUDA graphs. Each
+ * float32, or all mixed storage with one rounding mode) together: three time steps
+ * per launch over the concatenated work items of all cavities, or, when a tile or
+ * a schedule is asked for (dmrt_batch_opts), one launch per time step of a
+ * persistent TMA kernel, replayed from CUDA graphs; the same bits. Each
  * member is also an ordinary context (dmrt_batch_context), so dmrt_fields,
  * dmrt_nusselt, dmrt_get_state, ... work on it, and stepping the members one
  * by one with dmrt_step is the sequential alternative. The paper's four cases
  * (Table 1) are such a sweep over (Ra, Pr). */
 typedef struct dmrt_batch dmrt_batch;
 
-/* Tile of the batched kernel: nodes per thread, rows per item, pipeline stages
+/* All zero (or no options): three steps per launch, as above. Otherwise the tile
+ * of the one-step batched kernel: nodes per thread, rows per item, pipeline stages
  * (0 = default: 2, 2, 2 for FLOAT32, 4, 2, 2 for MIXED storage), and steps
  * per CUDA graph (0 = 64; must be even). Compiled tiles (npt, R, S), for both
  * storages and roundings: (1,1,2) (1,2,2) (1,4,2) (1,4,3) (2,1,2) (2,1,3)
