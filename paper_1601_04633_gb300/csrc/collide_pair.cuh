@@ -36,9 +36,6 @@ __device__ __forceinline__ float f2_hi(F2 a) {
     asm("mov.b64 {_, %0}, %1;" : "=f"(hi) : "l"(a));
     return hi;
 }
-__device__ __forceinline__ F2 f2_set(F2 a, bool hi, float v) {
-    return hi ? f2_pack(f2_lo(a), v) : f2_pack(v, f2_hi(a));
-}
 __device__ __forceinline__ F2 f2_add(F2 a, F2 b) {
     F2 d;
     asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));

@@ -204,7 +204,8 @@ struct MarchLane {
     bool two;          // both columns inside
     bool left, right;  // holds x = 0 (low half) / x = nx - 1
     bool rhi;          // right: nx - 1 is the high half
-    bool wall;         // the warp holds a side wall (uniform)
+    bool wall;         // the warp holds a side wall (uniform): the left one, the right one
+    bool wall_l, wall_r;
 };
 
 // The pair of direction k (flow: f, thermal: g) at columns x - EX, x + 1 - EX
@@ -262,19 +263,26 @@ __device__ __forceinline__ float wall_value(float sign, float og, float add) { r
 // Side walls at a pulled pair: links from outside x = 0 (directions 1, 5, 8 and
 // g 1) and x = nx - 1 (3, 6, 7 and g 3) from the node's own opposites: own f 3,
 // f 7, f 6, g 3 (left) or f 1, f 8, f 5, g 1 (right), and the wall's temperature term.
+template <bool FLAT>
 __device__ __forceinline__ void side_walls(F2 (&f)[9], F2 (&g)[5], const MarchLane& n, const MarchArgs& M, float of,
                                            float oa, float ob, float og, float add) {
-    if (n.left) {
-        f[1] = f2_set(f[1], false, of);
-        f[5] = f2_set(f[5], false, oa);
-        f[8] = f2_set(f[8], false, ob);
-        g[1] = f2_set(g[1], false, wall_value(M.sign_l, og, add));
+    // Selects: changing one half of a packed pair in a divergent branch is not safe
+    // with nvcc 13.0 (see step_band.cuh). FLAT: both sides' without a branch (float32,
+    // 1 % faster; in 16-bit storage the registers it takes cost 2 %).
+    const bool rl = n.right && !n.rhi, rh = n.right && n.rhi;
+    auto left = [&](F2 v, float w) { return f2_pack(n.left ? w : f2_lo(v), f2_hi(v)); };
+    auto right = [&](F2 v, float w) { return f2_pack(rl ? w : f2_lo(v), rh ? w : f2_hi(v)); };
+    if (FLAT || n.wall_l) {
+        f[1] = left(f[1], of);
+        f[5] = left(f[5], oa);
+        f[8] = left(f[8], ob);
+        g[1] = left(g[1], wall_value(M.sign_l, og, add));
     }
-    if (n.right) {
-        f[3] = f2_set(f[3], n.rhi, of);
-        f[6] = f2_set(f[6], n.rhi, oa);
-        f[7] = f2_set(f[7], n.rhi, ob);
-        g[3] = f2_set(g[3], n.rhi, wall_value(M.sign_r, og, add));
+    if (FLAT || n.wall_r) {
+        f[3] = right(f[3], of);
+        f[6] = right(f[6], oa);
+        f[7] = right(f[7], ob);
+        g[3] = right(g[3], wall_value(M.sign_r, og, add));
     }
 }
 
@@ -416,7 +424,9 @@ __device__ __forceinline__ void march_item(const CUtensorMap* ld, const CUtensor
     n.left = n.x0 == 0;
     n.right = n.x0 >= 0 && (n.x0 == A.nx - 1 || n.x0 + 1 == A.nx - 1);
     n.rhi = n.x0 + 1 == A.nx - 1;
-    n.wall = strip == 0 || (strip + 1) * G::kCols + G::kLead >= A.nx;
+    n.wall_l = strip == 0;
+    n.wall_r = (strip + 1) * G::kCols + G::kLead >= A.nx;
+    n.wall = n.wall_l || n.wall_r;
     unsigned salt[T];
 #pragma unroll
     for (int s = 0; s < T; ++s)
@@ -522,7 +532,7 @@ __device__ __forceinline__ void march_item(const CUtensorMap* ld, const CUtensor
             const float oa = own(lf ? row_f<L, 0>(Z, 7, c) : row_f<L, 0>(Z, 8, c));
             const float ob = own(lf ? row_f<L, 0>(Z, 6, c) : row_f<L, 0>(Z, 5, c));
             const float og = own(lf ? row_g<L, 0>(Z, 3, c, M) : row_g<L, 0>(Z, 1, c, M));
-            side_walls(f, g, n, M, of, oa, ob, og, add);
+            side_walls<!G::k16>(f, g, n, M, of, oa, ob, og, add);
             if (r < last) nadd = wall_term(r + 1);  // in flight during this row
         }
         __syncwarp();  // every lane has read row r - 1: its stage takes the next row to load
@@ -562,7 +572,7 @@ __device__ __forceinline__ void march_item(const CUtensorMap* ld, const CUtensor
             const float padd = X.wadd;
             if (n.wall) {
                 const bool lf = n.left;
-                side_walls(F, H, n, M, own(lf ? X.zf3 : X.zf1), X.wa, own(lf ? X.pf6 : X.pf5),
+                side_walls<!G::k16>(F, H, n, M, own(lf ? X.zf3 : X.zf1), X.wa, own(lf ? X.pf6 : X.pf5),
                            own(lf ? X.zg3 : X.zg1), padd);
                 X.wa = n.left ? f2_lo(f[7]) : own(f[8]);
                 X.wadd = add;
