@@ -316,6 +316,13 @@ int dmrt_load(dmrt_ctx* c, const void* host_buf, size_t size);
  * Uses a file-scope device word; allocates nothing. Synchronises the stream. */
 int dmrt_probe_bounded_wait(int64_t limit_ns, void* stream, int64_t* waited_ns);
 
+/* The same for a launch of several steps per pass: one warp's work on the top row of
+ * a float32 context that takes such launches (else DMRT_E_ARG), with the copy of
+ * the row'th row it loads (0 to 3) never complete. The warp must store nothing and record
+ * the expiry: returns DMRT_E_TIMEOUT, which stays the context's error (DMRT_OK: a
+ * defect). limit_ns in [1 ms, 2 s]. Synchronises. */
+int dmrt_probe_march_wait(dmrt_ctx* c, int32_t row, int64_t limit_ns);
+
 /* ---- One step without any device allocation (the paper has no counterpart) ----
  *
  * For callers that cannot allocate device memory where they step a cavity: code

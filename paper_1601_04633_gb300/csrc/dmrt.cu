@@ -1892,6 +1892,24 @@ int dmrt_check(dmrt_ctx* c) {
     return poll_error(c);
 }
 
+int dmrt_probe_march_wait(dmrt_ctx* c, int32_t row, int64_t limit_ns) {
+    if (!c) return DMRT_E_ARG;
+    if (!c->march[3] || c->p.storage != DMRT_FP32 || c->p.ny < 4 || row < 0 || row >= dmrt::kMarchStages ||
+        limit_ns < 1000000 || limit_ns > (int64_t)dmrt::kWaitLimitNs) {
+        set_err(c, "dmrt_probe_march_wait: float32 context with march launches, row in [0, 3], limit in [1 ms, 2 s]");
+        return DMRT_E_ARG;
+    }
+    // The cavity's last row as a chunk of its own: its launch loads the last four
+    // rows only, so that each stage is filled once.
+    dmrt::MarchArgs M = march_args(c, c->cur, 3);
+    M.chunk = 1;
+    M.n_chunks = c->p.ny;
+    CK(dmrt::launch_march_wait_probe(c->mmaps[c->cur], M, c->pc, M.n_strips * (c->p.ny - 1), row,
+                                     (unsigned long long)limit_ns, c->stream),
+       "march wait probe");
+    return poll_error(c);
+}
+
 int64_t dmrt_steps_done(const dmrt_ctx* c) { return c ? c->t : -1; }
 
 int dmrt_nusselt_flux(dmrt_ctx* c, double* nu_mean, double* nu_local) {

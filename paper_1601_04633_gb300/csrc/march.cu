@@ -25,4 +25,28 @@ MarchForm march_form(int storage, int rounding, int steps) {
     return {nullptr, 0, 0, 0};
 }
 
+static __global__ void __launch_bounds__(32)
+    march_wait_probe_kernel(const __grid_constant__ MarchMaps maps, const __grid_constant__ MarchArgs M,
+                            const __grid_constant__ PairConsts K, int item, int row, unsigned long long limit_ns) {
+    using L = OneType<float>;
+    extern __shared__ __align__(1024) unsigned char smem_m[];
+    const int lane = threadIdx.x;
+    uint64_t* bars = reinterpret_cast<uint64_t*>(smem_m + MarchGeo<L>::kWarp);
+    if (lane == 0) {
+        for (int s = 0; s < kMarchStages; ++s) mbar_init(&bars[s], s == row ? 2 : 1);
+        mbar_fence_init();
+    }
+    __syncwarp();
+    march_item<L, false, 3>(maps.ld, maps.st, M, K.r, K.n, item, lane, smem_m, bars, limit_ns);
+}
+
+cudaError_t launch_march_wait_probe(const MarchMaps& maps, const MarchArgs& M, const PairConsts& K, int item, int row,
+                                    unsigned long long limit_ns, cudaStream_t stream) {
+    constexpr unsigned smem = MarchGeo<OneType<float>>::kSmem;
+    const cudaError_t e = cudaFuncSetAttribute(march_wait_probe_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    march_wait_probe_kernel<<<1, 32, smem, stream>>>(maps, M, K, item, row, limit_ns);
+    return cudaGetLastError();
+}
+
 }  // namespace dmrt

@@ -408,7 +408,8 @@ struct MarchCarry {
 template <typename L, bool SR, int T>
 __device__ __forceinline__ void march_item(const CUtensorMap* ld, const CUtensorMap* st, const MarchArgs& M,
                                            const PairRates& K, const PairNumbers& C9, int item, int lane,
-                                           unsigned char* ring, uint64_t* bars) {
+                                           unsigned char* ring, uint64_t* bars,
+                                           unsigned long long limit_ns = kWaitLimitNs) {
     using G = MarchGeo<L>;
     static_assert(T >= 2 && T <= kMarchMax && T - 1 <= G::kLead, "a strip's side columns");
     const StepArgs& A = M.A;
@@ -447,13 +448,13 @@ __device__ __forceinline__ void march_item(const CUtensorMap* ld, const CUtensor
         if constexpr (L::kTheta) tma_load_3d(s + G::d_at(G::kBox), &ld[2], x, row, 0, b);
     };
     auto arrived = [&](int row) {
-        return __all_sync(kFull, mbar_wait_bounded(bar(row), (unsigned)((row - lb) / kMarchStages) & 1u));
+        return __all_sync(kFull, mbar_wait_bounded(bar(row), (unsigned)((row - lb) / kMarchStages) & 1u, limit_ns));
     };
     int issued = min(ub + 1, lb + kMarchStages);  // rows below this one have been issued
     if (lane == 0)
         for (int row = lb; row < issued; ++row) issue(row);
     bool ok = true;
-    int waited = lb;  // rows below this one have arrived
+    int waited = lb;  // rows below this one have arrived (!ok: those below waited - 1)
     for (; waited <= rs && ok; ++waited) ok = arrived(waited);
 
     MarchCarry C[T - 1];
@@ -485,7 +486,7 @@ __device__ __forceinline__ void march_item(const CUtensorMap* ld, const CUtensor
     // unrolling the loop, in instruction fetches.)
     const int last = min(rend, A.ny - 1);
 #pragma unroll 1
-    for (int r = rs; r <= rend; ++r) {
+    for (int r = ok ? rs : rend + 1; r <= rend; ++r) {  // (no row when the first ones did not arrive)
         if (waited <= ub) {
             ok = arrived(waited);
             ++waited;
@@ -616,7 +617,7 @@ __device__ __forceinline__ void march_item(const CUtensorMap* ld, const CUtensor
     if (!ok && lane == 0) {
         atomicOr(A.err, kErrTimeout);
         for (int row = waited - 1; row < issued; ++row)
-            mbar_wait_bounded(bar(row), (unsigned)((row - lb) / kMarchStages) & 1u);
+            mbar_wait_bounded(bar(row), (unsigned)((row - lb) / kMarchStages) & 1u, limit_ns);
     }
     if (n.out && (!(peak0 < 1e30f) || (n.two && !(peak1 < 1e30f)))) atomicOr(A.err, kErrNonFinite);
 }
@@ -716,5 +717,10 @@ struct MarchForm {
 };
 MarchForm march_form(int storage, int rounding, int steps);
 MarchForm batch_march_form(int storage, int rounding, int steps);  // float32 and mixed storage
+
+// One float32 item by one warp, the copy of the chunk's row `row` (from its first one
+// loaded) never complete: the barrier waits for an arrival that nobody makes.
+cudaError_t launch_march_wait_probe(const MarchMaps& maps, const MarchArgs& M, const PairConsts& K, int item, int row,
+                                    unsigned long long limit_ns, cudaStream_t stream);
 
 }  // namespace dmrt

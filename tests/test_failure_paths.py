@@ -54,6 +54,24 @@ def test_bounded_wait_gives_up_and_the_context_stays_usable(D):
     assert L.dmrt_probe_bounded_wait(10, ctypes.c_void_p(stream), None) == D.DMRT_E_ARG
 
 
+@pytest.mark.parametrize("row", [0, 1, 2, 3])
+def test_a_march_launch_reports_any_row_that_does_not_arrive(D, row):
+    # 0 and 1 are waited for before the first row of the chunk, 2 and 3 in its rows.
+    import torch
+
+    sim = D.Cavity2D.from_inputs(inputs.Cavity(1100, 64, 1e4, 0.01, noise_amp=1e-3, seed=8), nu_capacity=64)
+    sim.step(6)
+    sim.check()
+    before = sim.workspace.clone()
+    assert D.load().dmrt_probe_march_wait(sim.h, row, 20_000_000) == D.DMRT_E_TIMEOUT
+    torch.cuda.synchronize()
+    assert int((sim.workspace != before).sum()) == 1  # one bit of the error word, and no row stored
+    with pytest.raises(D.DmrtError) as ei:
+        sim.check()
+    assert ei.value.code == D.DMRT_E_TIMEOUT
+    sim.close()
+
+
 def test_long_step_call_stops_at_the_divergence_poll(D):
     # A NaN temperature in one node: dmrt_step polls the error word each time the
     # step count passes a multiple of 65536 and returns DMRT_E_DIVERGED there.
