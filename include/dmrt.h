@@ -416,15 +416,36 @@ int dmrt_slab_pack(dmrt_ctx* c, void* to_below, void* to_above);
 int dmrt_slab_unpack(dmrt_ctx* c, const void* from_below, const void* from_above);
 int dmrt_slab_step(dmrt_ctx* c, void* to_below, void* to_above);
 
-/* Launch configuration a context resolved to (for reports and tuning). */
+/* Launch configuration a context resolved to (for reports and tuning): of single
+ * steps (DIRECT or TMA and its tile), or of the cluster kernel where the context has
+ * that one. Runs of steps under AUTO may take another kernel with several steps per
+ * launch: dmrt_get_run_launch says which. */
 typedef struct {
-    int32_t kernel;       /* DMRT_KERNEL_DIRECT or DMRT_KERNEL_TMA */
+    int32_t kernel;       /* DMRT_KERNEL_DIRECT, DMRT_KERNEL_TMA or DMRT_KERNEL_CLUSTER */
     int32_t tma_npt, tma_rows, tma_stages;
     int32_t grid, block;  /* blocks per step launch, threads per block */
     int64_t smem_bytes;   /* dynamic shared memory per block */
-    int32_t graph_steps;  /* steps per captured CUDA graph */
+    int32_t graph_steps;  /* one-step launches per captured CUDA graph */
 } dmrt_launch;
 int dmrt_get_launch(const dmrt_ctx* c, dmrt_launch* out);
+
+/* The launches of a run: what dmrt_step(c, nsteps), called now, would enqueue, and the
+ * kernel that takes the most steps of it. MARCH and BAND are kernels of AUTO alone
+ * (dmrt_create refuses them). Host logic, no device call. DMRT_E_ARG for NULL or nsteps < 1. */
+#define DMRT_KERNEL_MARCH 4 /* two or three steps per pass over the state */
+#define DMRT_KERNEL_BAND 5  /* many steps per launch, the state on chip across blocks */
+typedef struct {
+    int32_t kernel;            /* DMRT_KERNEL_DIRECT, _TMA, _CLUSTER, _MARCH or _BAND */
+    int32_t steps_per_launch;  /* steps of its longest launch */
+    int32_t rows;              /* rows of a block (CLUSTER, BAND), of a chunk (MARCH) or of a tile (TMA) */
+    int32_t cluster;           /* 1: its blocks form one thread-block cluster */
+    int32_t grid, block;       /* blocks per launch, threads per block */
+    int64_t smem_bytes;        /* dynamic shared memory per block */
+    int64_t steps;             /* steps it takes of the run */
+    int64_t launches;          /* kernels that the whole run enqueues, Nusselt sums included */
+    int32_t graph_steps;       /* steps per CUDA-graph replay, 0 if the run replays none */
+} dmrt_run_launch;
+int dmrt_get_run_launch(const dmrt_ctx* c, int64_t nsteps, dmrt_run_launch* out);
 
 /* The kernel and tile (nodes per thread, rows, stages) that dmrt_create would
  * choose for parameters p on a GPU with sms streaming multiprocessors: host
@@ -565,7 +586,10 @@ int32_t dmrt_batch_group_count(const dmrt_batch* b);
 /* Member i as a context (borrowed: do not destroy it), or NULL. */
 dmrt_ctx* dmrt_batch_context(dmrt_batch* b, int32_t i);
 
+/* The batch's one-step kernel and tile (as dmrt_get_launch), and the launches that
+ * dmrt_batch_step(b, nsteps) enqueues (as dmrt_get_run_launch). */
 int dmrt_batch_get_launch(const dmrt_batch* b, dmrt_launch* out);
+int dmrt_batch_get_run_launch(const dmrt_batch* b, int64_t nsteps, dmrt_run_launch* out);
 const char* dmrt_batch_last_error(const dmrt_batch* b);
 
 /* Release the batch and its member contexts (not the workspace). */

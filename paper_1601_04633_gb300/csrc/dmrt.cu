@@ -6,6 +6,7 @@
 #include <cuda_runtime.h>
 #include <cudaTypedefs.h>
 
+#include <algorithm>
 #include <cmath>
 #include <cstdarg>
 #include <cstdio>
@@ -1684,6 +1685,32 @@ static int launch_band(dmrt_ctx* c, int n, float* record = nullptr, long long st
     return DMRT_OK;
 }
 
+// The next launch of a run with `left` steps to go (the rules that pick the kernel of a
+// run): its kernel and its steps. to_poll: steps until the next divergence poll;
+// pair: half of a pair of two-step march launches is done.
+enum RunKind { kRunOne, kRunCluster, kRunMarch, kRunGraph, kRunBand };
+struct RunLaunch {
+    RunKind kind;
+    int n;
+};
+static RunLaunch next_launch(const dmrt_ctx* c, int64_t left, int64_t to_poll, bool pair) {
+    if (c->band && left >= dmrt::kBandMinSteps) {
+        // Up to the next divergence poll, with no remainder too short for a launch of its own.
+        long long n = std::min<long long>(left, std::max<long long>(dmrt::kBandMinSteps, to_poll));
+        n = std::min<long long>(n, dmrt::kBandSteps);
+        const long long rest = left - n;
+        if (rest > 0 && rest < dmrt::kBandMinSteps) n = left <= dmrt::kBandSteps ? left : n - dmrt::kBandMinSteps;
+        return {kRunBand, (int)n};
+    }
+    if (c->cluster) {  // up to the next divergence poll, in one launch
+        const long long n = std::min<long long>(left, std::max<long long>(1, to_poll));
+        return {n >= 2 ? kRunCluster : kRunOne, (int)n};
+    }
+    if (left >= graph_steps(c)) return {kRunGraph, graph_steps(c)};
+    const int n = pair ? 2 : launch_steps(c, left);
+    return {n > 1 ? kRunMarch : kRunOne, n};
+}
+
 // nsteps steps; with `finalize`, the last step's Nusselt rows are summed into
 // the ring at the end (without, the next launch sums them). With `record`
 // (cluster kernel only), the state after the run's step s is also written to
@@ -1691,26 +1718,6 @@ static int launch_band(dmrt_ctx* c, int n, float* record = nullptr, long long st
 static int step_run(dmrt_ctx* c, int64_t nsteps, bool finalize, float* record = nullptr, long long stride = 0) {
     if (!c || nsteps < 0) return DMRT_E_ARG;
     if (record && !c->cluster) return DMRT_E_ARG;
-    if (c->cluster && (!c->band || nsteps < dmrt::kBandMinSteps)) {
-        while (nsteps > 0) {
-            if (c->t >= c->next_poll) {
-                c->next_poll = c->t + kPollSteps;
-                int rc = poll_error(c);
-                if (rc) return rc;
-            }
-            // Up to the next divergence poll, in one launch.
-            const long long n = std::min<long long>(nsteps, std::max<long long>(1, c->next_poll - c->t));
-            int rc = n >= 2 ? launch_cluster(c, (int)n, record, stride) : launch_one(c);
-            if (rc) return rc;
-            if (record && n < 2)
-                CK(cudaMemcpyAsync(record, buf(c, c->cur), (size_t)kPlanes * (size_t)c->L.plane * sizeof(float),
-                                   cudaMemcpyDeviceToDevice, c->stream),
-                   "record");
-            if (record) record += n * stride;
-            nsteps -= n;
-        }
-        return finalize ? finalize_nu(c) : DMRT_OK;
-    }
     if (c->slab && !(c->wall_lo && c->wall_hi) && nsteps > 1) {
         set_err(c, "a slab with neighbours takes one step at a time (dmrt_slab_step), its halo rows "
                    "exchanged in between");
@@ -1727,55 +1734,117 @@ static int step_run(dmrt_ctx* c, int64_t nsteps, bool finalize, float* record = 
             if (!rc) rc = poll_error(c);
             if (rc) return rc;
         }
-        if (c->band && (nsteps >= dmrt::kBandMinSteps || record)) {
-            // Up to the next divergence poll, with no remainder too short for a launch of its own.
-            long long n = std::min<long long>(nsteps, std::max<long long>(dmrt::kBandMinSteps, c->next_poll - c->t));
-            n = std::min<long long>(n, dmrt::kBandSteps);
-            const long long rest = nsteps - n;
-            if (rest > 0 && rest < dmrt::kBandMinSteps) n = nsteps <= dmrt::kBandSteps ? nsteps : n - dmrt::kBandMinSteps;
-            int rc = launch_band(c, (int)n, record, stride);
-            if (rc == kNoBand) {
-                (void)cudaGetLastError();
-                c->band = nullptr;  // the other kernels take the rest, and later runs
-                return step_run(c, nsteps, finalize, record, stride);
-            }
-            if (rc) return rc;
-            if (record) record += n * stride;
-            nsteps -= n;
-            finalize = finalize && nsteps > 0;
-            continue;
-        }
-        if (nsteps >= graph_steps(c)) {
-            if (!c->graph[c->cur]) {
-                int rc = build_graph(c, c->cur);
+        const RunLaunch r = next_launch(c, nsteps, c->next_poll - c->t, pair);
+        int rc = DMRT_OK;
+        switch (r.kind) {
+            case kRunBand:
+                rc = launch_band(c, r.n, record, stride);
+                if (rc == kNoBand) {
+                    (void)cudaGetLastError();
+                    c->band = nullptr;  // the other kernels take the rest, and later runs
+                    continue;
+                }
+                finalize = finalize && nsteps > r.n;  // (its Nusselt numbers are summed)
+                break;
+            case kRunCluster:
+                rc = launch_cluster(c, r.n, record, stride);
+                break;
+            case kRunGraph:
+                if (!c->graph[c->cur]) rc = build_graph(c, c->cur);
                 if (rc) return rc;
+                CK(cudaGraphLaunch(c->graph[c->cur], c->stream), "cudaGraphLaunch");
+                c->t += r.n;  // an even number of launches: the state stays in the same buffer
+                marched = c->march[2] != nullptr;
+                c->nu_open = true;
+                break;
+            case kRunMarch: {
+                pair = r.n == 2 && !pair;  // the second launch of a pair
+                dmrt::MarchArgs M = march_args(c, c->cur, r.n);
+                void* params[3] = {&c->mmaps[c->cur], &M, &c->pc};
+                CK(launch_overlapped(c->march[r.n], dim3(march_grid(c, r.n)), dim3(dmrt::kMarchThreads), c->msmem,
+                                     c->stream, params),
+                   "march launch");
+                c->cur ^= 1;
+                c->t += r.n;
+                marched = true;
+                c->nu_open = true;
+                break;
             }
-            CK(cudaGraphLaunch(c->graph[c->cur], c->stream), "cudaGraphLaunch");
-            c->t += graph_steps(c);  // an even number of launches: the state stays in the same buffer
-            nsteps -= graph_steps(c);
-            marched = c->march[2] != nullptr;
-            c->nu_open = true;
-        } else if (const int n = pair ? 2 : launch_steps(c, nsteps); n > 1) {
-            pair = n == 2 && !pair;  // the second launch of a pair
-            dmrt::MarchArgs M = march_args(c, c->cur, n);
-            void* params[3] = {&c->mmaps[c->cur], &M, &c->pc};
-            CK(launch_overlapped(c->march[n], dim3(march_grid(c, n)), dim3(dmrt::kMarchThreads), c->msmem, c->stream, params),
-               "march launch");
-            c->cur ^= 1;
-            c->t += n;
-            nsteps -= n;
-            marched = true;
-            c->nu_open = true;
-        } else {
-            // (a single step sums one earlier step's Nusselt rows, not a march launch's two)
-            int rc = marched ? finalize_nu(c) : DMRT_OK;
-            if (!rc) rc = launch_one(c);
-            if (rc) return rc;
-            marched = false;
-            nsteps -= 1;
+            case kRunOne:
+                // (a single step sums one earlier step's Nusselt rows, not a march launch's)
+                rc = marched ? finalize_nu(c) : DMRT_OK;
+                if (!rc) rc = launch_one(c);
+                if (!rc && record)
+                    CK(cudaMemcpyAsync(record, buf(c, c->cur), (size_t)kPlanes * (size_t)c->L.plane * sizeof(float),
+                                       cudaMemcpyDeviceToDevice, c->stream),
+                       "record");
+                marched = false;
+                break;
         }
+        if (rc) return rc;
+        if (record) record += r.n * stride;
+        nsteps -= r.n;
     }
     return finalize || marched ? finalize_nu(c) : DMRT_OK;
+}
+
+int dmrt_get_run_launch(const dmrt_ctx* c, int64_t nsteps, dmrt_run_launch* out) {
+    if (!c || !out || nsteps < 1) return DMRT_E_ARG;
+    std::memset(out, 0, sizeof *out);
+    long long steps[5] = {}, to_poll = c->next_poll - c->t;
+    bool pair = false, marched = false, summed = false;
+    for (long long left = nsteps; left > 0;) {  // the run, as step_run takes it
+        if (to_poll <= 0) to_poll = kPollSteps, out->launches += 1;
+        const RunLaunch r = next_launch(c, left, to_poll, pair);
+        pair = r.kind == kRunMarch && r.n == 2 && !pair;
+        if (r.kind == kRunOne && marched) out->launches += 1;  // the march launches' sums
+        marched = r.kind == kRunMarch || (r.kind == kRunGraph && c->march[2]);
+        summed = r.kind == kRunBand;
+        out->launches += r.kind == kRunGraph ? c->graph_len : r.kind == kRunBand ? 2 : 1;
+        steps[r.kind] += r.n;
+        left -= r.n;
+        to_poll -= r.n;
+    }
+    if (!summed) out->launches += 1;
+    out->graph_steps = steps[kRunGraph] > 0 ? graph_steps(c) : 0;
+    steps[c->march[2] ? kRunMarch : kRunOne] += steps[kRunGraph];  // (the graphs' launches)
+    steps[kRunGraph] = 0;
+    const int most = (int)(std::max_element(steps, steps + 5) - steps);
+    out->steps = steps[most];
+    if (most == kRunBand) {
+        out->kernel = DMRT_KERNEL_BAND;
+        out->steps_per_launch = (int32_t)std::min<long long>(nsteps, dmrt::kBandSteps);
+        out->cluster = c->band_cluster;
+        out->rows = c->brows;
+        out->grid = c->bblocks;
+        out->block = c->bthreads;
+        out->smem_bytes = (int64_t)c->bsmem;
+    } else if (most == kRunMarch) {
+        const int n = launch_steps(c, nsteps);
+        out->kernel = DMRT_KERNEL_MARCH;
+        out->steps_per_launch = n;
+        out->rows = c->mchunk[n];
+        out->grid = march_grid(c, n);
+        out->block = dmrt::kMarchThreads;
+        out->smem_bytes = (int64_t)c->msmem;
+    } else if (most == kRunCluster) {
+        out->kernel = DMRT_KERNEL_CLUSTER;
+        out->steps_per_launch = (int32_t)std::min<long long>(nsteps, kPollSteps);
+        out->cluster = 1;
+        out->rows = c->crows;
+        out->grid = c->csize;
+        out->block = c->cthreads;
+        out->smem_bytes = (int64_t)c->csmem;
+    } else {
+        out->kernel = c->kernel;
+        out->steps_per_launch = 1;
+        const bool tma = c->kernel == DMRT_KERNEL_TMA;
+        out->rows = tma ? c->R : 0;
+        out->grid = tma ? c->tma_grid : (int32_t)(c->grid.x * c->grid.y);
+        out->block = tma ? c->tma_block : dmrt::kDirectThreads;
+        out->smem_bytes = tma ? (int64_t)c->tma_smem : 0;
+    }
+    return DMRT_OK;
 }
 
 int dmrt_step(dmrt_ctx* c, int64_t nsteps) { return step_run(c, nsteps, true); }
@@ -2995,6 +3064,9 @@ static int batch_march(dmrt_batch* b, int n, int parity) {
     return DMRT_OK;
 }
 
+// Steps of the next march launch: three, or two in a pair of launches (see launch_steps).
+static int batch_march_steps(int64_t n) { return n == 4 || n == 5 ? 2 : 3; }
+
 int dmrt_batch_step(dmrt_batch* b, int64_t nsteps) {
     if (!b || nsteps < 0) return DMRT_E_ARG;
     for (int i = 0; i < b->n; ++i) {
@@ -3011,8 +3083,8 @@ int dmrt_batch_step(dmrt_batch* b, int64_t nsteps) {
     const int64_t total = nsteps;
     if (b->march[3] && nsteps >= 3) {
         while (nsteps >= 3) {
-            const int n = nsteps == 4 || nsteps == 5 ? 2 : 3;
-            for (int k = 0; k < (n == 2 ? 2 : 1); ++k) {  // two steps in pairs only (see launch_steps)
+            const int n = batch_march_steps(nsteps);
+            for (int k = 0; k < (n == 2 ? 2 : 1); ++k) {
                 int rc = batch_march(b, n, start);
                 if (rc) return rc;
                 start ^= 1;
@@ -3088,6 +3160,45 @@ int32_t dmrt_batch_size(const dmrt_batch* b) { return b ? b->n : 0; }
 dmrt_ctx* dmrt_batch_context(dmrt_batch* b, int32_t i) {
     if (!b || i < 0 || i >= b->n) return nullptr;
     return b->sub[i];
+}
+
+int dmrt_batch_get_run_launch(const dmrt_batch* b, int64_t nsteps, dmrt_run_launch* out) {
+    if (!b || !out || nsteps < 1) return DMRT_E_ARG;
+    std::memset(out, 0, sizeof *out);
+    const long long groups = (long long)b->groups.size();
+    if (b->march[3] && nsteps >= 3) {
+        const long long parts = (long long)b->margs[3][0].size();
+        long long left = nsteps, launches = 0;
+        while (left >= 3) {
+            const int n = batch_march_steps(left), k = n == 2 ? 2 : 1;
+            launches += k;
+            left -= k * n;
+        }
+        const int n = batch_march_steps(nsteps);
+        const dmrt::MarchBatchArgs& B = b->margs[n][0][0];
+        out->kernel = DMRT_KERNEL_MARCH;
+        out->steps_per_launch = n;
+        out->steps = nsteps - left;
+        out->launches = (launches + 1) * parts + (left > 0 ? left + 1 : 0);  // (march: one group)
+        out->rows = B.M[0].chunk;
+        out->grid = (B.items + dmrt::kMarchThreads / 32 - 1) / (dmrt::kMarchThreads / 32) + B.n_cav;
+        out->block = dmrt::kMarchThreads;
+        out->smem_bytes = (int64_t)b->msmem;
+        return DMRT_OK;
+    }
+    // Graphs of one-step launches, or of two launches of K steps; single steps for the rest.
+    const long long graphs = nsteps / b->graph_len, rest = nsteps - graphs * b->graph_len;
+    const bool multi = b->K > 1 && graphs > 0;
+    out->kernel = DMRT_KERNEL_TMA;
+    out->steps_per_launch = multi ? b->K : 1;
+    out->steps = multi ? graphs * b->graph_len : nsteps;
+    out->launches = (graphs * (b->K > 1 ? 2 : b->graph_len) + rest + 1) * groups;
+    out->rows = b->R;
+    out->block = b->block;
+    out->smem_bytes = (int64_t)b->smem;
+    for (const BatchGroup& G : b->groups) out->grid = std::max(out->grid, multi ? G.mgrid : G.grid);
+    out->graph_steps = graphs > 0 ? b->graph_len : 0;
+    return DMRT_OK;
 }
 
 int dmrt_batch_get_launch(const dmrt_batch* b, dmrt_launch* out) {

@@ -34,6 +34,7 @@ DMRT_E_BOUNDS = -8
 DMRT_FP32, DMRT_FP16, DMRT_BF16, DMRT_MIXED, DMRT_THETA32 = 0, 1, 2, 3, 4
 DMRT_WALL_FIXED, DMRT_WALL_ADIABATIC = 0, 1
 DMRT_KERNEL_AUTO, DMRT_KERNEL_DIRECT, DMRT_KERNEL_TMA, DMRT_KERNEL_CLUSTER = 0, 1, 2, 3
+DMRT_KERNEL_MARCH, DMRT_KERNEL_BAND = 4, 5  # reported by run_launch, AUTO's own
 DMRT_ROUND_NEAREST, DMRT_ROUND_STOCHASTIC, DMRT_ROUND_AUTO = 0, 1, 2
 DMRT_NOALLOC_MAX_NY = 8192
 # Device plane order of the population buffers: entry d is the index, in the host
@@ -89,6 +90,15 @@ class Launch(ctypes.Structure):
         return {n: getattr(self, n) for n, _ in self._fields_}
 
 
+class RunLaunch(ctypes.Structure):
+    _fields_ = [("kernel", ctypes.c_int32), ("steps_per_launch", ctypes.c_int32), ("rows", ctypes.c_int32),
+                ("cluster", ctypes.c_int32), ("grid", ctypes.c_int32), ("block", ctypes.c_int32),
+                ("smem_bytes", ctypes.c_int64), ("steps", ctypes.c_int64), ("launches", ctypes.c_int64),
+                ("graph_steps", ctypes.c_int32)]
+
+    as_dict = Launch.as_dict
+
+
 class BatchOpts(ctypes.Structure):
     _fields_ = [("tma_npt", ctypes.c_int32), ("tma_rows", ctypes.c_int32),
                 ("tma_stages", ctypes.c_int32), ("graph_steps", ctypes.c_int32),
@@ -120,6 +130,7 @@ SIGNATURES = {
     "dmrt_energy": (ctypes.c_int, [_VP, _DP, _DP]),
     "dmrt_get_consts": (ctypes.c_int, [_VP, ctypes.POINTER(Consts)]),
     "dmrt_get_launch": (ctypes.c_int, [_VP, ctypes.POINTER(Launch)]),
+    "dmrt_get_run_launch": (ctypes.c_int, [_VP, ctypes.c_int64, ctypes.POINTER(RunLaunch)]),
     "dmrt_choose_launch": (ctypes.c_int, [ctypes.POINTER(Params), ctypes.c_int32] + [ctypes.POINTER(ctypes.c_int32)] * 4),
     "dmrt_get_state": (ctypes.c_int, [_VP, _FP]),
     "dmrt_set_state": (ctypes.c_int, [_VP, _FP]),
@@ -151,6 +162,7 @@ SIGNATURES = {
     "dmrt_batch_size": (ctypes.c_int32, [_VP]),
     "dmrt_batch_group_count": (ctypes.c_int32, [_VP]),
     "dmrt_batch_context": (_VP, [_VP, ctypes.c_int32]),
+    "dmrt_batch_get_run_launch": (ctypes.c_int, [_VP, ctypes.c_int64, ctypes.POINTER(RunLaunch)]),
     "dmrt_batch_get_launch": (ctypes.c_int, [_VP, ctypes.POINTER(Launch)]),
     "dmrt_batch_last_error": (ctypes.c_char_p, [_VP]),
     "dmrt_batch_destroy": (None, [_VP]),
@@ -280,6 +292,12 @@ def dmrt_get_consts(h) -> Consts:
 def dmrt_get_launch(h) -> Launch:
     k = Launch()
     _check(load().dmrt_get_launch(h, ctypes.byref(k)), h)
+    return k
+
+
+def dmrt_get_run_launch(h, nsteps: int) -> RunLaunch:
+    k = RunLaunch()
+    _check(load().dmrt_get_run_launch(h, int(nsteps), ctypes.byref(k)), h)
     return k
 
 
@@ -423,6 +441,11 @@ class Cavity2D:
 
     def step(self, n: int):
         dmrt_step(self.h, n)
+
+    def run_launch(self, n: int) -> dict:
+        """The launches that ``step(n)`` would enqueue now, and the kernel that takes most of
+        its steps (see ``dmrt_run_launch``; ``launch`` is the kernel of single steps)."""
+        return dmrt_get_run_launch(self.h, n).as_dict()
 
     def check(self):
         dmrt_check(self.h)
@@ -600,8 +623,9 @@ class _Member(Cavity2D):
 
 
 class Batch:
-    """Independent cavities stepped together by the batched kernel (one launch
-    per time step); ``members[i]`` exposes each as a context."""
+    """Independent cavities stepped together, three time steps per launch, or with
+    ``opts`` (a tile or a schedule) by the one-step batched kernel; ``run_launch(n)``
+    says which. ``members[i]`` exposes each as a context."""
 
     def __init__(self, params_list, theta0_list=None, opts=None, device="cuda", stream=None):
         import torch
@@ -655,6 +679,12 @@ class Batch:
 
     def step(self, n: int):
         _check_batch(load().dmrt_batch_step(self.b, int(n)), self.b)
+
+    def run_launch(self, n: int) -> dict:
+        """The launches that ``step(n)`` would enqueue now (see ``dmrt_run_launch``)."""
+        k = RunLaunch()
+        _check_batch(load().dmrt_batch_get_run_launch(self.b, int(n), ctypes.byref(k)), self.b)
+        return k.as_dict()
 
     def check(self):
         _check_batch(load().dmrt_batch_check(self.b), self.b)

@@ -1,0 +1,63 @@
+"""dmrt_get_run_launch / dmrt_batch_get_run_launch: the kernel that takes a run of steps
+under AUTO, so that a comparison of AUTO with a named kernel compares two kernels."""
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+TMA, CLUSTER, MARCH, BAND = 2, 3, 4, 5
+
+
+@pytest.fixture(scope="module")
+def D():
+    import __graft_entry__
+
+    __graft_entry__.build()
+    from paper_1601_04633_gb300 import dmrt
+
+    return dmrt
+
+
+def plan(D, nx, ny, n, storage=0, **kw):
+    sim = D.Cavity2D(D.make_params(nx, ny, 1e4, 0.01, storage=storage, nu_capacity=16, **kw))
+    r = sim.run_launch(n)
+    sim.close()
+    return r
+
+
+@pytest.mark.parametrize("nx,ny,storage,n,kernel,cluster,launches", [
+    (32, 32, 0, 100, CLUSTER, 1, 2),          # and the Nusselt sum
+    (64, 64, 0, 5, CLUSTER, 1, 2),
+    (64, 64, 0, 2000, BAND, 1, 8),            # four launches and their sums
+    (64, 64, 3, 2000, BAND, 1, 8),
+    (256, 256, 0, 515, BAND, 0, 4),
+    (512, 512, 4, 100, BAND, 0, 2),
+    (1100, 900, 0, 5 * 192 + 30, MARCH, 0, 331),
+    (2048, 2048, 3, 9, MARCH, 0, 4),
+    (2048, 2048, 4, 4, MARCH, 0, 3),          # two pairs of steps
+    (2048, 2048, 0, 2, TMA, 0, 3),
+])
+def test_the_kernel_of_a_run(D, nx, ny, storage, n, kernel, cluster, launches):
+    r = plan(D, nx, ny, n, storage)
+    assert (r["kernel"], r["cluster"], r["launches"]) == (kernel, cluster, launches)
+    assert r["steps"] == n and r["grid"] > 0 and r["block"] > 0
+    assert r["graph_steps"] == (192 if kernel == MARCH and n >= 192 else 0)
+
+
+def test_a_named_kernel_or_tile_takes_one_step_per_launch(D):
+    for kw in ({"kernel": TMA}, {"kernel": TMA, "tma_rows": 2, "tma_npt": 2, "tma_stages": 2}):
+        r = plan(D, 256, 256, 100, **kw)
+        assert (r["kernel"], r["steps_per_launch"], r["launches"], r["graph_steps"]) == (TMA, 1, 101, 64)
+    assert plan(D, 64, 64, 100, kernel=CLUSTER)["kernel"] == CLUSTER
+
+
+def test_batch_runs(D):
+    from paper_1601_04633_gb300 import inputs
+
+    cavs = [inputs.Cavity(100 + 30 * k, 150, 1e4, 0.01) for k in range(5)]
+    for opts, n, want in ((None, 256, (MARCH, 3, 86 + 1)), (None, 5, (MARCH, 2, 2 + 1 + 1 + 1)), (None, 2, (TMA, 1, 3)),
+                          ({"tma_npt": 2, "tma_rows": 2, "tma_stages": 2}, 100, (TMA, 1, 101)),
+                          ({"tma_npt": 2, "tma_rows": 2, "tma_stages": 2, "steps_per_launch": 8}, 100, (TMA, 8, 12 + 4 + 1))):
+        b = D.Batch.from_inputs(cavs, opts=opts, nu_capacity=16)
+        r = b.run_launch(n)
+        assert (r["kernel"], r["steps_per_launch"], r["launches"]) == want
+        b.close()
