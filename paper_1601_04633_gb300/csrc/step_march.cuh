@@ -99,7 +99,7 @@ struct MarchArgs {
     double* prev_rows[kMarchMax];
     int n_strips, n_chunks, chunk;  // items: strip + n_strips * chunk index; rows per chunk
     float sign_l, sign_r;  // -1: fixed-temperature wall (anti-bounce-back), +1: adiabatic
-    float gsh0, gsh1, w0, w1, abb_l, abb_r;  // thermal shifts, rest weights, abb where the wall is fixed, else 0
+    float gsh0, gsh1, w0, w1, abb_l, abb_r;  // thermal shifts, rest weights, abb where the wall is fixed
     double nu_scale;
 };
 
@@ -465,8 +465,9 @@ __device__ __forceinline__ void march_item(const CUtensorMap* ld, const CUtensor
         X.zf0 = X.zf1 = X.zf3 = X.zg0 = X.zg1 = X.zg3 = 0;
         X.wa = X.wadd = 0.f;
     }
-    auto wall_term = [&](int r) {
-        return n.left ? __fmul_rn(M.abb_l, __ldg(A.hot + r)) : n.right ? __fmul_rn(M.abb_r, __ldg(A.cold + r)) : 0.f;
+    auto wall_term = [&](int r) {  // (0 at an adiabatic wall, whatever its profile holds)
+        return n.left && M.sign_l < 0.f ? __fmul_rn(M.abb_l, __ldg(A.hot + r))
+               : n.right && M.sign_r < 0.f ? __fmul_rn(M.abb_r, __ldg(A.cold + r)) : 0.f;
     };
     float nadd = n.wall ? wall_term(rs) : 0.f;  // the next row's wall term
     auto own = [&](F2 v) { return n.right && n.rhi ? f2_hi(v) : f2_lo(v); };
