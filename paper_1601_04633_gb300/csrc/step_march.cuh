@@ -323,8 +323,8 @@ __device__ __forceinline__ void pair_tile(const PairStored<L>& s, unsigned char*
 
 // Sums the rows of steps not yet in the ring (pending = 1: the last step's, local
 // Nusselt numbers; T: those of the T steps of a march launch, as temperatures),
-// in the order of nu_finish_prev; taken: the steps this launch takes (0: the
-// finalize launch). Called by a whole block of kMarchThreads.
+// in the order of nu_finish_prev; taken: the steps this launch takes. Called by a
+// whole block of kMarchThreads.
 __device__ __forceinline__ void march_nu_finish(const MarchArgs& M, int taken) {
     const StepArgs& A = M.A;
     const long long t = __ldcg(A.step_in);
@@ -378,18 +378,68 @@ __device__ __forceinline__ void march_nu_finish(const MarchArgs& M, int taken) {
         }
     }
     if (threadIdx.x == 0) {
-        if (taken > 0) {
-            *A.step_out = t + taken;
-            *A.pending = (unsigned)taken;
-        } else {
-            *A.pending = 0u;
-        }
+        *A.step_out = t + taken;
+        *A.pending = (unsigned)taken;
     }
 }
 
-static __global__ void march_finalize_kernel(MarchArgs M) {
+// The sums of the last march launch alone, after a run: one block of eight warps per
+// step, as nu_finish_prev has them, in the same order; a row's temperatures are
+// turned into its local Nusselt number on the way. (With the four warps of
+// march_nu_finish, which has a launch to hide behind, three steps of 1024^2 in float32 and
+// their sums took 54.5 us; 45.9 with these.)
+constexpr int kMarchSumThreads = 256 * kMarchMax;
+__device__ __forceinline__ void march_nu_sum(const MarchArgs& M) {
+    __shared__ double part[kMarchMax][8][32];
+    const StepArgs& A = M.A;
+    const long long t = __ldcg(A.step_in);
+    const int pend = (int)__ldcg(A.pending);
+    const int lane = threadIdx.x & 31, set = threadIdx.x >> 8, q = (threadIdx.x >> 5) & 7;
+    if (set < pend) {
+        double* rows = M.prev_rows[set];
+        auto local = [&](int r) {
+            if (pend == 1) return __ldcg(rows + r);
+            const float2 th = __ldcg(reinterpret_cast<const float2*>(rows) + r);
+            const double v = M.nu_scale * (8.0 * (double)__ldg(A.hot + r) - 9.0 * (double)th.x + (double)th.y);
+            if (DMRT_IN(r, 0, A.ny, A.err)) rows[r] = v;  // (a row's slot holds both forms)
+            return v;
+        };
+        double acc = 0.0;
+        int r = lane + 32 * q;
+        if (r < A.ny) {  // the partial starts from its first row
+            acc = local(r);
+            r += 256;
+        }
+        for (; r + 3 * 256 < A.ny; r += 4 * 256) {
+            double v[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) v[i] = local(r + 256 * i);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) acc += v[i];
+        }
+        for (; r < A.ny; r += 256) acc += local(r);
+        part[set][q][lane] = acc;
+    }
+    __syncthreads();
+    if (q == 0 && set < pend) {
+        double p8[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) p8[i] = part[set][i][lane];
+        double s = nu_combine(p8, nu_partials(A.ny));
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(kFull, s, o);
+        if (lane == 0) {
+            const double mean = s * A.nu_inv;
+            const long long slot = (t - 1 - set) % A.cap;
+            if (set < A.cap && DMRT_IN(slot, 0, A.cap, A.err)) A.nu_ring[slot] = mean;
+            if (set == 0) *A.nu_last = mean;
+        }
+    }
+    if (threadIdx.x == 0) *A.pending = 0u;  // (every thread has read it: the barrier above)
+}
+static __global__ void __launch_bounds__(kMarchSumThreads) march_finalize_kernel(MarchArgs M) {
     grid_dep_wait();  // (launched while the last step finishes)
-    march_nu_finish(M, 0);
+    march_nu_sum(M);
 }
 
 // What a step needs of the step before it (see the top), the next pull being
@@ -705,8 +755,9 @@ __global__ void __launch_bounds__(kMarchThreads, MINB) batch_march_kernel(const 
 }
 
 // The last launch's Nusselt sums of every cavity, one block each.
-static __global__ void batch_march_finalize_kernel(const __grid_constant__ MarchBatchArgs B) {
-    march_nu_finish(B.M[blockIdx.x], 0);
+static __global__ void __launch_bounds__(kMarchSumThreads)
+    batch_march_finalize_kernel(const __grid_constant__ MarchBatchArgs B) {
+    march_nu_sum(B.M[blockIdx.x]);
 }
 
 // The compiled form for a storage, rounding and steps per launch, its shared memory, and the

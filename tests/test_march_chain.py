@@ -1,0 +1,73 @@
+"""Runs that only the march kernel takes (cavities too wide or too large for the band
+kernel): chains of three-step launches, graphs of them, their Nusselt hand-over and
+every remainder, against the one-step TMA kernel, bit for bit."""
+import os
+import subprocess
+import sys
+
+import numpy as np
+import pytest
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+sys.path.insert(0, ROOT)
+
+pytestmark = pytest.mark.gpu
+
+MARCH = 4
+# Launches from either buffer; 200 and 400: one and two graphs of 192 steps, remainders of
+# 8 = 3 + 2 + 2 + 1 and 16 steps.
+RUNS = (3, 200, 1, 400, 4, 2, 5, 7, 6, 1)
+MODES = [(0, 0), (1, 0), (1, 1), (2, 0), (2, 1), (3, 0), (3, 1), (4, 0), (4, 1)]
+# Whole strips (60 columns in float32, 56 in 16-bit storage), one column more or less, several
+# chunks, few rows, and more than 1024 rows (Nusselt sums of several rows per partial).
+SIZES = [(1080, 43), (1081, 171), (1064, 181), (1063, 90), (777, 701), (241, 1501)]
+
+
+def advance(nx, ny, storage, rounding, kernel, walls=(0, 0), cap=4096, runs=RUNS):
+    from paper_1601_04633_gb300 import dmrt as D
+
+    p = D.make_params(nx, ny, min(1e4, 0.01 * (12 * ny) ** 2), 0.01, storage=storage, rounding=rounding, kernel=kernel,
+                      nu_capacity=cap, left_wall=walls[0], right_wall=walls[1], theta_ref=0.1)
+    rng = np.random.default_rng(nx * 10007 + ny)
+    sim = D.Cavity2D(p, theta0=0.3 * rng.standard_normal((ny, nx)),
+                     theta_hot_profile=0.5 + 0.01 * rng.standard_normal(ny))
+    if kernel == 0:
+        assert all(sim.run_launch(n)["kernel"] == MARCH for n in (200, 400))
+    out = []
+    for n in runs:
+        sim.step(n)
+        mean, rows, _ = sim.nusselt(1)
+        out += [np.array(mean), rows]
+    sim.check()
+    out += [sim.get_state(), sim.nusselt(cap)[2]] + [t.cpu().numpy() for t in sim.fields()]
+    sim.close()
+    return out
+
+
+def assert_same(a, b):
+    for x, y in zip(a, b):
+        np.testing.assert_array_equal(x, y)
+
+
+@pytest.mark.parametrize("storage,rounding", MODES)
+@pytest.mark.parametrize("nx,ny", SIZES)
+def test_march_chain_equals_single_steps(nx, ny, storage, rounding):
+    assert_same(advance(nx, ny, storage, rounding, 0), advance(nx, ny, storage, rounding, 2))
+
+
+@pytest.mark.parametrize("walls", [(1, 0), (0, 1), (1, 1)])
+@pytest.mark.parametrize("storage", [0, 1, 3, 4])
+def test_march_chain_wall_kinds(walls, storage):
+    assert_same(advance(1081, 171, storage, 2, 0, walls), advance(1081, 171, storage, 2, 2, walls))
+
+
+@pytest.mark.parametrize("cap", [1, 2, 3, 5])
+def test_march_chain_short_nusselt_ring(cap):
+    assert_same(advance(1081, 171, 0, 0, 0, cap=cap), advance(1081, 171, 0, 0, 2, cap=cap))
+
+
+def test_march_chain_bounds_checked_build():
+    code = ("import sys; sys.path.insert(0, %r); from tests.test_march_chain import advance;"
+            "[advance(nx, ny, s, 2, 0) for nx, ny in ((1081, 171), (241, 1501)) for s in range(5)]" % ROOT)
+    subprocess.run([sys.executable, "-c", code], check=True, cwd=ROOT,
+                   env=dict(os.environ, DMRT_LIBRARY="bounds_check"))
