@@ -42,7 +42,7 @@ struct Layout {
                           // flow planes, then 5 float32 thermal planes; THETA32: 9
                           // float16 flow planes, a float32 theta plane, 4 float16
                           // deviation planes)
-    size_t off_a, off_b, off_hot, off_cold, off_rows, off_ring, off_misc;
+    size_t off_a, off_b, off_hot, off_cold, off_zero, off_rows, off_ring, off_misc;  // (off_zero: a profile of zeros)
     size_t off_mail, off_record;  // band kernel: messages, theta at x = 0, 1 by step (0: none)
     size_t total;
 };
@@ -97,6 +97,7 @@ Layout make_layout(const dmrt_params& p, int halo_rows = 0, bool band = false) {
     L.off_b = o; o += L.buf_bytes;
     L.off_hot = o; o += align256((size_t)p.ny * sizeof(float));
     L.off_cold = o; o += align256((size_t)p.ny * sizeof(float));
+    L.off_zero = o; o += align256((size_t)p.ny * sizeof(float));
     L.off_rows = o; o += align256((size_t)2 * dmrt::kMarchMax * p.ny * sizeof(double));  // by source buffer; march launches: each of their steps
     L.off_ring = o; o += align256((size_t)p.nu_capacity * sizeof(double));
     L.off_misc = o; o += 256;
@@ -1114,6 +1115,9 @@ dmrt::MarchArgs march_args(dmrt_ctx* c, int from, int steps) {
     M.w1 = c->sc.w1;
     M.abb_l = c->sc.left_fixed ? c->sc.abb : 0.f;
     M.abb_r = c->sc.right_fixed ? c->sc.abb : 0.f;
+    const float* zero = reinterpret_cast<const float*>(c->ws + c->L.off_zero);
+    M.wall_l = c->sc.left_fixed ? M.A.hot : zero;
+    M.wall_r = c->sc.right_fixed ? M.A.cold : zero;
     M.nu_scale = c->sc.nu_scale;
     return M;
 }

@@ -378,14 +378,11 @@ __global__ void __launch_bounds__(MAXT) step_band_kernel(const __grid_constant__
             v1[0] = own(3, 0);
             v5[0] = own(7, 0);
             v8[0] = own(6, 0);
-            // (no term at an adiabatic wall, whatever its profile holds)
-            const float add = M.sign_l < 0.f ? __fmul_rn(M.abb_l, __ldg(A.hot + j)) : 0.f;
-            w1[0] = wall_value(M.sign_l, own(12, 0), add);
+            w1[0] = wall_value(M.sign_l, own(12, 0), __fmul_rn(M.abb_l, __ldg(M.wall_l + j)));
         }
         if (n.right) {
             const int e = n.rhi ? 1 : 0;
-            const float add = M.sign_r < 0.f ? __fmul_rn(M.abb_r, __ldg(A.cold + j)) : 0.f;
-            const float wall = wall_value(M.sign_r, own(10, e), add);
+            const float wall = wall_value(M.sign_r, own(10, e), __fmul_rn(M.abb_r, __ldg(M.wall_r + j)));
 #pragma unroll
             for (int i = 0; i < 2; ++i) {
                 if (i == e) v3[i] = own(1, e), v6[i] = own(8, e), v7[i] = own(5, e), w3[i] = wall;

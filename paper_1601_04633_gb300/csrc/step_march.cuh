@@ -99,7 +99,8 @@ struct MarchArgs {
     double* prev_rows[kMarchMax];
     int n_strips, n_chunks, chunk;  // items: strip + n_strips * chunk index; rows per chunk
     float sign_l, sign_r;  // -1: fixed-temperature wall (anti-bounce-back), +1: adiabatic
-    float gsh0, gsh1, w0, w1, abb_l, abb_r;  // thermal shifts, rest weights, abb where the wall is fixed
+    float gsh0, gsh1, w0, w1, abb_l, abb_r;  // thermal shifts, rest weights, abb where the wall is fixed, else 0
+    const float *wall_l, *wall_r;            // the walls' temperatures; zeros at an adiabatic wall (its profile is not read)
     double nu_scale;
 };
 
@@ -505,7 +506,6 @@ __device__ __forceinline__ void march_item(const CUtensorMap* ld, const CUtensor
         for (int row = lb; row < issued; ++row) issue(row);
     bool ok = true;
     int waited = lb;  // rows below this one have arrived (!ok: those below waited - 1)
-    for (; waited <= rs && ok; ++waited) ok = arrived(waited);
 
     MarchCarry C[T - 1];
 #pragma unroll
@@ -515,9 +515,8 @@ __device__ __forceinline__ void march_item(const CUtensorMap* ld, const CUtensor
         X.zf0 = X.zf1 = X.zf3 = X.zg0 = X.zg1 = X.zg3 = 0;
         X.wa = X.wadd = 0.f;
     }
-    auto wall_term = [&](int r) {  // (0 at an adiabatic wall, whatever its profile holds)
-        return n.left && M.sign_l < 0.f ? __fmul_rn(M.abb_l, __ldg(A.hot + r))
-               : n.right && M.sign_r < 0.f ? __fmul_rn(M.abb_r, __ldg(A.cold + r)) : 0.f;
+    auto wall_term = [&](int r) {
+        return n.left ? __fmul_rn(M.abb_l, __ldg(M.wall_l + r)) : n.right ? __fmul_rn(M.abb_r, __ldg(M.wall_r + r)) : 0.f;
     };
     float nadd = n.wall ? wall_term(rs) : 0.f;  // the next row's wall term
     auto own = [&](F2 v) { return n.right && n.rhi ? f2_hi(v) : f2_lo(v); };
@@ -537,12 +536,10 @@ __device__ __forceinline__ void march_item(const CUtensorMap* ld, const CUtensor
     // unrolling the loop, in instruction fetches.)
     const int last = min(rend, A.ny - 1);
 #pragma unroll 1
-    for (int r = ok ? rs : rend + 1; r <= rend; ++r) {  // (no row when the first ones did not arrive)
-        if (waited <= ub) {
-            ok = arrived(waited);
-            ++waited;
-            if (!ok) break;
-        }
+    for (int r = rs; r <= rend; ++r) {
+        // Rows up to r + 1 have arrived (the first iteration waits for all from lb on).
+        for (; ok && waited <= min(r + 1, ub); ++waited) ok = arrived(waited);
+        if (!ok) break;
         F2 f[9], g[5], rho, theta;
         float add = nadd;
         // Step 0 from the stages.
