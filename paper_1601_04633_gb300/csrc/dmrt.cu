@@ -42,7 +42,7 @@ struct Layout {
                           // flow planes, then 5 float32 thermal planes; THETA32: 9
                           // float16 flow planes, a float32 theta plane, 4 float16
                           // deviation planes)
-    size_t off_a, off_b, off_hot, off_cold, off_zero, off_rows, off_ring, off_misc;  // (off_zero: a profile of zeros)
+    size_t off_a, off_b, off_hot, off_cold, off_zero, off_rows, off_part, off_ring, off_misc;  // (off_zero: a profile of zeros)
     size_t off_mail, off_record;  // band kernel: messages, theta at x = 0, 1 by step (0: none)
     size_t total;
 };
@@ -99,6 +99,7 @@ Layout make_layout(const dmrt_params& p, int halo_rows = 0, bool band = false) {
     L.off_cold = o; o += align256((size_t)p.ny * sizeof(float));
     L.off_zero = o; o += align256((size_t)p.ny * sizeof(float));
     L.off_rows = o; o += align256((size_t)2 * dmrt::kMarchMax * p.ny * sizeof(double));  // by source buffer; march launches: each of their steps
+    L.off_part = o; o += sizeof(dmrt::MarchPart) * dmrt::kMarchMax;
     L.off_ring = o; o += align256((size_t)p.nu_capacity * sizeof(double));
     L.off_misc = o; o += 256;
     L.off_mail = L.off_record = 0;
@@ -118,8 +119,9 @@ struct Misc {
     long long step[2];   // steps recorded in the Nu ring; slot b is current when the
                          // state is in buffer b (a launch reads one slot, writes the other)
     double nu_last;      // mean Nu of the latest step
-    unsigned pending;    // the last step's local Nu rows are not yet summed into the ring
+    unsigned pending;    // steps of the last launch whose local Nu rows are not yet summed into the ring
     unsigned err;        // error bits
+    unsigned nu_arrivals;  // march launches: blocks that have summed their share of the rows
 };
 // The band kernel's scalars (second half of the block; kept when a checkpoint is loaded).
 struct BandScalars {
@@ -1090,9 +1092,12 @@ int setup_band(dmrt_ctx* c) {
     return DMRT_OK;
 }
 
+// Blocks that sum the Nusselt rows of a launch of ny rows (see march_nu_finish).
+int march_nu_blocks(int ny) { return std::min(dmrt::kMarchSumBlocks, std::max(1, ny / 512)); }
+
 int march_grid(const dmrt_ctx* c, int steps) {
     const int per = dmrt::kMarchThreads / 32;
-    return (c->mstrips * c->mchunks[steps] + per - 1) / per + 1;  // the last block sums Nusselt rows
+    return (c->mstrips * c->mchunks[steps] + per - 1) / per + march_nu_blocks(c->p.ny);  // (the last ones sum)
 }
 
 // Arguments of a march launch of `steps` steps from buffer `from` (the finalize launch takes any).
@@ -1119,6 +1124,9 @@ dmrt::MarchArgs march_args(dmrt_ctx* c, int from, int steps) {
     M.wall_l = c->sc.left_fixed ? M.A.hot : zero;
     M.wall_r = c->sc.right_fixed ? M.A.cold : zero;
     M.nu_scale = c->sc.nu_scale;
+    M.nu_part = reinterpret_cast<dmrt::MarchPart*>(c->ws + c->L.off_part);
+    M.nu_arrivals = &misc(c)->nu_arrivals;
+    M.nu_blocks = march_nu_blocks(c->p.ny);
     return M;
 }
 
@@ -1547,7 +1555,7 @@ static int finalize_nu(dmrt_ctx* c) {
     const int open = c->nu_open;
     c->nu_open = 0;
     if (open > 1) {
-        CK(launch_overlapped(dmrt::march_finalize_kernel, dim3(1), dim3(dmrt::kMarchSumThreads), c->stream,
+        CK(launch_overlapped(dmrt::march_finalize_kernel, dim3(march_nu_blocks(c->p.ny)), dim3(dmrt::kMarchSumThreads), c->stream,
                              march_args(c, c->cur, 2)),
            "step launch");
         return DMRT_OK;
@@ -2722,6 +2730,8 @@ int batch_setup_march(dmrt_batch* b, CUtensorMap* d_maps, int sms) {
             for (int i = first; i < first + count; ++i)
                 cav.emplace_back(b->sub[i]->p.ny, (b->sub[i]->p.nx + F[t].cols - 1) / F[t].cols);
             const int chunk = march_chunk(cav, t, sms, per_sm);
+            int tall = 0;
+            for (const auto& cv : cav) tall = std::max(tall, cv.first);
             for (int bf = 0; bf < 2; ++bf) {
                 dmrt::MarchBatchArgs B;
                 std::memset((void*)&B, 0, sizeof B);
@@ -2729,10 +2739,12 @@ int batch_setup_march(dmrt_batch* b, CUtensorMap* d_maps, int sms) {
                 B.err = b->d_err;
                 B.n = dmrt::make_pair_numbers();
                 B.n_cav = count;
+                B.nu_blocks = march_nu_blocks(tall);
                 for (int i = 0; i < count; ++i) {
                     dmrt_ctx* c = b->sub[first + i];
                     dmrt::MarchArgs& M = B.M[i];
                     M = march_args(c, bf, t);
+                    M.nu_blocks = B.nu_blocks;
                     M.n_strips = cav[i].second;
                     M.chunk = std::min(chunk, c->p.ny);
                     M.n_chunks = (c->p.ny + M.chunk - 1) / M.chunk;
@@ -3054,13 +3066,13 @@ int dmrt_batch_create(const dmrt_params* arr, int32_t n, const double* const* th
 static int batch_march(dmrt_batch* b, int n, int parity) {
     for (dmrt::MarchBatchArgs& B : b->margs[n > 0 ? n : 3][parity]) {
         if (n == 0) {
-            dmrt::batch_march_finalize_kernel<<<B.n_cav, dmrt::kMarchSumThreads, 0, b->stream>>>(B);
+            dmrt::batch_march_finalize_kernel<<<B.n_cav * B.nu_blocks, dmrt::kMarchSumThreads, 0, b->stream>>>(B);
             BCK(cudaGetLastError(), "batch Nusselt launch");
             continue;
         }
         const int per = dmrt::kMarchThreads / 32;
         void* params[1] = {&B};
-        BCK(launch_overlapped(b->march[n], dim3((B.items + per - 1) / per + B.n_cav), dim3(dmrt::kMarchThreads), b->msmem,
+        BCK(launch_overlapped(b->march[n], dim3((B.items + per - 1) / per + B.n_cav * B.nu_blocks), dim3(dmrt::kMarchThreads), b->msmem,
                               b->stream, params),
             "batch march launch");
     }
@@ -3184,7 +3196,7 @@ int dmrt_batch_get_run_launch(const dmrt_batch* b, int64_t nsteps, dmrt_run_laun
         out->steps = nsteps - left;
         out->launches = (launches + 1) * parts + (left > 0 ? left + 1 : 0);  // (march: one group)
         out->rows = B.M[0].chunk;
-        out->grid = (B.items + dmrt::kMarchThreads / 32 - 1) / (dmrt::kMarchThreads / 32) + B.n_cav;
+        out->grid = (B.items + dmrt::kMarchThreads / 32 - 1) / (dmrt::kMarchThreads / 32) + B.n_cav * B.nu_blocks;
         out->block = dmrt::kMarchThreads;
         out->smem_bytes = (int64_t)b->msmem;
         return DMRT_OK;

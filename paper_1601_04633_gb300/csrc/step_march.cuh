@@ -102,6 +102,9 @@ struct MarchArgs {
     float gsh0, gsh1, w0, w1, abb_l, abb_r;  // thermal shifts, rest weights, abb where the wall is fixed, else 0
     const float *wall_l, *wall_r;            // the walls' temperatures; zeros at an adiabatic wall (its profile is not read)
     double nu_scale;
+    double (*nu_part)[8][32];  // [kMarchMax] partial sums of rows, when nu_blocks > 1
+    unsigned* nu_arrivals;     // blocks of this launch that have written theirs (0 between launches)
+    int nu_blocks;             // blocks that sum the rows of the launch before
 };
 
 // ---- storage forms --------------------------------------------------------------
@@ -323,50 +326,71 @@ __device__ __forceinline__ void pair_tile(const PairStored<L>& s, unsigned char*
 }
 
 // Sums the rows of steps not yet in the ring (pending = 1: the last step's, local
-// Nusselt numbers; T: those of the T steps of a march launch, as temperatures),
-// in the order of nu_finish_prev; taken: the steps this launch takes. Called by a
-// whole block of kMarchThreads.
-__device__ __forceinline__ void march_nu_finish(const MarchArgs& M, int taken) {
+// Nusselt numbers; T: those of the T steps of a march launch, as temperatures, each
+// turned into its local number on the way), in the order of nu_finish_prev; taken:
+// the steps this launch takes (0: the finalize launch). Called by all of block
+// `block` of the M.nu_blocks that share the partial streams; the last of them to
+// arrive adds these up.
+//
+// A row's number takes five float64 operations, and float64 is a slow pipe here, so for
+// tall cavities one block would be longer than the launch around it (200 x 20000 mixed,
+// 192 steps: 17.1 ms with one block, 9.1 with eight; 27.2 with one block, a pass of its
+// own for the numbers and then one warp per step): one block per 512 rows, up to eight
+// (march_args). U: rows of a stream in flight per lane, two in the single-cavity
+// launches (four cost 2048^2 in float32, whose registers are at their limit, 4 %), one in
+// the batched ones (two cost 64 cavities 2 %), four in the finalize launches.
+constexpr int kMarchSumThreads = 256 * kMarchMax;  // of the finalize launch
+constexpr int kMarchSumBlocks = 8;
+using MarchPart = double[8][32];                   // [kMarchMax] in shared memory
+template <int U>
+__device__ __forceinline__ void march_nu_finish(const MarchArgs& M, int taken, MarchPart* shared_part, int block) {
     const StepArgs& A = M.A;
     const long long t = __ldcg(A.step_in);
-    const int pend = (int)__ldcg(A.pending);
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    __syncthreads();  // every thread has read the flag before it is rewritten
-    if (pend > 1) {
-        for (int i = threadIdx.x; i < pend * A.ny; i += kMarchThreads) {
-            const int which = i / A.ny, r = i - which * A.ny;
-            if (!DMRT_IN(which, 0, kMarchMax, A.err) || !DMRT_IN(r, 0, A.ny, A.err)) continue;
-            double* rows = M.prev_rows[which];
+    const int pend = min((int)__ldcg(A.pending), kMarchMax);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
+    const int nq = nu_partials(A.ny);
+    MarchPart* const part = M.nu_blocks > 1 ? M.nu_part : shared_part;
+    for (int task = block * warps + warp; task < nq * pend; task += M.nu_blocks * warps) {
+        const int set = task / nq, q = task - set * nq;
+        double* rows = M.prev_rows[set];
+        auto local = [&](int r) {
+            if (pend == 1) return __ldcg(rows + r);
             const float2 th = __ldcg(reinterpret_cast<const float2*>(rows) + r);
             const double tw = (double)__ldg(A.hot + r);
-            rows[r] = M.nu_scale * (8.0 * tw - 9.0 * (double)th.x + (double)th.y);
+            return M.nu_scale * (8.0 * tw - 9.0 * (double)th.x + (double)th.y);
+        };
+        auto keep = [&](int r, double v) {  // (a row's slot holds both forms)
+            if (pend > 1 && DMRT_IN(r, 0, A.ny, A.err)) rows[r] = v;
+        };
+        double acc = 0.0;
+        int r = lane + 32 * q;
+        if (r < A.ny) {  // the partial starts from its first row
+            acc = local(r);
+            keep(r, acc);
+            r += 256;
         }
-        __syncthreads();  // (writes of this block, read by it below)
+#pragma unroll U
+        for (; r < A.ny; r += 256) {
+            const double v = local(r);
+            acc += v;
+            keep(r, v);
+        }
+        part[set][q][lane] = acc;
     }
-    if (warp < pend && warp < kMarchMax) {
-        const double* rows = M.prev_rows[warp];
+    // (every thread has read the counters before the last block rewrites them)
+    if (M.nu_blocks > 1) {
+        __threadfence();
+        __syncthreads();
+        const bool more = threadIdx.x == 0 && atomicInc(M.nu_arrivals, M.nu_blocks - 1) != M.nu_blocks - 1u;
+        if (__syncthreads_or(more)) return;
+        __threadfence();
+    } else {
+        __syncthreads();
+    }
+    if (warp < pend) {
         double p8[8];
-        const int nq = nu_partials(A.ny);
 #pragma unroll
-        for (int q = 0; q < 8; ++q) {
-            p8[q] = 0.0;
-            if (q >= nq) continue;
-            int r = lane + 32 * q;
-            double acc = 0.0;
-            if (r < A.ny) {
-                acc = __ldcg(rows + r);
-                r += 256;
-            }
-            for (; r + 3 * 256 < A.ny; r += 4 * 256) {
-                double v[4];
-#pragma unroll
-                for (int i = 0; i < 4; ++i) v[i] = __ldcg(rows + r + 256 * i);
-#pragma unroll
-                for (int i = 0; i < 4; ++i) acc += v[i];
-            }
-            for (; r < A.ny; r += 256) acc += __ldcg(rows + r);
-            p8[q] = acc;
-        }
+        for (int q = 0; q < 8; ++q) p8[q] = *(volatile double*)&part[warp][q][lane];  // (those past nq are left out)
         double s = nu_combine(p8, nq);
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(kFull, s, o);
@@ -379,68 +403,17 @@ __device__ __forceinline__ void march_nu_finish(const MarchArgs& M, int taken) {
         }
     }
     if (threadIdx.x == 0) {
-        *A.step_out = t + taken;
+        if (taken > 0) *A.step_out = t + taken;
         *A.pending = (unsigned)taken;
     }
 }
 
-// The sums of the last march launch alone, after a run: one block of eight warps per
-// step, as nu_finish_prev has them, in the same order; a row's temperatures are
-// turned into its local Nusselt number on the way. (With the four warps of
-// march_nu_finish, which has a launch to hide behind, three steps of 1024^2 in float32 and
-// their sums took 54.5 us; 45.9 with these.)
-constexpr int kMarchSumThreads = 256 * kMarchMax;
-__device__ __forceinline__ void march_nu_sum(const MarchArgs& M) {
-    __shared__ double part[kMarchMax][8][32];
-    const StepArgs& A = M.A;
-    const long long t = __ldcg(A.step_in);
-    const int pend = (int)__ldcg(A.pending);
-    const int lane = threadIdx.x & 31, set = threadIdx.x >> 8, q = (threadIdx.x >> 5) & 7;
-    if (set < pend) {
-        double* rows = M.prev_rows[set];
-        auto local = [&](int r) {
-            if (pend == 1) return __ldcg(rows + r);
-            const float2 th = __ldcg(reinterpret_cast<const float2*>(rows) + r);
-            const double v = M.nu_scale * (8.0 * (double)__ldg(A.hot + r) - 9.0 * (double)th.x + (double)th.y);
-            if (DMRT_IN(r, 0, A.ny, A.err)) rows[r] = v;  // (a row's slot holds both forms)
-            return v;
-        };
-        double acc = 0.0;
-        int r = lane + 32 * q;
-        if (r < A.ny) {  // the partial starts from its first row
-            acc = local(r);
-            r += 256;
-        }
-        for (; r + 3 * 256 < A.ny; r += 4 * 256) {
-            double v[4];
-#pragma unroll
-            for (int i = 0; i < 4; ++i) v[i] = local(r + 256 * i);
-#pragma unroll
-            for (int i = 0; i < 4; ++i) acc += v[i];
-        }
-        for (; r < A.ny; r += 256) acc += local(r);
-        part[set][q][lane] = acc;
-    }
-    __syncthreads();
-    if (q == 0 && set < pend) {
-        double p8[8];
-#pragma unroll
-        for (int i = 0; i < 8; ++i) p8[i] = part[set][i][lane];
-        double s = nu_combine(p8, nu_partials(A.ny));
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(kFull, s, o);
-        if (lane == 0) {
-            const double mean = s * A.nu_inv;
-            const long long slot = (t - 1 - set) % A.cap;
-            if (set < A.cap && DMRT_IN(slot, 0, A.cap, A.err)) A.nu_ring[slot] = mean;
-            if (set == 0) *A.nu_last = mean;
-        }
-    }
-    if (threadIdx.x == 0) *A.pending = 0u;  // (every thread has read it: the barrier above)
-}
+// The last launch's sums alone, after a run: M.nu_blocks blocks. (Three steps of 1024^2 in
+// float32 with their sums: 45.9 us; 54.5 by one block of four warps.)
 static __global__ void __launch_bounds__(kMarchSumThreads) march_finalize_kernel(MarchArgs M) {
+    __shared__ MarchPart part[kMarchMax];
     grid_dep_wait();  // (launched while the last step finishes)
-    march_nu_sum(M);
+    march_nu_finish<4>(M, 0, part, blockIdx.x);
 }
 
 // What a step needs of the step before it (see the top), the next pull being
@@ -696,8 +669,9 @@ __global__ void __launch_bounds__(kMarchThreads, MINB)
     grid_dep_launch();
     // After an expired wait in an earlier launch the state is invalid: return at once.
     if (__syncthreads_or(threadIdx.x == 0 && (*reinterpret_cast<volatile unsigned*>(M.A.err) & kErrTimeout))) return;
-    if (blockIdx.x == gridDim.x - 1) {  // the extra block: the previous launch's Nusselt sums
-        march_nu_finish(M, T);
+    const int extra = (int)blockIdx.x - ((int)gridDim.x - M.nu_blocks);
+    if (extra >= 0) {  // the last blocks: the previous launch's Nusselt sums (they have no rows)
+        march_nu_finish<2>(M, T, reinterpret_cast<MarchPart*>(smem_m), extra);
         return;
     }
     const int item = blockIdx.x * (kMarchThreads / 32) + warp;
@@ -710,13 +684,14 @@ __global__ void __launch_bounds__(kMarchThreads, MINB)
 // cavity. The cavities' arguments and rates are kernel parameters, so that a
 // warp takes them from the constant bank at its cavity's (uniform) index, as
 // the single-cavity kernel does; the tensor maps lie in global memory. The last
-// n_cav blocks take the cavities' Nusselt sums.
+// n_cav nu_blocks blocks take the cavities' Nusselt sums.
 constexpr int kMarchBatch = 64;
 struct MarchBatchArgs {
     const CUtensorMap* maps;  // [n_cav][6]: loads, stores of this launch's source buffer
     unsigned* err;            // the batch's error word (an expired wait)
     PairNumbers n;
     int n_cav, items;
+    int nu_blocks;            // of each cavity
     int first[kMarchBatch];   // first item of each cavity
     MarchArgs M[kMarchBatch];
     PairRates r[kMarchBatch];
@@ -733,9 +708,10 @@ __global__ void __launch_bounds__(kMarchThreads, MINB) batch_march_kernel(const 
     grid_dep_wait();
     grid_dep_launch();
     if (__syncthreads_or(threadIdx.x == 0 && (*reinterpret_cast<volatile unsigned*>(B.err) & kErrTimeout))) return;
-    const int extra = (int)blockIdx.x - ((int)gridDim.x - B.n_cav);
+    const int extra = (int)blockIdx.x - ((int)gridDim.x - B.n_cav * B.nu_blocks);
     if (extra >= 0) {
-        march_nu_finish(B.M[extra], T);
+        const int cav = extra / B.nu_blocks;
+        march_nu_finish<1>(B.M[cav], T, reinterpret_cast<MarchPart*>(smem_m), extra - cav * B.nu_blocks);
         return;
     }
     const int item = blockIdx.x * (kMarchThreads / 32) + warp;
@@ -751,10 +727,12 @@ __global__ void __launch_bounds__(kMarchThreads, MINB) batch_march_kernel(const 
     if (lane == 0 && (*reinterpret_cast<volatile unsigned*>(B.M[lo].A.err) & kErrTimeout)) atomicOr(B.err, kErrTimeout);
 }
 
-// The last launch's Nusselt sums of every cavity, one block each.
+// The last launch's Nusselt sums of every cavity, nu_blocks blocks each.
 static __global__ void __launch_bounds__(kMarchSumThreads)
     batch_march_finalize_kernel(const __grid_constant__ MarchBatchArgs B) {
-    march_nu_sum(B.M[blockIdx.x]);
+    __shared__ MarchPart part[kMarchMax];
+    const int cav = blockIdx.x / B.nu_blocks;
+    march_nu_finish<4>(B.M[cav], 0, part, blockIdx.x - cav * B.nu_blocks);
 }
 
 // The compiled form for a storage, rounding and steps per launch, its shared memory, and the

@@ -55,6 +55,34 @@ def test_march_chain_equals_single_steps(nx, ny, storage, rounding):
     assert_same(advance(nx, ny, storage, rounding, 0), advance(nx, ny, storage, rounding, 2))
 
 
+@pytest.mark.parametrize("storage,rounding", [(0, 0), (1, 1), (3, 1)])
+@pytest.mark.parametrize("nx,ny", [(167, 4100), (300, 1024), (300, 1023)])
+def test_march_chain_tall_cavities(nx, ny, storage, rounding):
+    """Nusselt sums by one, two and eight blocks."""
+    assert_same(advance(nx, ny, storage, rounding, 0), advance(nx, ny, storage, rounding, 2))
+
+
+@pytest.mark.parametrize("storage,rounding", [(0, 0), (3, 1)])
+def test_march_chain_of_a_batch_with_a_tall_member(storage, rounding):
+    from paper_1601_04633_gb300 import dmrt as D
+    from paper_1601_04633_gb300 import inputs
+
+    cavs = [inputs.Cavity(nx, ny, min(1e4, 0.01 * (12 * ny) ** 2), 0.01, noise_amp=1e-2, seed=k)
+            for k, (nx, ny) in enumerate(((60, 2100), (130, 19), (57, 300), (8, 8)))]
+    b = D.Batch.from_inputs(cavs, nu_capacity=512, storage=storage, rounding=rounding)
+    assert b.run_launch(30)["kernel"] == MARCH
+    for n in (30, 1, 4, 5, 7, 64):
+        b.step(n)
+    b.check()
+    for m, c in zip(b.members, cavs):
+        ref = D.Cavity2D.from_inputs(c, nu_capacity=512, storage=storage, rounding=rounding, kernel=2)
+        ref.step(111)
+        got, want = m.nusselt(512), ref.nusselt(512)
+        assert_same([m.get_state(), got[1], got[2]], [ref.get_state(), want[1], want[2]])
+        ref.close()
+    b.close()
+
+
 @pytest.mark.parametrize("walls", [(1, 0), (0, 1), (1, 1)])
 @pytest.mark.parametrize("storage", [0, 1, 3, 4])
 def test_march_chain_wall_kinds(walls, storage):
