@@ -1093,7 +1093,7 @@ int setup_band(dmrt_ctx* c) {
 }
 
 // Blocks that sum the Nusselt rows of a launch of ny rows (see march_nu_finish).
-int march_nu_blocks(int ny) { return std::min(dmrt::kMarchSumBlocks, std::max(1, ny / 512)); }
+int march_nu_blocks(int ny) { return std::min(dmrt::kMarchSumBlocks, std::max(1, ny / 256)); }
 
 int march_grid(const dmrt_ctx* c, int steps) {
     const int per = dmrt::kMarchThreads / 32;

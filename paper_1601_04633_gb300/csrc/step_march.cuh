@@ -350,7 +350,7 @@ __device__ __forceinline__ void march_nu_finish(const MarchArgs& M, int taken, M
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
     const int nq = nu_partials(A.ny);
     MarchPart* const part = M.nu_blocks > 1 ? M.nu_part : shared_part;
-    for (int task = block * warps + warp; task < nq * pend; task += M.nu_blocks * warps) {
+    for (int task = warp * M.nu_blocks + block; task < nq * pend; task += M.nu_blocks * warps) {
         const int set = task / nq, q = task - set * nq;
         double* rows = M.prev_rows[set];
         auto local = [&](int r) {
