@@ -910,21 +910,22 @@ int setup_kernel(dmrt_ctx* c) {
     return DMRT_OK;
 }
 
-// Runs of steps on the march kernel (step_march.cuh): three steps per launch,
-// two where three would leave a single step.
+// Runs of steps on the march kernel (step_march.cuh): three steps per launch.
 //
-// AUTO takes it for whole cavities of at least 40000 nodes and 160 columns (runs
-// too short for, or cavities too large for, the band kernel). Microseconds per step, march / one launch per step, on one GB300:
-// float32 192^2 3.4 / 3.1, 256^2 3.4 / 4.2, 512^2 6.1 / 9.5, 1024^2 12.7 / 22.7,
-// 2048^2 34.6 / 78.0, 4096^2 118 / 288; mixed, stochastic 128^2 3.7 / 3.0, 256^2
-// 3.7 / 4.4, 1024^2 14.6 / 20.0, 4096^2 145 / 212; THETA32, stochastic 1024^2
-// 15.9 / 18.1, 1999 x 1531 35.7 / 43.6; float16, stochastic 2048^2 45.9 / 51.6.
-// (Two steps per launch: 163 us at 4096^2 in float32, bound by HBM; three are
-// bound by the float32 pipe, 65 % busy, and by the tail of a launch.)
-//
-// Narrow cavities leave a strip's lanes idle (100 x 500: 4.3 against 3.9).
-constexpr long long kMarchNodes = 40000;
-constexpr int kMarchWidth = 160;
+// AUTO takes it for whole cavities of at least 160 columns that the band kernel does not
+// hold (or for runs too short for it), from these many nodes on: float32 40000, mixed
+// 600000, the other storages a million; all 16-bit storages 400000 up to 500 columns.
+// Microseconds per step over 192 steps, march / one launch per step, on one GB300:
+// float32 1100 x 40 2.9 / 4.4, 700 x 500 6.3 / 9.6, 1024^2 11.9 / 22.2, 2048^2 33 / 77,
+// 4096^2 115 / 289; mixed, stochastic 800 x 700 9.6 / 12.0, 1024^2 14.0 / 19.3, 2048^2
+// 41 / 55; THETA32, stochastic 2048^2 46 / 55; float16, stochastic 1024^2 15.1 / 16.3,
+// 2048^2 45 / 50, 230 x 4000 15.4 / 17.4, 165 x 3000 9.5 / 13.4. Below these sizes the two are near
+// each other in 16-bit storage, in either order (700 x 500 mixed 7.8 / 7.4; 5000 x 90
+// float16 9.0 / 8.8, THETA32 9.3 / 8.9, 3000 x 267 float16 12.9 / 12.0), so they keep one launch per step.
+// (Two steps per launch: 163 us at 4096^2 in float32.)
+constexpr long long kMarchNodes = 40000, kMarchNodesMixed = 600000, kMarchNodes16 = 1000000, kMarchNodes16Tall = 400000;
+constexpr int kMarchTall = 500;   // the widest of the last
+constexpr int kMarchWidth = 160;  // (not measured below, where the band kernel does not reach)
 
 // The march launches' tensor maps of c, by source buffer.
 int march_maps(dmrt_ctx* c, const dmrt::MarchForm& F, dmrt::MarchMaps* maps) {
@@ -988,7 +989,9 @@ int setup_march(dmrt_ctx* c) {
     std::memset(c->march, 0, sizeof c->march);
     if (c->cluster || c->slab || p.kernel != DMRT_KERNEL_AUTO || p.tma_npt > 0 || p.tma_rows > 0 || p.tma_stages > 0)
         return DMRT_OK;
-    if (p.nx < kMarchWidth || (long long)p.nx * p.ny < kMarchNodes) return DMRT_OK;
+    const long long least = p.storage == DMRT_FP32 ? kMarchNodes : p.nx <= kMarchTall ? kMarchNodes16Tall
+                            : p.storage == DMRT_MIXED ? kMarchNodesMixed : kMarchNodes16;
+    if (p.nx < kMarchWidth || (long long)p.nx * p.ny < least) return DMRT_OK;
     const dmrt::MarchForm F2 = dmrt::march_form(p.storage, p.rounding, 2), F = dmrt::march_form(p.storage, p.rounding, 3);
     int dev = 0, sms = 0, per_sm = 0;
     CK(cudaGetDevice(&dev), "cudaGetDevice");
@@ -1487,14 +1490,27 @@ static cudaError_t add_step_node(cudaGraph_t g, cudaGraphNode_t prev, const cuda
     return e;
 }
 
-// Steps of the next launch in a run of n steps. A march launch of three steps
+// Steps of the next launch in a run with n steps to go. A march launch of three steps
 // changes buffers once, as three single launches would; two steps go in a
 // launch only in pairs, so that a run of n steps always ends in the buffer that
 // n single steps would end in (a batch's members, and replays of captured
 // runs, rely on it).
-static int launch_steps(const dmrt_ctx* c, int64_t n) {
+//
+// What three-step launches leave goes in two-step ones in float32 and in single steps
+// in 16-bit storage, whose two-step launches gain nothing (1500 x 100 mixed, 8 steps:
+// 56.5 us with them, 44.5 without). The sums at the end of a march launch cost more than
+// those of a single step, so float16 and bfloat16, whose gain is small, begin with a march
+// launch from kMarchMin16 steps on (1100 x 512 float16: 5 steps 60.6 us, 58.8 in single
+// steps; 6 steps 66.4 and 70.4), and THETA32 below kMarchShort nodes as well (2000 x 501: 5
+// steps 4 % more, 6 the same). marched: the run's last launch was the march kernel's.
+constexpr int kMarchMin16 = 6;
+constexpr long long kMarchShort = 1200000;
+static int launch_steps(const dmrt_ctx* c, int64_t n, bool marched) {
     if (!c->march[2] || n < 3) return 1;
-    return n == 4 || n == 5 ? 2 : 3;
+    if (c->p.storage == DMRT_FP32) return n == 4 || n == 5 ? 2 : 3;
+    const bool any = c->p.storage == DMRT_MIXED ||
+                     (c->p.storage == DMRT_THETA32 && (long long)c->p.nx * c->p.ny >= kMarchShort);
+    return marched || any || n >= kMarchMin16 ? 3 : 1;
 }
 // Steps of a whole graph: graph_len launches.
 static int graph_steps(const dmrt_ctx* c) { return c->graph_len * (c->march[2] ? 3 : 1); }
@@ -1702,13 +1718,14 @@ static int launch_band(dmrt_ctx* c, int n, float* record = nullptr, long long st
 
 // The next launch of a run with `left` steps to go (the rules that pick the kernel of a
 // run): its kernel and its steps. to_poll: steps until the next divergence poll;
-// pair: half of a pair of two-step march launches is done.
+// marched: the run's last launch was the march kernel's; pair: half of a pair of
+// two-step march launches is done.
 enum RunKind { kRunOne, kRunCluster, kRunMarch, kRunGraph, kRunBand };
 struct RunLaunch {
     RunKind kind;
     int n;
 };
-static RunLaunch next_launch(const dmrt_ctx* c, int64_t left, int64_t to_poll, bool pair) {
+static RunLaunch next_launch(const dmrt_ctx* c, int64_t left, int64_t to_poll, bool marched, bool pair) {
     if (c->band && left >= dmrt::kBandMinSteps) {
         // Up to the next divergence poll, with no remainder too short for a launch of its own.
         long long n = std::min<long long>(left, std::max<long long>(dmrt::kBandMinSteps, to_poll));
@@ -1722,7 +1739,7 @@ static RunLaunch next_launch(const dmrt_ctx* c, int64_t left, int64_t to_poll, b
         return {n >= 2 ? kRunCluster : kRunOne, (int)n};
     }
     if (left >= graph_steps(c)) return {kRunGraph, graph_steps(c)};
-    const int n = pair ? 2 : launch_steps(c, left);
+    const int n = pair ? 2 : launch_steps(c, left, marched);
     return {n > 1 ? kRunMarch : kRunOne, n};
 }
 
@@ -1748,7 +1765,7 @@ static int step_run(dmrt_ctx* c, int64_t nsteps, bool finalize, float* record = 
             if (!rc) rc = poll_error(c);
             if (rc) return rc;
         }
-        const RunLaunch r = next_launch(c, nsteps, c->next_poll - c->t, pair);
+        const RunLaunch r = next_launch(c, nsteps, c->next_poll - c->t, c->nu_open > 1, pair);
         int rc = DMRT_OK;
         switch (r.kind) {
             case kRunBand:
@@ -1805,8 +1822,8 @@ int dmrt_get_run_launch(const dmrt_ctx* c, int64_t nsteps, dmrt_run_launch* out)
     long long steps[5] = {}, to_poll = c->next_poll - c->t;
     bool pair = false, marched = false, summed = false;
     for (long long left = nsteps; left > 0;) {  // the run, as step_run takes it
-        if (to_poll <= 0) to_poll = kPollSteps, out->launches += 1;
-        const RunLaunch r = next_launch(c, left, to_poll, pair);
+        if (to_poll <= 0) to_poll = kPollSteps, out->launches += 1, marched = false;
+        const RunLaunch r = next_launch(c, left, to_poll, marched, pair);
         pair = r.kind == kRunMarch && r.n == 2 && !pair;
         if (r.kind == kRunOne && marched) out->launches += 1;  // the march launches' sums
         marched = r.kind == kRunMarch || (r.kind == kRunGraph && c->march[2]);
@@ -1831,7 +1848,7 @@ int dmrt_get_run_launch(const dmrt_ctx* c, int64_t nsteps, dmrt_run_launch* out)
         out->block = c->bthreads;
         out->smem_bytes = (int64_t)c->bsmem;
     } else if (most == kRunMarch) {
-        const int n = launch_steps(c, nsteps);
+        const int n = launch_steps(c, nsteps, false);
         out->kernel = DMRT_KERNEL_MARCH;
         out->steps_per_launch = n;
         out->rows = c->mchunk[n];

@@ -15,12 +15,15 @@ pytestmark = pytest.mark.gpu
 
 MARCH = 4
 # Launches from either buffer; 200 and 400: one and two graphs of 192 steps, remainders of
-# 8 = 3 + 2 + 2 + 1 and 16 steps.
+# 8 = 3 + 2 + 2 + 1 steps (3 + 3 + 1 + 1 in 16-bit storage) and 16.
 RUNS = (3, 200, 1, 400, 4, 2, 5, 7, 6, 1)
 MODES = [(0, 0), (1, 0), (1, 1), (2, 0), (2, 1), (3, 0), (3, 1), (4, 0), (4, 1)]
 # Whole strips (60 columns in float32, 56 in 16-bit storage), one column more or less, several
-# chunks, few rows, and more than 1024 rows (Nusselt sums of several rows per partial).
+# chunks, few rows, and more than 1024 rows (Nusselt sums of several rows per partial);
+# 16-bit storage marches from 400000 nodes on up to 500 columns, else from a million.
 SIZES = [(1080, 43), (1081, 171), (1064, 181), (1063, 90), (777, 701), (241, 1501)]
+SIZES16 = [(448, 900), (447, 901), (449, 891), (241, 1701), (1065, 951), (5001, 201)]
+CASES = [(nx, ny, st, rd) for st, rd in MODES for nx, ny in (SIZES16 if st else SIZES)]
 
 
 def advance(nx, ny, storage, rounding, kernel, walls=(0, 0), cap=4096, runs=RUNS):
@@ -49,16 +52,15 @@ def assert_same(a, b):
         np.testing.assert_array_equal(x, y)
 
 
-@pytest.mark.parametrize("storage,rounding", MODES)
-@pytest.mark.parametrize("nx,ny", SIZES)
+@pytest.mark.parametrize("nx,ny,storage,rounding", CASES)
 def test_march_chain_equals_single_steps(nx, ny, storage, rounding):
     assert_same(advance(nx, ny, storage, rounding, 0), advance(nx, ny, storage, rounding, 2))
 
 
-@pytest.mark.parametrize("storage,rounding", [(0, 0), (1, 1), (3, 1)])
-@pytest.mark.parametrize("nx,ny", [(167, 4100), (300, 1024), (300, 1023)])
+@pytest.mark.parametrize("nx,ny,storage,rounding", [(1030, 511, 0, 0), (1030, 512, 0, 0), (300, 1023, 0, 0), (167, 4100, 0, 0),
+                                                    (167, 4100, 1, 1), (420, 1023, 3, 1)])
 def test_march_chain_tall_cavities(nx, ny, storage, rounding):
-    """Nusselt sums by one, two and eight blocks."""
+    """Nusselt sums by one, two, three and eight blocks."""
     assert_same(advance(nx, ny, storage, rounding, 0), advance(nx, ny, storage, rounding, 2))
 
 
@@ -86,7 +88,8 @@ def test_march_chain_of_a_batch_with_a_tall_member(storage, rounding):
 @pytest.mark.parametrize("walls", [(1, 0), (0, 1), (1, 1)])
 @pytest.mark.parametrize("storage", [0, 1, 3, 4])
 def test_march_chain_wall_kinds(walls, storage):
-    assert_same(advance(1081, 171, storage, 2, 0, walls), advance(1081, 171, storage, 2, 2, walls))
+    nx, ny = (449, 891) if storage else (1081, 171)
+    assert_same(advance(nx, ny, storage, 2, 0, walls), advance(nx, ny, storage, 2, 2, walls))
 
 
 @pytest.mark.parametrize("cap", [1, 2, 3, 5])
@@ -96,6 +99,6 @@ def test_march_chain_short_nusselt_ring(cap):
 
 def test_march_chain_bounds_checked_build():
     code = ("import sys; sys.path.insert(0, %r); from tests.test_march_chain import advance;"
-            "[advance(nx, ny, s, 2, 0) for nx, ny in ((1081, 171), (241, 1501)) for s in range(5)]" % ROOT)
+            "[advance(nx, ny, s, 2, 0) for nx, ny in ((449, 891), (241, 1701)) for s in range(5)]" % ROOT)
     subprocess.run([sys.executable, "-c", code], check=True, cwd=ROOT,
                    env=dict(os.environ, DMRT_LIBRARY="bounds_check"))
