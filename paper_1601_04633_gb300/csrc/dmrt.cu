@@ -1709,7 +1709,10 @@ static int launch_band(dmrt_ctx* c, int n, float* record = nullptr, long long st
         if (e == cudaErrorCooperativeLaunchTooLarge) return kNoBand;  // (fewer SMs than at creation)
         CK(e, "band launch");
     }
-    dmrt::band_nu_kernel<<<(n + dmrt::kBandNuWarps - 1) / dmrt::kBandNuWarps, 32 * dmrt::kBandNuWarps, 0, c->stream>>>(B);
+    if (c->p.ny > 256)
+        dmrt::band_nu_kernel<true><<<n, 32 * dmrt::kBandNuWarps, 0, c->stream>>>(B);
+    else
+        dmrt::band_nu_kernel<false><<<(n + dmrt::kBandNuWarps - 1) / dmrt::kBandNuWarps, 32 * dmrt::kBandNuWarps, 0, c->stream>>>(B);
     CK(cudaGetLastError(), "band Nusselt launch");
     c->cur = end;
     c->t += n;

@@ -133,3 +133,14 @@ def test_band_bounds_checked_build():
             "[advance(nx, ny, s, 2, 0) for nx, ny in ((130, 127), (193, 305), (640, 151), (100, 60)) for s in range(5)]" % ROOT)
     subprocess.run([sys.executable, "-c", code], check=True, cwd=ROOT,
                    env=dict(os.environ, DMRT_LIBRARY="bounds_check"))
+
+
+@pytest.mark.parametrize("storage,rounding", [(0, 0), (1, 1), (4, 0)])
+@pytest.mark.parametrize("nx,ny", [(9, 256), (9, 257), (16, 1100), (40, 1281), (8, 6001)])
+def test_band_nusselt_of_tall_cavities(nx, ny, storage, rounding):
+    """Sums of a step by one warp and by a block, streams of one and of several rows."""
+    assert_same(advance(nx, ny, storage, rounding, 0, runs=(6, 1, 530)), advance(nx, ny, storage, rounding, 2, runs=(6, 1, 530)))
+
+
+def test_band_nusselt_short_ring_of_a_tall_cavity():
+    assert_same(advance(40, 700, 0, 0, 0, cap=3), advance(40, 700, 0, 0, 2, cap=3))
