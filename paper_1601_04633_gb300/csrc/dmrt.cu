@@ -1709,11 +1709,11 @@ static int launch_band(dmrt_ctx* c, int n, float* record = nullptr, long long st
         if (e == cudaErrorCooperativeLaunchTooLarge) return kNoBand;  // (fewer SMs than at creation)
         CK(e, "band launch");
     }
-    if (c->p.ny > 256)
-        dmrt::band_nu_kernel<true><<<n, 32 * dmrt::kBandNuWarps, 0, c->stream>>>(B);
-    else
-        dmrt::band_nu_kernel<false><<<(n + dmrt::kBandNuWarps - 1) / dmrt::kBandNuWarps, 32 * dmrt::kBandNuWarps, 0, c->stream>>>(B);
-    CK(cudaGetLastError(), "band Nusselt launch");
+    const dim3 nu_threads(32 * dmrt::kBandNuWarps);
+    CK(c->p.ny > 256 ? launch_overlapped(dmrt::band_nu_kernel<true>, dim3(n), nu_threads, c->stream, B)
+                     : launch_overlapped(dmrt::band_nu_kernel<false>, dim3((n + dmrt::kBandNuWarps - 1) / dmrt::kBandNuWarps),
+                                         nu_threads, c->stream, B),
+       "band Nusselt launch");
     c->cur = end;
     c->t += n;
     return DMRT_OK;

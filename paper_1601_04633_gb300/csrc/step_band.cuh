@@ -504,6 +504,7 @@ __global__ void __launch_bounds__(32 * kBandNuWarps) band_nu_kernel(const __grid
     __shared__ double part[BLOCK ? 8 : 1][32];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int s = BLOCK ? (int)blockIdx.x : (int)blockIdx.x * kBandNuWarps + warp;
+    grid_dep_wait();           // (launched while the steps finish)
     if (s >= B.steps) return;  // (BLOCK: the whole block)
     const long long t = *B.t_base;
     const F2* rec = B.record + (size_t)s * A.ny;
