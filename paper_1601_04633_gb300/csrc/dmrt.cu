@@ -76,9 +76,15 @@ int band_rows(const dmrt_params& p) {
     return std::min(p.ny, std::max(p.nx > 512 ? 1 : 2, (p.ny + kBandBlocks - 1) / kBandBlocks));
 }
 // Whether a cavity's rows split like this fit the blocks' shared memory (up to
-// about 512^2), under AUTO. Batch members (stepped by the batch's launches) go without.
+// about 512^2), under AUTO. Batch members (stepped by the batch's launches) go without,
+// and so do wide cavities of few rows in 16-bit storage: a step of one-row blocks of 400
+// pairs and more takes 3.0 to 3.3 us, a launch per step 2.9 to 3.5 (800 x 8 float16 3.02 / 2.92,
+// 1024 x 60 mixed 3.33 / 3.40, and 28.7 / 25.7 us for six steps).
+constexpr int kBandFlat = 750;           // widest of 16-bit cavities below kBandFlatNodes nodes
+constexpr long long kBandFlatNodes = 80000;
 bool band_fits(const dmrt_params& p) {
     if (p.kernel != DMRT_KERNEL_AUTO || p.tma_npt > 0 || p.tma_rows > 0 || p.tma_stages > 0) return false;
+    if (p.storage != DMRT_FP32 && p.nx > kBandFlat && (long long)p.nx * p.ny < kBandFlatNodes) return false;
     return p.nx >= 8 && p.nx <= 1024 && dmrt::band_smem(band_rows(p), p.nx) <= (size_t)dmrt::kMaxSmem;
 }
 size_t band_mail_bytes(const dmrt_params& p) {
@@ -1017,8 +1023,11 @@ int setup_march(dmrt_ctx* c) {
 // Runs of at least kBandMinSteps steps on the band kernel: AUTO's choice for
 // whole cavities that fit it, in every storage mode. In one cluster while its
 // blocks hold at most kBandClusterItems pairs (rows rounded up to whole warps),
-// else across the GPU; the smallest float32 cavities, and those of at most
-// kClusterNodes nodes per block in between, stay with step_cluster.cuh.
+// else across the GPU; the smallest float32 cavities, those of at most kClusterNodes
+// nodes per block in between, and those whose blocks have one row, stay with
+// step_cluster.cuh up to kClusterRow columns (300 x 16 1.12, in one cluster here 1.19; 400 x 16
+// 1.27 and 1.15) and from 513 on, as far as it holds them (560 x 10 1.47, across the GPU 2.33;
+// 640 x 12 1.85 and 2.34).
 // Microseconds per step, one cluster / across the GPU / step_cluster.cuh / one
 // or three steps per launch: float32 16^2 1.10 / 1.26 / 0.97 / 2.7, 32^2 0.98 / 1.25 /
 // 0.96, 64^2 0.92 / 1.24 / 1.12, 100 x 60 1.11 / 1.25 / 1.19, 80^2 1.27 / 1.25 / 1.25,
@@ -1028,6 +1037,7 @@ int setup_march(dmrt_ctx* c) {
 // 3.75, 512^2 - / 3.87 / - / 6.63; 100 x 500 float32 - / 1.41 / - / 3.90. A call of 8
 // steps: 128^2 20.8 us against 32.0, 512^2 47.8 against 69.6.
 constexpr int kClusterNodes = 480;
+constexpr int kClusterRow = 352;
 constexpr int kBandClusterItems = 256;
 void band_cluster_config(const dmrt_ctx* c, cudaLaunchConfig_t* cfg, cudaLaunchAttribute* attr) {
     attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -1054,7 +1064,7 @@ int setup_band(dmrt_ctx* c) {
     };
     const int crows = (p.ny + dmrt::kBandCluster - 1) / dmrt::kBandCluster;
     const int citems = crows * (((p.nx + 1) / 2 + 31) / 32 * 32);
-    if (c->cluster && citems <= 64) return DMRT_OK;
+    if (c->cluster && (citems <= 64 || (crows == 1 && p.nx <= kClusterRow))) return DMRT_OK;
     if (citems <= kBandClusterItems && dmrt::band_cluster_smem(crows, p.nx) <= (size_t)dmrt::kMaxSmem) {
         const void* fn = dmrt::band_cluster_kernel(p.storage, p.rounding);
         c->brows = crows;
@@ -1076,6 +1086,7 @@ int setup_band(dmrt_ctx* c) {
         (void)cudaGetLastError();
     }
     if (c->cluster && (long long)c->crows * p.nx <= kClusterNodes) return DMRT_OK;
+    if (c->cluster && p.nx > 512) return DMRT_OK;  // (one-row blocks)
     int dev = 0, sms = 0, per_sm = 0, coop = 0;
     CK(cudaGetDevice(&dev), "cudaGetDevice");
     CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev), "SM count");

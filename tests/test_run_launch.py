@@ -35,6 +35,11 @@ def plan(D, nx, ny, n, storage=0, **kw):
     (300, 300, 4, 5, TMA, 0, 6), (300, 300, 0, 5, MARCH, 0, 5), (159, 9000, 0, 30, DIRECT, 0, 31),
     (32, 32, 0, 100, CLUSTER, 1, 2),          # and the Nusselt sum
     (64, 64, 0, 5, CLUSTER, 1, 2),
+    # One-row blocks: the cluster kernel up to 352 columns, and from 513 on while it holds them.
+    (300, 16, 0, 50, CLUSTER, 1, 2), (352, 10, 0, 50, CLUSTER, 1, 2), (353, 10, 0, 50, BAND, 1, 2),
+    (512, 4, 0, 50, BAND, 1, 2), (513, 16, 0, 50, CLUSTER, 1, 2), (640, 3, 0, 50, CLUSTER, 1, 2), (1000, 2, 0, 50, BAND, 0, 2),
+    # Wide and flat in 16-bit storage: a launch per step.
+    (751, 106, 1, 50, TMA, 0, 51), (751, 107, 1, 50, BAND, 0, 2), (750, 8, 3, 50, BAND, 0, 2), (1024, 60, 0, 50, BAND, 0, 2),
     (64, 64, 0, 2000, BAND, 1, 8),            # four launches and their sums
     (64, 64, 3, 2000, BAND, 1, 8),
     (256, 256, 0, 515, BAND, 0, 4),
