@@ -2771,6 +2771,7 @@ int batch_setup_march(dmrt_batch* b, CUtensorMap* d_maps, int sms) {
                 B.n = dmrt::make_pair_numbers();
                 B.n_cav = count;
                 B.nu_blocks = march_nu_blocks(tall);
+                B.ctr = first == 0 ? b->groups[0].d_ctr : nullptr;  // (no tile asked for: one group)
                 for (int i = 0; i < count; ++i) {
                     dmrt_ctx* c = b->sub[first + i];
                     dmrt::MarchArgs& M = B.M[i];
@@ -3140,10 +3141,6 @@ int dmrt_batch_step(dmrt_batch* b, int64_t nsteps) {
         int rc = batch_march(b, 0, start);
         if (rc) return rc;
     }
-    // The single-step launches' work-pool counters alternate by source buffer, which
-    // march launches in between do not keep up.
-    if (b->march[3] && nsteps > 0)
-        BCK(cudaMemsetAsync(b->d_err + 1, 0, sizeof(unsigned) * 2 * b->groups.size(), b->stream), "work-pool counters");
     // Group after group, each for all nsteps steps (independent cavities: the
     // order of the groups does not change any result).
     for (BatchGroup& G : b->groups) {

@@ -692,6 +692,9 @@ struct MarchBatchArgs {
     PairNumbers n;
     int n_cav, items;
     int nu_blocks;            // of each cavity
+    unsigned* ctr;            // the single-step launches' two work-pool counters, cleared here (they
+                              // alternate by source buffer, which march launches in between do not
+                              // keep up); nullptr: another launch clears them
     int first[kMarchBatch];   // first item of each cavity
     MarchArgs M[kMarchBatch];
     PairRates r[kMarchBatch];
@@ -710,6 +713,7 @@ __global__ void __launch_bounds__(kMarchThreads, MINB) batch_march_kernel(const 
     if (__syncthreads_or(threadIdx.x == 0 && (*reinterpret_cast<volatile unsigned*>(B.err) & kErrTimeout))) return;
     const int extra = (int)blockIdx.x - ((int)gridDim.x - B.n_cav * B.nu_blocks);
     if (extra >= 0) {
+        if (extra == 0 && B.ctr && threadIdx.x < 2) B.ctr[threadIdx.x] = 0u;
         const int cav = extra / B.nu_blocks;
         march_nu_finish<1>(B.M[cav], T, reinterpret_cast<MarchPart*>(smem_m), extra - cav * B.nu_blocks);
         return;
