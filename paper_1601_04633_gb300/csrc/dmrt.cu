@@ -2727,13 +2727,15 @@ int batch_build_graph(dmrt_batch* b, BatchGroup& G, int from) {
     return DMRT_OK;
 }
 
-// The march launches of a batch: its cavities in groups of kMarchBatch, one
+// The march launches of a batch: its cavities in equal groups of up to kMarchBatch, one
 // chunk height for all of a group. Taken whenever no tile or schedule was asked
-// for. Microseconds per step of all cavities, march / one launch per step
-// (default tile): the 64-cavity sweep (sides 128 to 384) float32 46.4 / 98.6,
-// mixed stochastic 55.0 / 73.0; 512 of 32^2 49.0 / 56.4; 64 of 32^2 5.7 / 11.7; 128 of
-// 64^2 17.5 / 24.1; 64 of 128^2 16.1 / 26.8; 9 of 300 x 280 10.1 / 22.1; 3 of 1024^2
-// 29.1 / 65.7; 3 of 100 x 80 3.5 / 6.4.
+// for. Microseconds per step of all cavities over 192 steps, march / one launch per step
+// (default tile): 64 of sides 128 to 384 float32 36.5 / 81.9, mixed stochastic 43.6 / 62.6;
+// 512 of 32^2 41.2 / 56.5; 200 of 40^2 18.6 / 28.1; 64 of 128^2 15.7 / 26.4; 9 of 300 x 280
+// 9.7 / 21.9; 3 of 1024^2 28.0 / 65.4; 64 of 12 x 1000 33.9 / 101. A group's launch waits for
+// the one before, so flat cavities in many groups gain least: 300 of 64 x 17 23.5 / 31.6,
+// mixed 27.8 / 32.8; 330 of them mixed 34.8 / 34.4, and short calls lose up to 5 % (3 steps
+// 113 us / 108).
 int batch_setup_march(dmrt_batch* b, CUtensorMap* d_maps, int sms) {
     const dmrt_params& p0 = b->sub[0]->p;
     const dmrt::MarchForm F[4] = {{}, {}, dmrt::batch_march_form(p0.storage, p0.rounding, 2),
@@ -2755,8 +2757,9 @@ int batch_setup_march(dmrt_batch* b, CUtensorMap* d_maps, int sms) {
         BCK(cudaFuncSetAttribute(F[t].func, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)F[t].smem), "march shared memory");
         BCK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, F[t].func, dmrt::kMarchThreads, F[t].smem), "occupancy");
         if (per_sm < 1) return DMRT_OK;
-        for (int first = 0; first < b->n; first += dmrt::kMarchBatch) {
-            const int count = std::min(dmrt::kMarchBatch, b->n - first);
+        const int parts = (b->n + dmrt::kMarchBatch - 1) / dmrt::kMarchBatch, share = (b->n + parts - 1) / parts;
+        for (int first = 0; first < b->n; first += share) {
+            const int count = std::min(share, b->n - first);
             std::vector<std::pair<int, int>> cav;
             for (int i = first; i < first + count; ++i)
                 cav.emplace_back(b->sub[i]->p.ny, (b->sub[i]->p.nx + F[t].cols - 1) / F[t].cols);
@@ -3098,8 +3101,9 @@ int dmrt_batch_create(const dmrt_params* arr, int32_t n, const double* const* th
 static int batch_march(dmrt_batch* b, int n, int parity) {
     for (dmrt::MarchBatchArgs& B : b->margs[n > 0 ? n : 3][parity]) {
         if (n == 0) {
-            dmrt::batch_march_finalize_kernel<<<B.n_cav * B.nu_blocks, dmrt::kMarchSumThreads, 0, b->stream>>>(B);
-            BCK(cudaGetLastError(), "batch Nusselt launch");
+            BCK(launch_overlapped(dmrt::batch_march_finalize_kernel, dim3(B.n_cav * B.nu_blocks),
+                                  dim3(dmrt::kMarchSumThreads), b->stream, B),
+                "batch Nusselt launch");
             continue;
         }
         const int per = dmrt::kMarchThreads / 32;
@@ -3111,8 +3115,11 @@ static int batch_march(dmrt_batch* b, int n, int parity) {
     return DMRT_OK;
 }
 
-// Steps of the next march launch: three, or two in a pair of launches (see launch_steps).
-static int batch_march_steps(int64_t n) { return n == 4 || n == 5 ? 2 : 3; }
+// Steps of the next march launch: three, or in float32 two in a pair of launches (see
+// launch_steps; mixed, 1000 of 64 x 17, 4 steps: 469 us with pairs, 411 with a single step).
+static int batch_march_steps(const dmrt_batch* b, int64_t n) {
+    return b->sub[0]->p.storage == DMRT_FP32 && (n == 4 || n == 5) ? 2 : 3;
+}
 
 int dmrt_batch_step(dmrt_batch* b, int64_t nsteps) {
     if (!b || nsteps < 0) return DMRT_E_ARG;
@@ -3124,13 +3131,14 @@ int dmrt_batch_step(dmrt_batch* b, int64_t nsteps) {
         }
     }
     // March launches for what they take of the steps (a remainder of one or two
-    // goes to the launches of single steps).
+    // goes to the launches of single steps; a launch of three changes buffers once, as
+    // three single ones would).
     const int start0 = b->parity;
     int start = start0;
     const int64_t total = nsteps;
     if (b->march[3] && nsteps >= 3) {
         while (nsteps >= 3) {
-            const int n = batch_march_steps(nsteps);
+            const int n = batch_march_steps(b, nsteps);
             for (int k = 0; k < (n == 2 ? 2 : 1); ++k) {
                 int rc = batch_march(b, n, start);
                 if (rc) return rc;
@@ -3163,8 +3171,9 @@ int dmrt_batch_step(dmrt_batch* b, int64_t nsteps) {
             }
         }
         if (nsteps > 0)  // each cavity's last step: its local Nu rows into its ring
-            dmrt::nu_finalize_batch_kernel<<<G.count, 256, 0, b->stream>>>(b->d_cav + G.first, parity);
-        BCK(cudaGetLastError(), "batch step launch");
+            BCK(launch_overlapped(dmrt::nu_finalize_batch_kernel, dim3(G.count), dim3(256), b->stream,
+                                  (const dmrt::BatchCavity*)(b->d_cav + G.first), parity),
+                "batch step launch");
     }
     b->parity = start0 ^ (int)(total & 1);
     b->t += total;
@@ -3213,11 +3222,11 @@ int dmrt_batch_get_run_launch(const dmrt_batch* b, int64_t nsteps, dmrt_run_laun
         const long long parts = (long long)b->margs[3][0].size();
         long long left = nsteps, launches = 0;
         while (left >= 3) {
-            const int n = batch_march_steps(left), k = n == 2 ? 2 : 1;
+            const int n = batch_march_steps(b, left), k = n == 2 ? 2 : 1;
             launches += k;
             left -= k * n;
         }
-        const int n = batch_march_steps(nsteps);
+        const int n = batch_march_steps(b, nsteps);
         const dmrt::MarchBatchArgs& B = b->margs[n][0][0];
         out->kernel = DMRT_KERNEL_MARCH;
         out->steps_per_launch = n;

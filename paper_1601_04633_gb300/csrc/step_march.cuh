@@ -685,7 +685,7 @@ __global__ void __launch_bounds__(kMarchThreads, MINB)
 // warp takes them from the constant bank at its cavity's (uniform) index, as
 // the single-cavity kernel does; the tensor maps lie in global memory. The last
 // n_cav nu_blocks blocks take the cavities' Nusselt sums.
-constexpr int kMarchBatch = 64;
+constexpr int kMarchBatch = 80;  // (parameters of at most 32764 bytes)
 struct MarchBatchArgs {
     const CUtensorMap* maps;  // [n_cav][6]: loads, stores of this launch's source buffer
     unsigned* err;            // the batch's error word (an expired wait)
@@ -735,6 +735,7 @@ __global__ void __launch_bounds__(kMarchThreads, MINB) batch_march_kernel(const 
 static __global__ void __launch_bounds__(kMarchSumThreads)
     batch_march_finalize_kernel(const __grid_constant__ MarchBatchArgs B) {
     __shared__ MarchPart part[kMarchMax];
+    grid_dep_wait();  // (launched while the last step, or another group's sums, finish)
     const int cav = blockIdx.x / B.nu_blocks;
     march_nu_finish<4>(B.M[cav], 0, part, blockIdx.x - cav * B.nu_blocks);
 }
@@ -746,6 +747,7 @@ struct MarchForm {
     unsigned smem;
     int cols, box;
 };
+static_assert(sizeof(MarchBatchArgs) <= 32764, "kernel parameters");
 MarchForm march_form(int storage, int rounding, int steps);
 MarchForm batch_march_form(int storage, int rounding, int steps);  // float32 and mixed storage
 

@@ -311,6 +311,7 @@ __global__ void __launch_bounds__(R * (256 / NPT), MINB)
 
 // Sums each cavity's last step of a run (one block of 256 threads per cavity).
 static __global__ void nu_finalize_batch_kernel(const BatchCavity* __restrict__ cav, int parity) {
+    grid_dep_wait();  // (launched while the last step finishes)
     nu_finish_prev(cav[blockIdx.x].args[parity], false);
 }
 

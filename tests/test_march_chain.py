@@ -85,6 +85,25 @@ def test_march_chain_of_a_batch_with_a_tall_member(storage, rounding):
     b.close()
 
 
+@pytest.mark.parametrize("count,storage,rounding", [(80, 0, 0), (81, 0, 0), (81, 3, 1), (163, 3, 0)])
+def test_march_chain_of_several_groups_of_a_batch(count, storage, rounding):
+    """Groups of up to 80 cavities, single steps and short runs in between, every member."""
+    from paper_1601_04633_gb300 import dmrt as D
+    from paper_1601_04633_gb300 import inputs
+
+    cavs = [inputs.Cavity(8 + k % 61, 8 + k % 23, 1e3, 0.01, noise_amp=1e-2, seed=k) for k in range(count)]
+    b = D.Batch.from_inputs(cavs, nu_capacity=64, storage=storage, rounding=rounding)
+    for n in (1, 3, 2, 4, 1, 5, 9, 8):
+        b.step(n)
+    b.check()
+    for m, c in zip(b.members, cavs):
+        ref = D.Cavity2D.from_inputs(c, nu_capacity=64, storage=storage, rounding=rounding, kernel=2)
+        ref.step(33)
+        assert_same([m.get_state(), m.nusselt(64)[2]], [ref.get_state(), ref.nusselt(64)[2]])
+        ref.close()
+    b.close()
+
+
 @pytest.mark.parametrize("walls", [(1, 0), (0, 1), (1, 1)])
 @pytest.mark.parametrize("storage", [0, 1, 3, 4])
 def test_march_chain_wall_kinds(walls, storage):

@@ -74,3 +74,9 @@ def test_batch_runs(D):
         r = b.run_launch(n)
         assert (r["kernel"], r["steps_per_launch"], r["launches"]) == want
         b.close()
+    # Mixed storage leaves a remainder to single steps; more than 80 cavities: groups, each with its launches.
+    for count, storage, n, launches in ((5, 3, 5, 1 + 1 + 2 + 1), (81, 0, 6, 2 * (2 + 1))):
+        b = D.Batch.from_inputs([inputs.Cavity(20, 20, 1e3, 0.01)] * count, nu_capacity=16, storage=storage)
+        r = b.run_launch(n)
+        assert (r["kernel"], r["steps_per_launch"], r["launches"]) == (MARCH, 3, launches)
+        b.close()
