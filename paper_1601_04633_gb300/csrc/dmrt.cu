@@ -80,10 +80,26 @@ int band_rows(const dmrt_params& p) {
 // and so do wide cavities of few rows in 16-bit storage: a step of one-row blocks of 400
 // pairs and more takes 3.0 to 3.3 us, a launch per step 2.9 to 3.5 (800 x 8 float16 3.02 / 2.92,
 // 1024 x 60 mixed 3.33 / 3.40, and 28.7 / 25.7 us for six steps).
+// Small float32 cavities whose runs stay with step_cluster.cuh (rules at setup_band) hold no
+// messages and no record either.
+bool auto_cluster(const dmrt_params& p);
+constexpr int kClusterNodes = 480;
+constexpr int kClusterRow = 352;
+constexpr int kBandClusterItems = 256;
+int band_cluster_items(const dmrt_params& p) {
+    return (p.ny + dmrt::kBandCluster - 1) / dmrt::kBandCluster * (((p.nx + 1) / 2 + 31) / 32 * 32);
+}
+bool cluster_keeps(const dmrt_params& p) {
+    if (!auto_cluster(p)) return false;
+    const int items = band_cluster_items(p), crows = (p.ny + 15) / 16;
+    if (items <= 64 || (crows == 1 && p.nx <= kClusterRow) || p.nx > 512) return true;
+    return items > kBandClusterItems && (long long)crows * p.nx <= kClusterNodes;
+}
 constexpr int kBandFlat = 750;           // widest of 16-bit cavities below kBandFlatNodes nodes
 constexpr long long kBandFlatNodes = 80000;
 bool band_fits(const dmrt_params& p) {
     if (p.kernel != DMRT_KERNEL_AUTO || p.tma_npt > 0 || p.tma_rows > 0 || p.tma_stages > 0) return false;
+    if (cluster_keeps(p)) return false;
     if (p.storage != DMRT_FP32 && p.nx > kBandFlat && (long long)p.nx * p.ny < kBandFlatNodes) return false;
     return p.nx >= 8 && p.nx <= 1024 && dmrt::band_smem(band_rows(p), p.nx) <= (size_t)dmrt::kMaxSmem;
 }
@@ -1036,9 +1052,6 @@ int setup_march(dmrt_ctx* c) {
 // mixed, stochastic 64^2 0.95 / 1.28 / - / 3.26, 96^2 1.46 / 1.29, 256^2 - / 1.58 / - /
 // 3.75, 512^2 - / 3.87 / - / 6.63; 100 x 500 float32 - / 1.41 / - / 3.90. A call of 8
 // steps: 128^2 20.8 us against 32.0, 512^2 47.8 against 69.6.
-constexpr int kClusterNodes = 480;
-constexpr int kClusterRow = 352;
-constexpr int kBandClusterItems = 256;
 void band_cluster_config(const dmrt_ctx* c, cudaLaunchConfig_t* cfg, cudaLaunchAttribute* attr) {
     attr[0].id = cudaLaunchAttributeClusterDimension;
     attr[0].val.clusterDim.x = c->bblocks;
@@ -1063,9 +1076,7 @@ int setup_band(dmrt_ctx* c) {
         return ((items + passes - 1) / passes + 31) / 32 * 32;
     };
     const int crows = (p.ny + dmrt::kBandCluster - 1) / dmrt::kBandCluster;
-    const int citems = crows * (((p.nx + 1) / 2 + 31) / 32 * 32);
-    if (c->cluster && (citems <= 64 || (crows == 1 && p.nx <= kClusterRow))) return DMRT_OK;
-    if (citems <= kBandClusterItems && dmrt::band_cluster_smem(crows, p.nx) <= (size_t)dmrt::kMaxSmem) {
+    if (band_cluster_items(p) <= kBandClusterItems && dmrt::band_cluster_smem(crows, p.nx) <= (size_t)dmrt::kMaxSmem) {
         const void* fn = dmrt::band_cluster_kernel(p.storage, p.rounding);
         c->brows = crows;
         c->bblocks = (p.ny + crows - 1) / crows;
@@ -1085,8 +1096,6 @@ int setup_band(dmrt_ctx* c) {
         }
         (void)cudaGetLastError();
     }
-    if (c->cluster && (long long)c->crows * p.nx <= kClusterNodes) return DMRT_OK;
-    if (c->cluster && p.nx > 512) return DMRT_OK;  // (one-row blocks)
     int dev = 0, sms = 0, per_sm = 0, coop = 0;
     CK(cudaGetDevice(&dev), "cudaGetDevice");
     CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev), "SM count");
@@ -1350,8 +1359,9 @@ static int create_ctx(const dmrt_params* pg, int y0, int rows, bool slab, bool b
     if (!rc2) rc2 = setup_march(c);
     if (!rc2) rc2 = setup_band(c);
     if (rc2) return fail(rc2);
-    // Zero the scalars and the ring, set the wall profiles, write the initial state.
-    if (cudaMemsetAsync(c->ws + L.off_hot, 0, L.total - L.off_hot, c->stream) != cudaSuccess)
+    // Zero the scalars and the ring, set the wall profiles, write the initial state. (The band
+    // kernel's record, last in the workspace, is written before it is read.)
+    if (cudaMemsetAsync(c->ws + L.off_hot, 0, (L.off_record ? L.off_record : L.total) - L.off_hot, c->stream) != cudaSuccess)
         return fail(cuda_fail(c, cudaGetLastError(), "cudaMemsetAsync"));
     fill_kernel<<<(p->ny + 255) / 256, 256, 0, c->stream>>>(
         reinterpret_cast<float*>(c->ws + L.off_hot), nullptr, p->theta_hot, p->ny);
@@ -2091,7 +2101,7 @@ int dmrt_fields(dmrt_ctx* c, float* u, float* v, float* theta, int on_device) {
     // Tiles of up to 256 nodes of a row, a power of two near the row's length.
     int width = 32;
     while (width < 256 && width < p.nx) width *= 2;
-    const int blocks = (int)std::min<long long>((long long)((p.nx + width - 1) / width) * p.ny, 152 * 2048 / width);
+    const int blocks = (int)std::min<long long>((long long)((p.nx + width - 1) / width) * p.ny, 152 * 4096 / width);
     cudaError_t fe = cudaSuccess;
     with_layout(p.storage, [&](auto tag) {
         using Lt = decltype(tag);
