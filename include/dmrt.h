@@ -316,6 +316,10 @@ int dmrt_load(dmrt_ctx* c, const void* host_buf, size_t size);
  * Uses a file-scope device word; allocates nothing. Synchronises the stream. */
 int dmrt_probe_bounded_wait(int64_t limit_ns, void* stream, int64_t* waited_ns);
 
+/* The same for the two waits of the kernel that keeps a cavity on chip: kind 0, for a
+ * neighbour block's words in global memory; kind 1, for its message in shared memory. */
+int dmrt_probe_band_wait(int32_t kind, int64_t limit_ns, void* stream, int64_t* waited_ns);
+
 /* The same for a launch of several steps per pass: one warp's work on the top row of
  * a float32 context that takes such launches (else DMRT_E_ARG), with the copy of
  * the row'th row it loads (0 to 3) never complete. The warp must store nothing and record

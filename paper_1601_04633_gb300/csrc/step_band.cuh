@@ -106,7 +106,7 @@ __device__ __forceinline__ unsigned long long mail_get(const unsigned long long*
 // column 0, plane 0. false: the poll expired.
 template <int EX>
 __device__ __forceinline__ bool mail_read(const unsigned long long* box, int words, int x0, bool first, bool last,
-                                          unsigned tag, F2 (&v)[4]) {
+                                          unsigned tag, F2 (&v)[4], unsigned long long limit_ns = kWaitLimitNs) {
     const unsigned long long* p = box + x0;
     const unsigned long long* pl = p + (EX > 0 ? 1 : 2) * words;  // the plane pulled from the left
     const unsigned long long* pr = p + (EX > 0 ? 2 : 1) * words;  // and from the right
@@ -131,7 +131,7 @@ __device__ __forceinline__ bool mail_read(const unsigned long long* box, int wor
         if ((tries & 255) == 255) {
             const unsigned long long now = global_ns();
             if (t0 == 0) t0 = now;
-            else if (now - t0 > kWaitLimitNs) return false;
+            else if (now - t0 > limit_ns) return false;
         }
     }
 }
@@ -150,7 +150,7 @@ __device__ __forceinline__ void cluster_put(unsigned addr, F2 v, unsigned bar) {
     asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.b64 [%0], %1, [%2];" ::"r"(addr), "l"(v), "r"(bar)
                  : "memory");
 }
-__device__ __forceinline__ bool cluster_wait(uint64_t* bar, unsigned parity) {
+__device__ __forceinline__ bool cluster_wait(uint64_t* bar, unsigned parity, unsigned long long limit_ns = kWaitLimitNs) {
     unsigned long long t0 = 0;
     for (;;) {
         unsigned ok;
@@ -164,7 +164,7 @@ __device__ __forceinline__ bool cluster_wait(uint64_t* bar, unsigned parity) {
         if (ok) return true;
         const unsigned long long now = global_ns();
         if (t0 == 0) t0 = now;
-        else if (now - t0 > kWaitLimitNs) return false;
+        else if (now - t0 > limit_ns) return false;
     }
 }
 

@@ -54,6 +54,20 @@ def test_bounded_wait_gives_up_and_the_context_stays_usable(D):
     assert L.dmrt_probe_bounded_wait(10, ctypes.c_void_p(stream), None) == D.DMRT_E_ARG
 
 
+@pytest.mark.parametrize("kind", [0, 1])
+def test_the_band_kernels_waits_give_up(D, kind):
+    import torch
+
+    L = D.load()
+    stream = ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
+    waited = ctypes.c_int64(0)
+    for limit_ms in (5, 50):
+        assert L.dmrt_probe_band_wait(kind, limit_ms * 1_000_000, stream, ctypes.byref(waited)) == D.DMRT_E_TIMEOUT
+        assert limit_ms * 1e6 <= waited.value < limit_ms * 1e6 + 2e8
+    assert L.dmrt_probe_band_wait(kind, 10, stream, None) == D.DMRT_E_ARG
+    assert L.dmrt_probe_band_wait(2, 5_000_000, stream, None) == D.DMRT_E_ARG
+
+
 @pytest.mark.parametrize("row", [0, 1, 2, 3])
 def test_a_march_launch_reports_any_row_that_does_not_arrive(D, row):
     # 0 and 1 are waited for before the first row of the chunk, 2 and 3 in its rows.
