@@ -1,9 +1,9 @@
 #!/usr/bin/env python3
 """Benchmark of the fused double-MRT time step (MLUPS and fraction of the HBM roofline).
 
-One "step" is one time step of the whole cavity: one launch of the fused kernel
-(pull-stream of both lattices with the walls, D2Q9 MRT + force, D2Q5 MRT, store,
-hot-wall Nusselt reduction). The default workload is the largest single cavity,
+One "step" is one time step of the whole cavity (pull-stream of both lattices with the
+walls, D2Q9 MRT + force, D2Q5 MRT, store, hot-wall Nusselt reduction); which kernel takes a
+run and how many steps a launch does is the library's own report. The default workload is the largest single cavity,
 4096 x 4096 at Ra = 1e7, Pr = 0.001, alpha = 0.1, started at rest with seeded
 1e-6 noise; its two float32 population buffers (3.76 GB) are far larger than L2,
 so no flush is needed between steps.
@@ -22,6 +22,7 @@ import argparse
 import hashlib
 import json
 import os
+import re
 import statistics
 import subprocess
 import sys
@@ -52,23 +53,36 @@ KERNEL_SOURCES = [os.path.join(ROOT, "paper_1601_04633_gb300", "csrc", f)
                   for f in ("lattice.cuh", "collide_pair.cuh", "step_tma.cuh", "step_march.cuh", "step_direct.cuh")]
 
 
-def steps_per_pass(args, cav):
-    """Steps that one pass over the state takes: three by the march kernel, which AUTO
-    runs for the large cavities (no kernel or tile asked for), else one."""
-    auto = args.kernel == 0 and args.tma_npt <= 0 and args.tma_rows <= 0 and args.tma_stages <= 0
-    return 3 if auto and cav.nx >= 1024 and cav.ny >= 1024 else 1
+KERNELS = {1: "dmrt::step_direct_kernel", 2: "dmrt::step_tma_kernel", 3: "dmrt::step_cluster_kernel",
+           4: "dmrt::step_march_kernel", 5: "dmrt::step_band_kernel"}
+ON_CHIP = (3, 5)  # the state stays on chip for a launch's steps
 
 
-def launches_of(steps, per_pass):
-    """Kernel launches of one run of `steps` steps, Nusselt sums included."""
-    if per_pass == 1 or steps < 3:
-        return steps + 1
-    rest = steps % 3
-    if rest == 0:
-        return steps // 3 + 1
-    if rest == 1:  # the last four steps in two launches
-        return (steps - 4) // 3 + 2 + 1
-    return (steps - 5) // 3 + 2 + 1 + 2  # the last five in two launches, their sums, and a single step
+def steps_per_pass(run):
+    """Steps that one pass over the state in memory takes, from the library's report of a run."""
+    return run["steps_per_launch"] if run["kernel"] not in ON_CHIP else None
+
+
+def short_launch(run):
+    return {"kernel": KERNELS[run["kernel"]], **{k: run[k] for k in ("steps_per_launch", "grid", "block")}}
+
+
+def compact(x):
+    """Secondary results in six digits, tiles without their zeros: the line stays short
+    enough for a reader that keeps only its last kilobytes."""
+    if isinstance(x, float):
+        return float(f"{x:.6g}")
+    if isinstance(x, dict):
+        return {k: {t: v for t, v in y.items() if v} if k == "tile" else compact(y) for k, y in x.items()}
+    return [compact(y) for y in x] if isinstance(x, list) else x
+
+
+def bytes_and_frac(bytes_per_node, per_pass, mlups):
+    """Bytes per node and step, and the share of the HBM copy rate; None for a state on chip."""
+    if per_pass is None:
+        return {"bytes_per_node": None, "roofline_frac": None}
+    b = bytes_per_node / per_pass
+    return {"bytes_per_node": b, "roofline_frac": b * mlups * 1e6 / 1e9 / hbm_peak()[0]}
 
 
 def workload(name):
@@ -100,10 +114,12 @@ def dist_env():
 
 
 def kernel_hash():
+    """Of the kernel sources' code: comments and layout do not count."""
     h = hashlib.sha256()
     for f in KERNEL_SOURCES:
-        with open(f, "rb") as fh:
-            h.update(fh.read())
+        with open(f) as fh:
+            code = re.sub(r"//[^\n]*|/\*.*?\*/", "", fh.read(), flags=re.S)
+        h.update(" ".join(code.split()).encode())
     return h.hexdigest()[:16]
 
 
@@ -120,17 +136,18 @@ def hbm_peak():
     return FALLBACK_HBM_GBS, "fallback"
 
 
-def ncu_traffic_per_launch(nodes):
-    """DRAM bytes per launch from the committed ncu summary, scaled to ``nodes``;
-    None if absent or taken on a different kernel source."""
+def ncu_traffic_per_step(nodes, run):
+    """DRAM bytes per step from the committed ncu summary, scaled to ``nodes``; None if
+    absent, taken on a different kernel source or of another kernel than the run's."""
     try:
         with open(PROFILE_SUMMARY) as fh:
             d = json.load(fh)
     except (OSError, ValueError):
         return None
-    if d.get("kernel_source_hash") != kernel_hash():
+    if d.get("kernel_source_hash") != kernel_hash() or not d["kernel"].startswith(KERNELS[run["kernel"]] + "<") \
+            or d["steps_per_launch"] != run["steps_per_launch"]:
         return None
-    return d["dram_bytes_per_launch"] * nodes / d["nodes"]
+    return d["dram_bytes_per_step"] * nodes / d["nodes"]
 
 
 class ClockSampler:
@@ -322,8 +339,6 @@ def run_dmrt(args):
     kw = dict(kernel=args.kernel, tma_rows=args.tma_rows, tma_stages=args.tma_stages,
               tma_npt=args.tma_npt, storage=STORAGES[args.storage][0], rounding=STORAGES[args.storage][1])
     sim = D.Cavity2D.from_inputs(cav, nu_capacity=max(args.steps + args.warmup, 1), **kw)
-    launch = dict(sim.launch)
-    per_pass = steps_per_pass(args, cav)
     sim.step(args.warmup)
     sim.check()
     torch.cuda.synchronize()
@@ -336,6 +351,8 @@ def run_dmrt(args):
     if dist:
         dist.barrier()
     torch.cuda.synchronize()
+    run = sim.run_launch(max(args.steps, 1))
+    per_pass = steps_per_pass(run)
     ev0.record(stream)
     sim.step(args.steps)
     ev1.record(stream)
@@ -369,7 +386,7 @@ def run_dmrt(args):
             ms2 = e0.elapsed_time(e1)
             s2.check()
             series2 = s2.nusselt(series_cap=gate_steps)[2]
-            launch2 = dict(s2.launch)
+            launch2 = s2.run_launch(gate_steps)
             s2.close()
             return ms2, series2, launch2
 
@@ -381,8 +398,8 @@ def run_dmrt(args):
             err = nu_rel_dev(nu2, nu_ref)
             v2 = nodes * gate_steps / (ms2 / 1e3) / 1e6
             secondary[st] = {"value": v2, "unit": UNIT, "steps": gate_steps,
-                             "bytes_per_node": BYTES_PER_NODE[st] / per_pass, "launch": launch2,
-                             "roofline_frac": BYTES_PER_NODE[st] / per_pass * v2 * 1e6 / 1e9 / hbm_peak()[0],
+                             "launch": short_launch(launch2),
+                             **bytes_and_frac(BYTES_PER_NODE[st], steps_per_pass(launch2), v2),
                              "nu_mean_last": float(nu2[-1]),
                              "nu_max_rel_dev_vs_fp32": err, "nu_gate_ok": bool(err <= NU_GATE),
                              "vs_fp32_single": v2 / secondary["fp32_gate_reference"]["value"]}
@@ -410,7 +427,7 @@ def run_dmrt(args):
             s3.check()
             ms3 = e0.elapsed_time(e1)
             small[name] = {"value": cav_s.nx * cav_s.ny * n_s / (ms3 / 1e3) / 1e6, "unit": UNIT,
-                           "steps": n_s, "us_per_step": 1e3 * ms3 / n_s, "launch": dict(s3.launch)}
+                           "steps": n_s, "us_per_step": 1e3 * ms3 / n_s, "launch": short_launch(s3.run_launch(n_s))}
             s3.close()
             del s3
         secondary["small_cavities"] = small
@@ -434,7 +451,7 @@ def run_dmrt(args):
         def run_batch(opts, storage, rounding):
             batch = D.Batch.from_inputs(sweep, opts=opts, nu_capacity=bsteps + args.warmup, storage=storage,
                                         rounding=rounding)
-            groups = batch.groups
+            run_b = batch.run_launch(bsteps)
             batch.step(max(args.warmup, 64))
             torch.cuda.synchronize()
             e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
@@ -450,7 +467,11 @@ def run_dmrt(args):
                 tt = torch.tensor([ms_b], dtype=torch.float64, device="cuda")
                 dist.all_reduce(tt, op=dist.ReduceOp.MAX)
                 ms_b = tt.tolist()[0]
-            return ms_b, nu, groups
+            return ms_b, nu, run_b
+
+        def batch_pass(run_b, opts):
+            # Several steps of a resident group (a schedule with a tile) still move a state per step.
+            return run_b["steps_per_launch"] if opts["tma_npt"] <= 0 else 1
 
         def max_dev(xs, refs):
             return max(nu_rel_dev(a, b_) for a, b_ in zip(xs, refs))
@@ -463,28 +484,28 @@ def run_dmrt(args):
             one = [t for t in tuned["trials"] if t["opts"]["tma_npt"] > 0
                    and t["opts"].get("group_bytes", 0) == 0 and t["opts"].get("steps_per_launch", 1) <= 1]
             best_one = max(one, key=lambda t: t["mlups"])["opts"]
-            ms_st, nu_st, _ = run_batch(best_one, storage, rnd)
+            ms_st, nu_st, run_best = run_batch(best_one, storage, rnd)
             v1 = bnodes * bsteps / (ms_st / 1e3) / 1e6
-            entry = {"nodes": bnodes, "steps": bsteps, "bytes_per_node": bpn,
+            entry = {"nodes": bnodes, "steps": bsteps,
                      "one_launch_per_step": {"value": v1, "unit": UNIT, "tile": best_one,
                                              "roofline_frac": bpn * v1 * 1e6 / 1e9 / peak_hbm}}
             nu_best, best_value, entry["tile"] = nu_st, v1, best_one
             if tuned["opts"] != best_one:
-                ms_b2, nu_b2, ngroups = run_batch(tuned["opts"], storage, rnd)
+                ms_b2, nu_b2, run_b2 = run_batch(tuned["opts"], storage, rnd)
                 v2 = bnodes * bsteps / (ms_b2 / 1e3) / 1e6
-                bpn2 = bpn / (1 if tuned["opts"]["tma_npt"] > 0 else 3)  # no tile: three steps per pass
-                entry["tuned_schedule"] = {"value": v2, "unit": UNIT, "tile": tuned["opts"], "groups": ngroups,
-                                           "bytes_per_node": bpn2,
-                                           "roofline_frac": bpn2 * v2 * 1e6 / 1e9 / peak_hbm,
+                entry["tuned_schedule"] = {"value": v2, "unit": UNIT, "tile": tuned["opts"],
+                                           "launch": short_launch(run_b2),
+                                           **bytes_and_frac(bpn, batch_pass(run_b2, tuned["opts"]), v2),
                                            "nu_max_rel_diff_vs_one_launch_per_step": max_dev(nu_b2, nu_st)}
                 if v2 > best_value:
-                    best_value, nu_best, entry["tile"] = v2, nu_b2, tuned["opts"]
+                    best_value, nu_best, entry["tile"], run_best = v2, nu_b2, tuned["opts"], run_b2
             entry["value"] = best_value
             entry["unit"] = UNIT
-            if entry["tile"]["tma_npt"] <= 0:
-                entry["bytes_per_node"] = bpn / 3
-            entry["roofline_frac"] = entry["bytes_per_node"] * best_value * 1e6 / 1e9 / peak_hbm
-            entry["tuner_trials"] = [{"tile": t["opts"], "mlups": round(t["mlups"])} for t in tuned["trials"]]
+            entry.update(bytes_and_frac(bpn, batch_pass(run_best, entry["tile"]), best_value))
+            # The three best of the tuner's trials (all of them would make a line of 40 KB).
+            top = sorted(tuned["trials"], key=lambda t: -t["mlups"])[:3]
+            entry["tuner"] = {"trials": len(tuned["trials"]),
+                              "best": [{"tile": t["opts"], "mlups": round(t["mlups"])} for t in top]}
             if storage == 0:
                 nu_fp32 = nu_best
                 entry["workload"] = ("64 cavities, sides {128,192,256,384}, Ra log-uniform [1e4,1e6], "
@@ -579,10 +600,19 @@ def run_dmrt(args):
     steps = max(args.steps, 1)
     value = ws * nodes * args.steps / (ms / 1e3) / 1e6
     per_launch_s = ms / 1e3 / steps
-    bpn = BYTES_PER_NODE[args.storage] / per_pass  # one pass over the state takes per_pass steps
-    achieved = bpn * nodes / per_launch_s / 1e9
     peak, peak_src = hbm_peak()
-    traffic = ncu_traffic_per_launch(nodes) if args.storage == "fp32" else None
+    one_step = BYTES_PER_NODE[args.storage] * nodes / per_launch_s / 1e9
+    if per_pass is None:
+        roofline = {"bound": "latency (the state stays on chip)", "achieved": None, "peak": peak, "unit": "GB/s",
+                    "frac": None, "traffic": None, "peak_source": f"{peak_src} HBM copy bandwidth",
+                    "steps_per_launch": run["steps_per_launch"], "kernel": KERNELS[run["kernel"]]}
+    else:
+        traffic = ncu_traffic_per_step(nodes, run) if args.storage == "fp32" else None
+        roofline = {"bound": "hbm", "achieved": one_step / per_pass, "peak": peak, "unit": "GB/s",
+                    "frac": one_step / per_pass / peak, "traffic": traffic,
+                    "peak_source": f"{peak_src} HBM copy bandwidth",
+                    "bytes_per_node": BYTES_PER_NODE[args.storage] / per_pass, "steps_per_pass": per_pass,
+                    "one_step_per_pass_frac": one_step / peak, "kernel": KERNELS[run["kernel"]]}
     line = {
         "metric": METRIC, "value": value, "unit": UNIT, "n_gpus": ws, "steps": args.steps,
         "warmup": args.warmup, "ms_per_step": ms / steps, "higher_is_better": True,
@@ -590,21 +620,14 @@ def run_dmrt(args):
         "data": "synthetic",
         "config": {"workload": label, "nx": cav.nx, "ny": cav.ny, "Ra": cav.Ra, "Pr": cav.Pr,
                    "alpha": cav.alpha, "storage": args.storage, "parallelism": f"{ws} independent cavities",
-                   "launch": launch,
+                   "launch": short_launch(run),
                    "l2": "state (two 14-plane fp32 buffers) larger than L2: no flush"
                    if BYTES_PER_NODE[args.storage] * nodes > 129e6 else "state fits in L2"},
-        "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
-                     "frac": achieved / peak, "traffic": traffic,
-                     "peak_source": f"{peak_src} HBM copy bandwidth",
-                     "bytes_per_node": bpn,
-                     "steps_per_pass": per_pass,
-                     "one_step_per_pass_frac": BYTES_PER_NODE[args.storage] * nodes / per_launch_s / 1e9 / peak,
-                     "kernel": "dmrt::step_march_kernel" if per_pass > 1 else
-                     "dmrt::step_tma_kernel" if launch["kernel"] == 2 else "dmrt::step_direct_kernel"},
+        "roofline": roofline,
         "e2e": {"value": ws * nodes * args.steps / e2e_s / 1e6, "unit": UNIT,
                 "h2d_bytes_per_step": 8 * nodes / steps,
                 "d2h_bytes_per_step": (12 * nodes + 8 * args.steps) / steps},
-        "gpu_launches": launches_of(args.steps, per_pass),
+        "gpu_launches": run["launches"],
         "clocks": sampler.summary(),
         "nu_mean_last": nu_mean,
     }
@@ -612,7 +635,7 @@ def run_dmrt(args):
         if tag in secondary:
             secondary[tag]["vs_fp32_single"] = secondary[tag]["value"] / value
     if secondary:
-        line["secondary"] = secondary
+        line["secondary"] = compact(secondary)
     if ws == 1 and not args.no_cpu_baseline:
         line["cpu_baseline"] = time_oracle(cav, budget_s=12.0)
     print(json.dumps(line), flush=True)
