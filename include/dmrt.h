@@ -105,9 +105,13 @@ extern "C" {
  * below where the GPU fits it. Runs of steps of a whole cavity under AUTO, no tile
  * asked for, take several steps per launch, with the same bits: six steps or
  * more of a cavity up to about 512^2, in every storage mode, keep the state on
- * chip across the GPU (64^2 0.92, 256^2 1.44, 512^2 3.5 us per step); larger
- * cavities, from 40000 nodes and 160 columns, take three steps per pass over
- * the state (4096^2 118 us per step, 288 with one). TMA tiles
+ * chip across the GPU (float32 64^2 0.92, 256^2 1.44, 512^2 3.4 us per step); larger
+ * cavities of at least 160 columns, float32 from 40000 nodes, 16-bit storage from 400000
+ * (550000 above 900 columns; above 1600 mixed 600000, the others a million), take three
+ * steps per pass over the state (float32 4096^2 115 us per step, 288 with one); dmrt_get_run_launch says
+ * which. The on-chip kernel is a cooperative launch above about 64^2: its blocks, up
+ * to one per SM, start together, so a kernel on another stream that never ends before
+ * this run does keeps it from starting (ask for TMA then). TMA tiles
  * compiled in, as (nodes per
  * thread, rows R, stages S): NPT 4 with (R,S) in (1,2) (1,3) (1,4) (1,5) (1,6)
  * (2,2) (2,3) (2,4) (4,2) (4,3); NPT 2 with (1,3) (1,4) (1,5) (2,2) (2,3)

@@ -935,19 +935,28 @@ int setup_kernel(dmrt_ctx* c) {
 // Runs of steps on the march kernel (step_march.cuh): three steps per launch.
 //
 // AUTO takes it for whole cavities of at least 160 columns that the band kernel does not
-// hold (or for runs too short for it), from these many nodes on: float32 40000, mixed
-// 600000, the other storages a million; all 16-bit storages 400000 up to 500 columns.
+// hold (or for runs too short for it), from these many nodes on: float32 40000, 16-bit
+// storage 400000 up to 900 columns, 550000 up to 1600, above that mixed 600000 and the others a million.
 // Microseconds per step over 192 steps, march / one launch per step, on one GB300:
 // float32 1100 x 40 2.9 / 4.4, 700 x 500 6.3 / 9.6, 1024^2 11.9 / 22.2, 2048^2 33 / 77,
 // 4096^2 115 / 289; mixed, stochastic 800 x 700 9.6 / 12.0, 1024^2 14.0 / 19.3, 2048^2
-// 41 / 55; THETA32, stochastic 2048^2 46 / 55; float16, stochastic 1024^2 15.1 / 16.3,
-// 2048^2 45 / 50, 230 x 4000 15.4 / 17.4, 165 x 3000 9.5 / 13.4. Below these sizes the two are near
-// each other in 16-bit storage, in either order (700 x 500 mixed 7.8 / 7.4; 5000 x 90
-// float16 9.0 / 8.8, THETA32 9.3 / 8.9, 3000 x 267 float16 12.9 / 12.0), so they keep one launch per step.
+// 41 / 55; THETA32, stochastic 2048^2 46 / 55; float16, stochastic 800 x 700 10.3 / 12.7, 1024^2
+// 15.1 / 16.3, 2048^2 45 / 50, 230 x 4000 15.4 / 17.4, 165 x 3000 9.5 / 13.4. Below these lines the two
+// are near each other in 16-bit storage, in either order (700 x 500 mixed 7.8 / 7.4; 5000 x 90
+// float16 9.0 / 8.8, THETA32 9.3 / 8.9, 3000 x 267 float16 12.9 / 12.0, 1200 x 340 float16 9.2 / 8.0): one
+// launch per step there. (Above them the largest loss seen is 7 %: 1440 x 600 float16, whose columns
+// fill the one-step kernel's strips.)
 // (Two steps per launch: 163 us at 4096^2 in float32.)
-constexpr long long kMarchNodes = 40000, kMarchNodesMixed = 600000, kMarchNodes16 = 1000000, kMarchNodes16Tall = 400000;
-constexpr int kMarchTall = 500;   // the widest of the last
+constexpr long long kMarchNodes = 40000, kMarchNodes16[4] = {400000, 550000, 1000000, 600000};  // (the last: mixed)
+constexpr int kMarchColumns[2] = {900, 1600};  // up to which the first two hold
 constexpr int kMarchWidth = 160;  // (not measured below, where the band kernel does not reach)
+bool march_takes(const dmrt_params& p) {
+    const long long nodes = (long long)p.nx * p.ny;
+    if (p.nx < kMarchWidth) return false;
+    if (p.storage == DMRT_FP32) return nodes >= kMarchNodes;
+    const int range = p.nx <= kMarchColumns[0] ? 0 : p.nx <= kMarchColumns[1] ? 1 : p.storage == DMRT_MIXED ? 3 : 2;
+    return nodes >= kMarchNodes16[range];
+}
 
 // The march launches' tensor maps of c, by source buffer.
 int march_maps(dmrt_ctx* c, const dmrt::MarchForm& F, dmrt::MarchMaps* maps) {
@@ -1011,9 +1020,7 @@ int setup_march(dmrt_ctx* c) {
     std::memset(c->march, 0, sizeof c->march);
     if (c->cluster || c->slab || p.kernel != DMRT_KERNEL_AUTO || p.tma_npt > 0 || p.tma_rows > 0 || p.tma_stages > 0)
         return DMRT_OK;
-    const long long least = p.storage == DMRT_FP32 ? kMarchNodes : p.nx <= kMarchTall ? kMarchNodes16Tall
-                            : p.storage == DMRT_MIXED ? kMarchNodesMixed : kMarchNodes16;
-    if (p.nx < kMarchWidth || (long long)p.nx * p.ny < least) return DMRT_OK;
+    if (!march_takes(p)) return DMRT_OK;
     const dmrt::MarchForm F2 = dmrt::march_form(p.storage, p.rounding, 2), F = dmrt::march_form(p.storage, p.rounding, 3);
     int dev = 0, sms = 0, per_sm = 0;
     CK(cudaGetDevice(&dev), "cudaGetDevice");
@@ -1522,15 +1529,17 @@ static cudaError_t add_step_node(cudaGraph_t g, cudaGraphNode_t prev, const cuda
 // 56.5 us with them, 44.5 without). The sums at the end of a march launch cost more than
 // those of a single step, so float16 and bfloat16, whose gain is small, begin with a march
 // launch from kMarchMin16 steps on (1100 x 512 float16: 5 steps 60.6 us, 58.8 in single
-// steps; 6 steps 66.4 and 70.4), and THETA32 below kMarchShort nodes as well (2000 x 501: 5
-// steps 4 % more, 6 the same). marched: the run's last launch was the march kernel's.
+// steps; 6 steps 66.4 and 70.4), and so do smaller cavities in the other two (THETA32 2000 x 501, 5
+// steps 4 % more, 6 the same; mixed 600 x 700, 4 steps 5 % more). marched: the run's last
+// launch was the march kernel's.
 constexpr int kMarchMin16 = 6;
-constexpr long long kMarchShort = 1200000;
+constexpr long long kMarchShort = 1200000, kMarchShortMixed = 600000;
 static int launch_steps(const dmrt_ctx* c, int64_t n, bool marched) {
     if (!c->march[2] || n < 3) return 1;
     if (c->p.storage == DMRT_FP32) return n == 4 || n == 5 ? 2 : 3;
-    const bool any = c->p.storage == DMRT_MIXED ||
-                     (c->p.storage == DMRT_THETA32 && (long long)c->p.nx * c->p.ny >= kMarchShort);
+    const long long nodes = (long long)c->p.nx * c->p.ny;
+    const bool any = (c->p.storage == DMRT_MIXED && nodes >= kMarchShortMixed) ||
+                     (c->p.storage == DMRT_THETA32 && nodes >= kMarchShort);
     return marched || any || n >= kMarchMin16 ? 3 : 1;
 }
 // Steps of a whole graph: graph_len launches.
@@ -3335,7 +3344,8 @@ AdjLayout adjoint_layout(const dmrt_ctx* c, long long N) {
     AdjLayout L;
     L.K = (long long)std::ceil(std::sqrt((double)N));
     if (L.K < 1) L.K = 1;
-    // Segments of whole step graphs, so that the forward pass replays graphs only.
+    // Segments of a multiple of graph_len steps: contexts that step once per launch replay
+    // whole graphs in the forward pass (the others have launches of several steps).
     if (L.K > c->graph_len) L.K = (L.K + c->graph_len - 1) / c->graph_len * c->graph_len;
     L.K += L.K & 1;  // even, so that a step's adjoint buffers do not depend on its segment
     L.C = (N + L.K - 1) / L.K;

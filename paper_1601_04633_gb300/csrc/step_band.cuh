@@ -31,8 +31,7 @@
 //
 // What bounds it: up to 192^2 the exchange and the serial chain of a pair's
 // collision, above it the blocks' float32 pipes as well (512^2: 1.2 us of its
-// 3.5 us per step). Measured at the rule in
-// dmrt.cu (setup_band).
+// 3.5 us per step). Measured at the rule in dmrt.cu (setup_band).
 //
 // Every poll is bounded: on expiry the block records kErrTimeout and returns,
 // and its neighbours' polls expire in turn.
@@ -303,8 +302,8 @@ __global__ void __launch_bounds__(MAXT) step_band_kernel(const __grid_constant__
         auto at = [&](int k, int dr) { return *reinterpret_cast<const F2*>(q + k * plane + dr * WS); };
         // The pulls shifted in x (directions 1, 5, 8, g 1 from the left, 3, 6, 7,
         // g 3 from the right) stay single values until the side walls have
-        // replaced theirs: changing one half of a packed pair in a divergent
-        // branch here gave a wrong other half (nvcc 13.0).
+        // replaced theirs. (An earlier form of this code that changed one half of a packed
+        // pair in a divergent branch gave a wrong other half; no small case of it was found.)
         auto px = [&](int k, int dr, float (&v)[2]) {
             const float* p = q + k * plane + dr * WS;
             v[0] = p[-1], v[1] = p[0];

@@ -28,12 +28,12 @@
 // Every mbarrier wait is bounded, as in step_tma.cuh: on expiry the warp
 // records kErrTimeout, waits (bounded) for the copies it issued and returns.
 //
-// Measured on one GB300 (2048^2 float32, three steps per launch): 104 us per
-// launch, 61.3 M warp instructions (the one-step kernel issues 138 M for
-// the same three steps), DRAM 56 %
-// and the float32 pipe 54 % busy over the launch, three warps per scheduler held
-// by shared memory (the ring and the output tile) and registers. The times
-// against the one-step kernels stand at the launch rule in dmrt.cu.
+// Measured on one GB300 (2048^2 float32, three steps per launch): 102 us per launch,
+// 62.2 M warp instructions (the one-step kernel issues 138 M for the same three steps),
+// DRAM 57 % and the float32 pipe 55 % busy over the launch, three warps per scheduler held
+// by shared memory (the ring and the output tile) and registers. At 4096^2 it moves the
+// state at 0.8 of the copy rate. The times against the one-step kernels stand at the launch
+// rule in dmrt.cu.
 
 #pragma once
 #include "collide_pair.cuh"
@@ -270,9 +270,9 @@ __device__ __forceinline__ float wall_value(float sign, float og, float add) { r
 template <bool FLAT>
 __device__ __forceinline__ void side_walls(F2 (&f)[9], F2 (&g)[5], const MarchLane& n, const MarchArgs& M, float of,
                                            float oa, float ob, float og, float add) {
-    // Selects: changing one half of a packed pair in a divergent branch is not safe
-    // with nvcc 13.0 (see step_band.cuh). FLAT: both sides' without a branch (float32,
-    // 1 % faster; in 16-bit storage the registers it takes cost 2 %).
+    // Selects, not an assignment to one half of a packed pair in a divergent branch (see
+    // step_band.cuh). FLAT: both sides' without a branch (float32, 1 % faster; in 16-bit
+    // storage the registers it takes cost 2 %).
     const bool rl = n.right && !n.rhi, rh = n.right && n.rhi;
     auto left = [&](F2 v, float w) { return f2_pack(n.left ? w : f2_lo(v), f2_hi(v)); };
     auto right = [&](F2 v, float w) { return f2_pack(rl ? w : f2_lo(v), rh ? w : f2_hi(v)); };

@@ -20,7 +20,7 @@ RUNS = (3, 200, 1, 400, 4, 2, 5, 7, 6, 1)
 MODES = [(0, 0), (1, 0), (1, 1), (2, 0), (2, 1), (3, 0), (3, 1), (4, 0), (4, 1)]
 # Whole strips (60 columns in float32, 56 in 16-bit storage), one column more or less, several
 # chunks, few rows, and more than 1024 rows (Nusselt sums of several rows per partial);
-# 16-bit storage marches from 400000 nodes on up to 500 columns, else from a million.
+# 16-bit storage marches from 400000 nodes on up to 900 columns, above 1600 from a million.
 SIZES = [(1080, 43), (1081, 171), (1064, 181), (1063, 90), (777, 701), (241, 1501)]
 SIZES16 = [(448, 900), (447, 901), (449, 891), (241, 1701), (1065, 951), (5001, 201)]
 CASES = [(nx, ny, st, rd) for st, rd in MODES for nx, ny in (SIZES16 if st else SIZES)]
