@@ -326,10 +326,10 @@ int dmrt_probe_band_wait(int32_t kind, int64_t limit_ns, void* stream, int64_t* 
 
 /* The same for a launch of several steps per pass: one warp's work on the top row of
  * a float32 context that takes such launches (else DMRT_E_ARG), with the copy of
- * the row'th row it loads (0 to 3) never complete. The warp must store nothing and record
+ * the row'th row it loads (0 to 3) never complete; batched: the form of a batch's launches. The warp must store nothing and record
  * the expiry: returns DMRT_E_TIMEOUT, which stays the context's error (DMRT_OK: a
  * defect). limit_ns in [1 ms, 2 s]. Synchronises. */
-int dmrt_probe_march_wait(dmrt_ctx* c, int32_t row, int64_t limit_ns);
+int dmrt_probe_march_wait(dmrt_ctx* c, int32_t row, int32_t batched, int64_t limit_ns);
 
 /* ---- One step without any device allocation (the paper has no counterpart) ----
  *

@@ -2022,7 +2022,7 @@ int dmrt_check(dmrt_ctx* c) {
     return poll_error(c);
 }
 
-int dmrt_probe_march_wait(dmrt_ctx* c, int32_t row, int64_t limit_ns) {
+int dmrt_probe_march_wait(dmrt_ctx* c, int32_t row, int32_t batched, int64_t limit_ns) {
     if (!c) return DMRT_E_ARG;
     if (!c->march[3] || c->p.storage != DMRT_FP32 || c->p.ny < 4 || row < 0 || row >= dmrt::kMarchStages ||
         limit_ns < 1000000 || limit_ns > (int64_t)dmrt::kWaitLimitNs) {
@@ -2035,7 +2035,7 @@ int dmrt_probe_march_wait(dmrt_ctx* c, int32_t row, int64_t limit_ns) {
     M.chunk = 1;
     M.n_chunks = c->p.ny;
     CK(dmrt::launch_march_wait_probe(c->mmaps[c->cur], M, c->pc, M.n_strips * (c->p.ny - 1), row,
-                                     (unsigned long long)limit_ns, c->stream),
+                                     batched != 0, (unsigned long long)limit_ns, c->stream),
        "march wait probe");
     return poll_error(c);
 }

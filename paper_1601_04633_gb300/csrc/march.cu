@@ -25,6 +25,7 @@ MarchForm march_form(int storage, int rounding, int steps) {
     return {nullptr, 0, 0, 0};
 }
 
+template <bool FIRST>
 static __global__ void __launch_bounds__(32)
     march_wait_probe_kernel(const __grid_constant__ MarchMaps maps, const __grid_constant__ MarchArgs M,
                             const __grid_constant__ PairConsts K, int item, int row, unsigned long long limit_ns) {
@@ -37,15 +38,16 @@ static __global__ void __launch_bounds__(32)
         mbar_fence_init();
     }
     __syncwarp();
-    march_item<L, false, 3>(maps.ld, maps.st, M, K.r, K.n, item, lane, smem_m, bars, limit_ns);
+    march_item<L, false, 3, FIRST>(maps.ld, maps.st, M, K.r, K.n, item, lane, smem_m, bars, limit_ns);
 }
 
 cudaError_t launch_march_wait_probe(const MarchMaps& maps, const MarchArgs& M, const PairConsts& K, int item, int row,
-                                    unsigned long long limit_ns, cudaStream_t stream) {
+                                    bool first, unsigned long long limit_ns, cudaStream_t stream) {
     constexpr unsigned smem = MarchGeo<OneType<float>>::kSmem;
-    const cudaError_t e = cudaFuncSetAttribute(march_wait_probe_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const auto kernel = first ? march_wait_probe_kernel<true> : march_wait_probe_kernel<false>;
+    const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    march_wait_probe_kernel<<<1, 32, smem, stream>>>(maps, M, K, item, row, limit_ns);
+    kernel<<<1, 32, smem, stream>>>(maps, M, K, item, row, limit_ns);
     return cudaGetLastError();
 }
 

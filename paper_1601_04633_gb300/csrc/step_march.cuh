@@ -28,9 +28,9 @@
 // Every mbarrier wait is bounded, as in step_tma.cuh: on expiry the warp
 // records kErrTimeout, waits (bounded) for the copies it issued and returns.
 //
-// Measured on one GB300 (2048^2 float32, three steps per launch): 102 us per launch,
+// Measured on one GB300 (2048^2 float32, three steps per launch): 103 us per launch,
 // 62.2 M warp instructions (the one-step kernel issues 138 M for the same three steps),
-// DRAM 57 % and the float32 pipe 55 % busy over the launch, three warps per scheduler held
+// DRAM 56 % and the float32 pipe 54 % busy over the launch, three warps per scheduler held
 // by shared memory (the ring and the output tile) and registers. At 4096^2 it moves the
 // state at 0.8 of the copy rate. The times against the one-step kernels stand at the launch
 // rule in dmrt.cu.
@@ -428,8 +428,11 @@ struct MarchCarry {
 };
 
 // One item (strip, chunk) of a cavity by one warp: ring and bars are the warp's,
-// the barriers freshly initialised.
-template <typename L, bool SR, int T>
+// the barriers freshly initialised. FIRST: the rows that the first iteration needs are
+// waited for before the loop, as the batched launches have it (64 cavities in float32
+// 36.2 us per step, 36.4 with that wait in the loop); the single-cavity launches wait in the
+// loop (2048^2 in float32 33.0 us, 34.0 with it before).
+template <typename L, bool SR, int T, bool FIRST>
 __device__ __forceinline__ void march_item(const CUtensorMap* ld, const CUtensorMap* st, const MarchArgs& M,
                                            const PairRates& K, const PairNumbers& C9, int item, int lane,
                                            unsigned char* ring, uint64_t* bars,
@@ -479,6 +482,17 @@ __device__ __forceinline__ void march_item(const CUtensorMap* ld, const CUtensor
         for (int row = lb; row < issued; ++row) issue(row);
     bool ok = true;
     int waited = lb;  // rows below this one have arrived (!ok: those below waited - 1)
+    // On expiry: record it, and wait (bounded) for the copies from the row that failed on.
+    auto give_up = [&]() {
+        if (lane != 0) return;
+        atomicOr(A.err, kErrTimeout);
+        for (int row = waited - 1; row < issued; ++row)
+            mbar_wait_bounded(bar(row), (unsigned)((row - lb) / kMarchStages) & 1u, limit_ns);
+    };
+    if constexpr (FIRST) {
+        for (; waited <= rs && ok; ++waited) ok = arrived(waited);
+        if (!ok) return give_up();
+    }
 
     MarchCarry C[T - 1];
 #pragma unroll
@@ -510,9 +524,17 @@ __device__ __forceinline__ void march_item(const CUtensorMap* ld, const CUtensor
     const int last = min(rend, A.ny - 1);
 #pragma unroll 1
     for (int r = rs; r <= rend; ++r) {
-        // Rows up to r + 1 have arrived (the first iteration waits for all from lb on).
-        for (; ok && waited <= min(r + 1, ub); ++waited) ok = arrived(waited);
-        if (!ok) break;
+        // Rows up to r + 1 have arrived (without FIRST, the first iteration waits for all from lb on).
+        if constexpr (FIRST) {
+            if (waited <= ub) {
+                ok = arrived(waited);
+                ++waited;
+                if (!ok) break;
+            }
+        } else {
+            for (; ok && waited <= min(r + 1, ub); ++waited) ok = arrived(waited);
+            if (!ok) break;
+        }
         F2 f[9], g[5], rho, theta;
         float add = nadd;
         // Step 0 from the stages.
@@ -635,11 +657,7 @@ __device__ __forceinline__ void march_item(const CUtensorMap* ld, const CUtensor
         }
     }
     if (lane == 0) bulk_wait_all();  // the stores have read the tile and written global memory
-    if (!ok && lane == 0) {
-        atomicOr(A.err, kErrTimeout);
-        for (int row = waited - 1; row < issued; ++row)
-            mbar_wait_bounded(bar(row), (unsigned)((row - lb) / kMarchStages) & 1u, limit_ns);
-    }
+    if (!ok) give_up();
     if (n.out && (!(peak0 < 1e30f) || (n.two && !(peak1 < 1e30f)))) atomicOr(A.err, kErrNonFinite);
 }
 
@@ -676,7 +694,7 @@ __global__ void __launch_bounds__(kMarchThreads, MINB)
     }
     const int item = blockIdx.x * (kMarchThreads / 32) + warp;
     if (item >= M.n_strips * M.n_chunks) return;
-    march_item<L, SR, T>(maps.ld, maps.st, M, K.r, K.n, item, lane, ring, bars);
+    march_item<L, SR, T, false>(maps.ld, maps.st, M, K.r, K.n, item, lane, ring, bars);
 }
 
 // ---- batched sweep ----------------------------------------------------------------
@@ -727,7 +745,7 @@ __global__ void __launch_bounds__(kMarchThreads, MINB) batch_march_kernel(const 
         else hi = mid - 1;
     }
     const CUtensorMap* maps = B.maps + (size_t)lo * 6;
-    march_item<L, SR, T>(maps, maps + 3, B.M[lo], B.r[lo], B.n, item - B.first[lo], lane, ring, bars);
+    march_item<L, SR, T, true>(maps, maps + 3, B.M[lo], B.r[lo], B.n, item - B.first[lo], lane, ring, bars);
     if (lane == 0 && (*reinterpret_cast<volatile unsigned*>(B.M[lo].A.err) & kErrTimeout)) atomicOr(B.err, kErrTimeout);
 }
 
@@ -751,9 +769,10 @@ static_assert(sizeof(MarchBatchArgs) <= 32764, "kernel parameters");
 MarchForm march_form(int storage, int rounding, int steps);
 MarchForm batch_march_form(int storage, int rounding, int steps);  // float32 and mixed storage
 
-// One float32 item by one warp, the copy of the chunk's row `row` (from its first one
-// loaded) never complete: the barrier waits for an arrival that nobody makes.
+// One float32 item by one warp (first: in the batched launches' form), the copy of the
+// chunk's row `row` (from its first one loaded) never complete: the barrier waits for an
+// arrival that nobody makes.
 cudaError_t launch_march_wait_probe(const MarchMaps& maps, const MarchArgs& M, const PairConsts& K, int item, int row,
-                                    unsigned long long limit_ns, cudaStream_t stream);
+                                    bool first, unsigned long long limit_ns, cudaStream_t stream);
 
 }  // namespace dmrt

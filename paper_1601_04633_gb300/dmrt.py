@@ -137,7 +137,7 @@ SIGNATURES = {
     "dmrt_save": (ctypes.c_int, [_VP, _VP, ctypes.c_size_t, ctypes.POINTER(ctypes.c_size_t)]),
     "dmrt_probe_bounded_wait": (ctypes.c_int, [ctypes.c_int64, _VP, ctypes.POINTER(ctypes.c_int64)]),
     "dmrt_probe_band_wait": (ctypes.c_int, [ctypes.c_int32, ctypes.c_int64, _VP, ctypes.POINTER(ctypes.c_int64)]),
-    "dmrt_probe_march_wait": (ctypes.c_int, [_VP, ctypes.c_int32, ctypes.c_int64]),
+    "dmrt_probe_march_wait": (ctypes.c_int, [_VP, ctypes.c_int32, ctypes.c_int32, ctypes.c_int64]),
     "dmrt_load": (ctypes.c_int, [_VP, _VP, ctypes.c_size_t]),
     "dmrt_step_noalloc": (ctypes.c_int, [ctypes.POINTER(Params), _VP, _VP, _VP, _VP, _VP, _VP]),
     "dmrt_adjoint_workspace_size": (ctypes.c_int, [_VP, ctypes.c_int64, ctypes.POINTER(ctypes.c_size_t)]),

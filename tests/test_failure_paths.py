@@ -68,16 +68,17 @@ def test_the_band_kernels_waits_give_up(D, kind):
     assert L.dmrt_probe_band_wait(2, 5_000_000, stream, None) == D.DMRT_E_ARG
 
 
+@pytest.mark.parametrize("batched", [0, 1])
 @pytest.mark.parametrize("row", [0, 1, 2, 3])
-def test_a_march_launch_reports_any_row_that_does_not_arrive(D, row):
-    # 0 and 1 are waited for before the first row of the chunk, 2 and 3 in its rows.
+def test_a_march_launch_reports_any_row_that_does_not_arrive(D, row, batched):
+    # 0 and 1 are waited for before the first row of the chunk is collided, 2 and 3 in its rows.
     import torch
 
     sim = D.Cavity2D.from_inputs(inputs.Cavity(1100, 64, 1e4, 0.01, noise_amp=1e-3, seed=8), nu_capacity=64)
     sim.step(6)
     sim.check()
     before = sim.workspace.clone()
-    assert D.load().dmrt_probe_march_wait(sim.h, row, 20_000_000) == D.DMRT_E_TIMEOUT
+    assert D.load().dmrt_probe_march_wait(sim.h, row, batched, 20_000_000) == D.DMRT_E_TIMEOUT
     torch.cuda.synchronize()
     assert int((sim.workspace != before).sum()) == 1  # one bit of the error word, and no row stored
     with pytest.raises(D.DmrtError) as ei:
